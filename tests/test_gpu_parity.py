@@ -124,6 +124,33 @@ def test_brute_force_on_warps_of_unlike_blocks(B, fmt, sweep_mode):
     check_parity(x.to(torch.bfloat16), B, fmt, mxq.MXQ_BRUTE_PZ, 1.0)
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B", BLOCKS)
+@pytest.mark.parametrize("fmt", FMTS)
+def test_pruned_sweep_at_the_edges_of_its_bounds(dtype, B, fmt):
+    """Tensors of one block, of part of a store unit and of one tile and a bit; blocks whose bounds leave nearly every code
+    (several elements far above the largest decode scale), whose codes are subnormal, whose elements are exact grid
+    multiples of a scale (the bounds are met with equality), and blocks and tensor scales outside the shortcuts' ranges."""
+    tile = 512 if B == 16 else max(256, 4096 // B)     # blocks the kernel sorts together
+    gen = torch.Generator().manual_seed(77 + B + fmt)
+    mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 1)
+    try:
+        for nb in (1, 2, 3, 31, tile + 1, 3 * tile + 5):
+            x = inputs.student_t(nb * B, 4, 0.05, 31 + nb, torch.float32).view(nb, B)
+            x[1::9] *= 2.0 ** 26                       # above 6 times the top scale
+            x[2::9] = x[2::9].sign() * 2.0 ** 24       # all elements equal and above it
+            x[3::9] *= 2.0 ** -12                      # subnormal scale codes of UE4M3, code 0
+            grid = torch.tensor([0.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, 6.0])
+            x[4::9] = grid[torch.randint(0, 8, x[4::9].shape, generator=gen)] * (1 + torch.randint(0, 8, (x[4::9].shape[0], 1), generator=gen) / 8) * 0.0625
+            x[5::9, 0] *= 2.0 ** 62                    # one huge element
+            x[6::9] *= 2.0 ** -60                      # below the range of the shortcuts
+            xd = x.reshape(-1).to(dtype).contiguous()
+            for recipe, g in ((mxq.MXQ_BRUTE, 1.0), (mxq.MXQ_BRUTE_PZ, 1.0), (mxq.MXQ_BRUTE, 0.0173), (mxq.MXQ_BRUTE, 2.0 ** -45), (mxq.MXQ_BRUTE_PZ, 1.5 * 2.0 ** 55)):
+                check_parity(xd, B, fmt, recipe, g)
+    finally:
+        mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 0)
+
+
 def test_option_calls_reject_bad_arguments():
     with pytest.raises(mxq.MxqError):
         mxq.mxq_set_option(99, 1)
