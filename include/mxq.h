@@ -295,8 +295,10 @@ int mxq_mask_interval(const void* x, int dtype, size_t n, float lo, float hi, vo
 
 /* Process-wide options, read by the entry points when they are called.
  *
- * MXQ_OPT_BRUTE_PRUNE (default 0).  With 0 the brute-force recipes evaluate every finite scale code
- * on every block, exactly as the search is stated (Experimental Setup).  With 1 the kernel leaves out the
+ * MXQ_OPT_BRUTE_PRUNE (default 0).  With 0 the brute-force recipes form the block SSE of every finite scale
+ * code, as the search is stated (Experimental Setup), and keep the smallest; nothing depends on the SSEs of
+ * other codes.  (Codes under which the same sum of squares arises by definition -- every element rounds
+ * to zero, or the scale is too small to change any element -- share one evaluation.)  With 1 the kernel leaves out the
  * codes that provably cannot change an output of the block, given the better SSE of two codes tried first:
  *   - decode scales of at least four times the block maximum: every element quantizes to zero
  *     (|v|/D <= 1/4 rounds to the grid value 0), so all of them have the SSE of the all-zero

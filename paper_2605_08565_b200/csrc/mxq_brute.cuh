@@ -21,9 +21,8 @@
 // formats, one for the power-of-two format) have decode scales that differ by exact powers of two,
 // D_c = Dref * 2^k, as long as D_c is a normal number.  Hence fl(v / D_c) = fl(v / Dref) * 2^-k
 // exactly: the correctly rounded quotient is formed once per class and element, and a candidate
-// costs one multiply by a power of two, the FP4 rounding, and the two FMAs of the SSE.  Codes
-// whose decode scale is zero, subnormal or above 2^126 need no quotient at all (every element
-// rounds to zero, or saturates) and form one more list.  Threads holding a magnitude above 2^60
+// costs one multiply by a power of two, the FP4 rounding, and the two FMAs of the SSE.  Codes under
+// which every element of the warp rounds to zero or saturates cost less (search_group()).  Threads holding a magnitude above 2^60
 // or a nonzero one below 2^-62 take the general path (IEEE division), candidate by candidate.
 //
 // Inside a class the members are visited in ascending code order and the smallest SSE bit pattern
@@ -49,40 +48,34 @@ __device__ __forceinline__ int code_class(int c) {
     return (int)((0x64204000u >> (4 * c)) & 7u);
 }
 
-// Per-CTA tables of the search.  Every code with a finite decode scale D sits in one candidate list:
-//   * D normal with a biased exponent of at most 253 ("paired": D = Dref * 2^k and 2^-k are both
-//     representable): list 2 * class + kind, where kind 1 holds the codes whose -D is exactly
-//     representable in f16 (their residual is one mixed-precision FMA from the unpacked f16 grid
-//     value) and kind 0 the others (f16 -> f32 convert, then an FFMA);
-//   * the "flat" list kFlatList for the rest.  D = 0 or D >= 2^127: every quotient of a magnitude
-//     <= 2^60 rounds to FP4 zero, so the candidate is entered with the multiplier 0.  D subnormal:
-//     every nonzero magnitude >= 2^-62 divided by it exceeds 2^64 and saturates at 6, so it is
-//     entered with the multiplier 2^126.  The flat list is evaluated on the elements themselves
-//     (Dref = 1), which needs no quotient.
-constexpr int kLists = 17;
-constexpr int kFlatList = 16;
-constexpr int kCandSlots = 16 * kMaxMembers + 256;
+// Per-CTA tables of the search.  Every code whose decode scale D is normal with a biased exponent of at most 253 (D = Dref *
+// 2^k and 2^-k are both representable) sits in the candidate list 2 * class + kind, where kind 1 holds the codes whose -D is
+// exactly representable in f16 (their residual is one mixed-precision FMA from the unpacked f16 grid value) and kind 0
+// the others (f16 -> f32 convert, then an FFMA).  Codes with D zero, subnormal or at least 2^127 never need the full
+// evaluation (see search_group()).
+constexpr int kLists = 16;
+constexpr int kCandSlots = kLists * kMaxMembers;
 struct BruteTables {
     float D[256];            // decode scale of the code; NaN for codes that do not exist
     float R[256];            // RN(1 / D) when 2^-60 <= D <= 2^60, else 0 (used by the final encode)
     float4 cand[kCandSlots];    // per list, ascending code order: (-D, multiplier, f16(-D) twice as bits, 0)
     uint8_t member[kCandSlots]; // the code of each slot of cand[]
-    uint8_t kind[256];       // 0, 1 paired as above; 3 = flat list; 2 = not a candidate
     float clsD[8];           // Dref of the class, in [1, 2)
     float clsR[8];           // RN(1 / Dref)
     int cnt[kLists];         // members per list
-    uint32_t kind_mask[3][8];
+    int flat_min;            // smallest code with D zero, subnormal or at least 2^127; 256 if there is none
+    uint8_t below[kLists][256];   // members of the list whose code is smaller
+    uint8_t in_warp[kThreads / 32][kLists];   // members of the list among the 32 codes of a warp (scratch of the build)
 };
 
 template <int FMT>
 __device__ __forceinline__ int members_base(int list) {
-    if (list == kFlatList) return 16 * kMaxMembers;
     // the power-of-two format has one class: its two lists get half of the class area each
-    return FMT == kUE8M0 ? list * (16 * kMaxMembers / 2) : list * kMaxMembers;
+    return FMT == kUE8M0 ? list * (kCandSlots / 2) : list * kMaxMembers;
 }
 
-// first: smallest admissible code (1 under prevent-zero for the FP8 formats, else 0).
-template <int FMT>
+// first: smallest admissible code (1 under prevent-zero for the FP8 formats, else 0).  BELOW: with the index by code.
+template <int FMT, bool BELOW>
 __device__ __forceinline__ void build_brute_tables(BruteTables& T, float g, int first) {
     static_assert(kThreads == 256, "one thread per table entry");
     build_scale_tables<FMT>(T.D, T.R, g);
@@ -93,56 +86,52 @@ __device__ __forceinline__ void build_brute_tables(BruteTables& T, float g, int 
     const bool usable = c >= first && c < num_codes(FMT) && (b >> 31) == 0 && e != 255;
     const bool is_paired = usable && e >= 1 && e <= 253;
     const __half hD = __float2half_rn(-D);
-    const int kind = !usable ? 2 : (!is_paired ? 3 : (__half2float(hD) == -D ? 1 : 0));
-    T.kind[c] = (uint8_t)kind;
-    if (c < kLists) T.cnt[c] = 0;
-    const uint32_t ballot0 = __ballot_sync(0xFFFFFFFFu, kind == 0);
-    const uint32_t ballot1 = __ballot_sync(0xFFFFFFFFu, kind == 1);
-    const uint32_t ballot3 = __ballot_sync(0xFFFFFFFFu, kind == 3);
-    if ((c & 31) == 0) {
-        T.kind_mask[0][c >> 5] = ballot0;
-        T.kind_mask[1][c >> 5] = ballot1;
-        T.kind_mask[2][c >> 5] = ballot3;
+    const int my_list = !is_paired ? -1 : 2 * code_class<FMT>(c) + (__half2float(hD) == -D ? 1 : 0);
+    if (c == 0) T.flat_min = 256;
+    constexpr int NL = FMT == kUE8M0 ? 2 : kLists;
+    const int warp = c >> 5, lane = c & 31;
+    uint32_t members[NL];
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+        members[l] = __ballot_sync(0xFFFFFFFFu, my_list == l);
+        if (lane == l) T.in_warp[warp][l] = (uint8_t)__popc(members[l]);
     }
     __syncthreads();
-    const uint32_t below = (1u << (c & 31)) - 1u;
-    if (kind == 3) {
-        int rank = __popc(ballot3 & below);
-        for (int w = 0; w < (c >> 5); ++w) rank += __popc(T.kind_mask[2][w]);
-        // multiplier 0 -> every quotient is zero; 2^126 -> every nonzero quotient saturates
-        const float P = (e == 0 && D != 0.0f) ? __uint_as_float(0x7E800000u) : 0.0f;
-        const int slot = members_base<FMT>(kFlatList) + rank;
-        T.cand[slot] = make_float4(-D, P, 0.0f, 0.0f);
-        T.member[slot] = (uint8_t)c;
-        atomicAdd(&T.cnt[kFlatList], 1);
-    }
-    if (is_paired) {
-        const int cls = code_class<FMT>(c);
-        int rank = 0;
-        if constexpr (FMT == kUE8M0) {
-            for (int w = 0; w < (c >> 5); ++w) rank += __popc(T.kind_mask[kind][w]);
-            rank += __popc((kind ? ballot1 : ballot0) & below);
-        } else {
-            for (int o = 1; o < 8 && o < c; ++o) rank += (T.kind[o] == kind && code_class<FMT>(o) == cls) ? 1 : 0;
-            for (int o = 8 + cls; o < c; o += 8) rank += (T.kind[o] == kind) ? 1 : 0;
+    if (c < NL) {   // exclusive prefix sums over the warps, and the total
+        int n = 0;
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) {
+            const int here = T.in_warp[w][c];
+            T.in_warp[w][c] = (uint8_t)n;
+            n += here;
         }
+        T.cnt[c] = n;
+    }
+    __syncthreads();
+    int rank = 0;
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+        const int n = T.in_warp[warp][l] + __popc(members[l] & ((1u << lane) - 1u));
+        if constexpr (BELOW) T.below[l][c] = (uint8_t)n;
+        if (l == my_list) rank = n;
+    }
+    if (usable && !is_paired) atomicMin(&T.flat_min, c);
+    if (is_paired) {
         const float P = __uint_as_float((254u - e) << 23);
         const uint32_t h16 = (uint32_t)__half_as_ushort(hD);
-        const int list = 2 * cls + kind;
-        const int slot = members_base<FMT>(list) + rank;
+        const int slot = members_base<FMT>(my_list) + rank;
         T.cand[slot] = make_float4(-D, P, __uint_as_float(h16 | (h16 << 16)), 0.0f);
         T.member[slot] = (uint8_t)c;
-        atomicAdd(&T.cnt[list], 1);
         if (rank == 0) {   // both kinds of a class write the same values
             const float Dref = __uint_as_float((b & 0x007FFFFFu) | 0x3F800000u);
-            T.clsD[cls] = Dref;
-            T.clsR[cls] = __frcp_rn(Dref);
+            T.clsD[my_list >> 1] = Dref;
+            T.clsR[my_list >> 1] = __frcp_rn(Dref);
         }
     }
     __syncthreads();
     // the search takes two members per trip: a range that ends with the list may read one slot
     // past it, which repeats the last member
-    if (c < kLists && T.cnt[c] > 0) {
+    if (c < NL && T.cnt[c] > 0) {
         const int last = members_base<FMT>(c) + T.cnt[c] - 1;
         T.cand[last + 1] = T.cand[last];
         T.member[last + 1] = T.member[last];
@@ -284,16 +273,27 @@ __device__ __forceinline__ void keep_smaller(uint32_t& best_bits, int& best_slot
     best_bits = min(best_bits, bits);
 }
 
+// Largest code whose value is at most S (0 if there is none), S >= 0.
+template <int FMT>
+__device__ __forceinline__ int floor_code(float S) {
+    const uint32_t b = __float_as_uint(S);
+    if constexpr (FMT == kUE8M0) return (int)min(b >> 23, 254u);
+    constexpr int bias = (FMT == kUE4M3) ? 7 : 15;
+    const int normal = (int)(b >> 20) - ((127 - bias) << 3);
+    const int sub = __float2int_rz(__fmul_rn(S, (float)(1 << (bias + 2))));
+    return min(normal < 8 ? sub : normal, num_codes(FMT) - 1);
+}
+
 // All members of one range of one list (one mantissa class, one residual kind) against the
 // thread's elements; the winner of every block is folded into best[].
 // Members first .. first + cnt_raw - 1 of the list are evaluated.
-template <int B, int FMT, bool HALF, int NP, int NBT>
+template <int B, int FMT, bool HALF, int NP, typename Best>
 __device__ __forceinline__ void search_list(const BruteTables& T, int list, int first, int cnt_raw,
-                                            const float2 (&v2)[NP], const float2 (&tb)[NP],
-                                            unsigned long long (&best)[NBT]) {
+                                            const float2 (&v2)[NP], const float2 (&tb)[NP], Best& best) {
     constexpr bool ONEBLK = (B >= 32);
     constexpr int BL = ONEBLK ? NP : B;
     constexpr int NBL = NP / BL;
+    constexpr int NBT = ONEBLK ? 1 : 2 * NBL;
     if (cnt_raw <= 0) return;
     [[maybe_unused]] const int cnt = cnt_raw;
     const int base = members_base<FMT>(list) + first;
@@ -384,8 +384,275 @@ __host__ __device__ constexpr int brute_group_elems(int B) { return B >= 32 ? B 
 
 constexpr int brute_min_ctas(int B) { return B <= 32 ? 2 : 1; }
 
+// The best (SSE bits, code) keys of a thread's blocks in shared memory, 32 lanes apart.
+struct SharedBest {
+    unsigned long long* p;
+    __device__ __forceinline__ unsigned long long& operator[](int k) const { return p[32 * k]; }
+};
+
+template <int B>
+struct BruteShape {
+    static constexpr bool ONEBLK = (B >= 32);       // the thread owns exactly one block
+    static constexpr int G = brute_group_elems(B);  // elements per thread
+    static constexpr int NP = G / 2;                // pairs per thread
+    static constexpr int BL = ONEBLK ? NP : B;      // elements of one block inside one half
+    static constexpr int NBL = NP / BL;             // blocks per half (1 when ONEBLK)
+    static constexpr int NBT = G / B;               // blocks per thread
+};
+
+// What a thread knows of its elements beside their magnitudes.
+struct GroupRange {
+    float amax, amin;      // largest magnitude; smallest nonzero one (+inf if there is none)
+    bool has_zero;
+    bool fast;             // no magnitude above 2^60, no nonzero one below 2^-62 (its quotient by Dref may be inexact)
+};
+
+// A thread's elements.  n_here: elements of the tensor in this group (a multiple of B, at most G); what is missing is taken
+// as zero.
+template <int DT, int B>
+__device__ __forceinline__ void load_group(float (&v)[BruteShape<B>::G], const void* x, size_t e0, int n_here) {
+    using S = BruteShape<B>;
+    if (n_here >= S::G) {
+        load_elems<DT, S::G>(x, e0, v);
+        return;
+    }
+#pragma unroll
+    for (int k = 0; k < S::NBT; ++k) {
+        float w[B];
+        if (k * B < n_here) {
+            load_elems<DT, B>(x, e0 + k * B, w);
+        } else {
+#pragma unroll
+            for (int i = 0; i < B; ++i) w[i] = 0.0f;
+        }
+#pragma unroll
+        for (int i = 0; i < B; ++i) v[k * B + i] = w[i];
+    }
+}
+
+// Stores a thread's results; blocks: how many of them the tensor has (fewer than NBT in its last group).
+template <int B>
+__device__ __forceinline__ void store_group(const QuantArgs& p, size_t grp, int blocks, const uint32_t (&packed)[BruteShape<B>::G / 8],
+                                            const uint32_t (&sc)[(BruteShape<B>::NBT + 3) / 4], const uint32_t (&sw)[BruteShape<B>::NBT]) {
+    using S = BruteShape<B>;
+    if (blocks == S::NBT) {
+        store_bytes<S::G / 2>(p.codes + grp * (S::G / 2), packed);
+        store_bytes<S::NBT>(p.scales + grp * S::NBT, sc);
+        if (p.block_sse) store_bytes<4 * S::NBT>(p.block_sse + grp * S::NBT, sw);
+    } else {
+#pragma unroll
+        for (int k = 0; k < S::NBT; ++k) {
+            if (k >= blocks) break;
+            const size_t b = grp * S::NBT + k;
+            uint32_t w[(B + 7) / 8];
+            if constexpr (B < 8) {
+                w[0] = packed[k * B / 8] >> (4 * (k * B % 8));
+            } else {
+#pragma unroll
+                for (int i = 0; i < B / 8; ++i) w[i] = packed[k * B / 8 + i];
+            }
+            store_bytes<B / 2>(p.codes + b * (B / 2), w);
+            p.scales[b] = (uint8_t)(sc[k / 4] >> (8 * (k % 4)));
+            if (p.block_sse) p.block_sse[b] = __uint_as_float(sw[k]);
+        }
+    }
+}
+
+// Their magnitudes (an SSE does not depend on signs): pair i = adjacent elements (one block per thread) or element i of
+// either half.
+template <int B>
+__device__ __forceinline__ GroupRange take_magnitudes(float2 (&v2)[BruteShape<B>::NP], float (&v)[BruteShape<B>::G]) {
+    using S = BruteShape<B>;
+    constexpr float kTiny = 2.168404344971009e-19f;  // 2^-62
+    GroupRange r;
+    r.amax = 0.0f;
+    r.amin = __uint_as_float(0x7F800000u);
+    r.has_zero = false;
+#pragma unroll
+    for (int i = 0; i < S::G; ++i) {
+        v[i] = fabsf(v[i]);
+        r.amax = fmaxf(r.amax, v[i]);
+        r.amin = fminf(r.amin, v[i] == 0.0f ? __uint_as_float(0x7F800000u) : v[i]);
+        r.has_zero |= v[i] == 0.0f;
+    }
+#pragma unroll
+    for (int i = 0; i < S::NP; ++i) v2[i] = S::ONEBLK ? make_float2(v[2 * i], v[2 * i + 1]) : make_float2(v[i], v[S::NP + i]);
+    r.fast = r.amax <= kFastMax && r.amin >= kTiny;
+    return r;
+}
+
+// SSEs of all blocks of a thread when every element saturates, for the codes lo .. hi - 1: q = 6 and e = fma(6, -D, |v|).
+template <int B>
+__device__ __forceinline__ void search_saturated(const BruteTables& T, int lo, int hi, const float2 (&v2)[BruteShape<B>::NP],
+                                                 const SharedBest& best) {
+    using S = BruteShape<B>;
+    if (lo >= hi) return;
+    uint32_t cbest[S::NBT];
+    int ccode[S::NBT];
+#pragma unroll
+    for (int k = 0; k < S::NBT; ++k) { cbest[k] = 0xFFFFFFFFu; ccode[k] = 0; }
+    for (int c = lo; c < hi; c += 2) {
+        const int cB = min(c + 1, hi - 1);   // an odd code out is evaluated twice
+        const float nDA = -T.D[c], nDB = -T.D[cB];
+        if constexpr (!S::ONEBLK) {
+            const float2 six = make_float2(6.0f, 6.0f), A2 = make_float2(nDA, nDA), B2 = make_float2(nDB, nDB);
+            float2 sA[S::NBL], sB[S::NBL];
+#pragma unroll
+            for (int k = 0; k < S::NBL; ++k) sA[k] = sB[k] = make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int i = 0; i < S::NP; ++i) {
+                const float2 eA = __ffma2_rn(six, A2, v2[i]), eB = __ffma2_rn(six, B2, v2[i]);
+                sA[i / S::BL] = __ffma2_rn(eA, eA, sA[i / S::BL]);
+                sB[i / S::BL] = __ffma2_rn(eB, eB, sB[i / S::BL]);
+            }
+#pragma unroll
+            for (int k = 0; k < S::NBL; ++k) {
+                keep_smaller(cbest[k], ccode[k], __float_as_uint(sA[k].x), c);
+                keep_smaller(cbest[S::NBL + k], ccode[S::NBL + k], __float_as_uint(sA[k].y), c);
+                keep_smaller(cbest[k], ccode[k], __float_as_uint(sB[k].x), cB);
+                keep_smaller(cbest[S::NBL + k], ccode[S::NBL + k], __float_as_uint(sB[k].y), cB);
+            }
+        } else {
+            float2 s = make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int i = 0; i < S::NP; ++i) {
+                const float2 e0 = make_float2(__fmaf_rn(6.0f, nDA, v2[i].x), __fmaf_rn(6.0f, nDB, v2[i].x));
+                s = __ffma2_rn(e0, e0, s);
+                const float2 e1 = make_float2(__fmaf_rn(6.0f, nDA, v2[i].y), __fmaf_rn(6.0f, nDB, v2[i].y));
+                s = __ffma2_rn(e1, e1, s);
+            }
+            keep_smaller(cbest[0], ccode[0], __float_as_uint(s.x), c);
+            keep_smaller(cbest[0], ccode[0], __float_as_uint(s.y), cB);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < S::NBT; ++k) merge_class_winner(best[k], cbest[k], ccode[k]);
+}
+
+// The SSE of every code on every block of the warp's threads; best[k] (shared memory: registers are what these kernels
+// are short of) receives the smallest of block k, ties to the smaller code.  Rg = RN(1 / g), or 0 for g beyond 2^+-60.
+// Called by whole warps; `live` lanes take part.  Slice `slice` of `slices` covers its share of the codes.
+//
+// Three stretches of the codes need less than the full evaluation, and are the same for the whole warp (decode scales rise
+// with the code; lo and hi are the warp's smallest nonzero and largest magnitude):
+//   D <  lo * 2^-30   fl(|v| - 6 D) = |v|: the SSE is the sum of squares of the elements, and
+//   D >= 4 hi         every quotient is at most 1/4 and rounds to 0: the same sum.  It is formed once and entered with the
+//                     smallest of these codes, which is how the full evaluation of each would end.
+//   D <= lo / 6       (no zero among the elements) every element saturates: the error is fl(|v| - 6 D), two packed FMAs
+//                     per pair of elements and code instead of quotient, rounding, widening and two FMAs.
+template <int B, int FMT>
+__device__ __forceinline__ void search_group(const BruteTables& T, const float2 (&v2)[BruteShape<B>::NP], const GroupRange& gr, bool live,
+                                             float Rg, int first, int slice, int slices, const SharedBest& best) {
+    using S = BruteShape<B>;
+    constexpr int NCLS = (FMT == kUE8M0) ? 1 : 8;
+    constexpr int NC = num_codes(FMT);
+    constexpr uint32_t kFull = 0xFFFFFFFFu;
+    const bool fast = live && gr.fast;
+    const float hi = __uint_as_float(__reduce_max_sync(kFull, fast ? __float_as_uint(gr.amax) : 0u));
+    const float lo = __uint_as_float(__reduce_min_sync(kFull, fast ? __float_as_uint(gr.amin) : 0x7F800000u));
+    const bool zeros = __any_sync(kFull, fast && gr.has_zero);
+    const float same_below = __fmul_rn(lo, 9.31322574615478515625e-10f /* 2^-30 */);
+    const float sat_below = zeros ? 0.0f : __fmul_rn(lo, 0.1666f);
+    const float zero_from = __fmul_rn(4.0f, hi);
+    int c_same = 0, c_sat = 0, c_zero = 0;    // every code below c_same (c_sat) has its D below the limit, every one from c_zero on D >= 4 hi
+    if (Rg != 0.0f && lo <= hi) {
+        // from the limits' quotients by g, 2^-20 (far more than their rounding) to the safe side; code 0 of the FP8 formats is 0
+        constexpr float kUp = 1.00000095367431640625f, kDown = 0.99999904632568359375f;
+        constexpr int kZero = FMT == kUE8M0 ? 0 : 1;
+        c_same = floor_code<FMT>(__fmul_rn(__fmul_rn(same_below, Rg), kDown)) + kZero;
+        c_sat = floor_code<FMT>(__fmul_rn(__fmul_rn(sat_below, Rg), kDown));
+        c_zero = floor_code<FMT>(__fmul_rn(__fmul_rn(zero_from, Rg), kUp)) + 1;
+    } else {   // tensor scales beyond 2^+-60, or no nonzero element at all: by the table
+#pragma unroll 1
+        for (int k = 0; k < 8; ++k) {
+            const float D = T.D[32 * k + (threadIdx.x & 31)];   // NaN past the last code
+            c_same += __popc(__ballot_sync(kFull, D < same_below));
+            c_sat += __popc(__ballot_sync(kFull, D < sat_below));
+            c_zero += __popc(__ballot_sync(kFull, D < zero_from));
+        }
+    }
+    c_same = max(c_same, first);
+    c_sat = max(c_sat, c_same);
+    c_zero = max(c_zero, c_sat);
+    if (fast) {
+        const int zc = first < c_same ? first : c_zero;
+        if (slice == 0 && zc < NC && fabsf(T.D[zc]) <= 3.402823466e38f) {
+            if constexpr (!S::ONEBLK) {
+                float2 s[S::NBL];
+#pragma unroll
+                for (int k = 0; k < S::NBL; ++k) s[k] = make_float2(0.0f, 0.0f);
+#pragma unroll
+                for (int i = 0; i < S::NP; ++i) s[i / S::BL] = __ffma2_rn(v2[i], v2[i], s[i / S::BL]);
+#pragma unroll
+                for (int k = 0; k < S::NBL; ++k) {
+                    merge_class_winner(best[k], __float_as_uint(s[k].x), zc);
+                    merge_class_winner(best[S::NBL + k], __float_as_uint(s[k].y), zc);
+                }
+            } else {
+                float s = 0.0f;
+#pragma unroll
+                for (int i = 0; i < S::NP; ++i) {
+                    s = __fmaf_rn(v2[i].x, v2[i].x, s);
+                    s = __fmaf_rn(v2[i].y, v2[i].y, s);
+                }
+                merge_class_winner(best[0], __float_as_uint(s), zc);
+            }
+        }
+        const int n = c_sat - c_same;
+        search_saturated<B>(T, c_same + n * slice / slices, c_same + n * (slice + 1) / slices, v2, best);
+        // the rest, one mantissa class after the other (slices share the classes, or the one class of the power-of-two format)
+        for (int cls = NCLS == 1 ? 0 : slice; cls < NCLS; cls += NCLS == 1 ? 1 : slices) {
+            int f0 = T.below[2 * cls][c_sat], n0 = T.below[2 * cls][c_zero] - f0;
+            int f1 = T.below[2 * cls + 1][c_sat], n1 = T.below[2 * cls + 1][c_zero] - f1;
+            if (NCLS == 1) {
+                const int a0 = n0 * slice / slices, a1 = n1 * slice / slices;
+                n0 = n0 * (slice + 1) / slices - a0;
+                n1 = n1 * (slice + 1) / slices - a1;
+                f0 += a0;
+                f1 += a1;
+            }
+            if (n0 + n1 == 0) continue;
+            const float Dr = T.clsD[cls], Rr = T.clsR[cls];
+            const float2 nDr2 = make_float2(-Dr, -Dr), Rr2 = make_float2(Rr, Rr);
+            float2 tb[S::NP];
+#pragma unroll
+            for (int i = 0; i < S::NP; ++i) tb[i] = quotient_pair(v2[i], nDr2, Rr2);
+            search_list<B, FMT, false>(T, 2 * cls, f0, n0, v2, tb, best);
+            search_list<B, FMT, true>(T, 2 * cls + 1, f1, n1, v2, tb, best);
+        }
+    }
+    // general path (IEEE division), candidate by candidate
+    const int n_general = live && !gr.fast ? NC - first : 0;
+    const int c_end = first + n_general * (slice + 1) / slices;
+    for (int c = first + n_general * slice / slices; c < c_end; ++c) {
+        const float D = T.D[c];
+        if (!(fabsf(D) <= 3.402823466e38f)) continue;  // decode scale overflowed: not usable
+        if constexpr (!S::ONEBLK) {
+#pragma unroll
+            for (int k = 0; k < S::NBL; ++k) {
+                merge_class_winner(best[k], __float_as_uint(general_sse<B, S::NP>(v2, k * S::BL, 0, D)), c);
+                merge_class_winner(best[S::NBL + k], __float_as_uint(general_sse<B, S::NP>(v2, k * S::BL, 1, D)), c);
+            }
+        } else {
+            float s = 0.0f;
+#pragma unroll
+            for (int i = 0; i < S::NP; ++i) {
+                const float a = v2[i].x, b = v2[i].y;
+                const float2 q = round_e2m1x2(quotient_general(a, D), quotient_general(b, D));
+                const float e0 = __fmaf_rn(-q.x, D, a);
+                s = __fmaf_rn(e0, e0, s);
+                const float e1 = __fmaf_rn(-q.y, D, b);
+                s = __fmaf_rn(e1, e1, s);
+            }
+            merge_class_winner(best[0], __float_as_uint(s), c);
+        }
+    }
+}
+
+// One thread searches its elements under every code, all of them evaluated in full; whole groups only (n_items counts
+// groups here).
 template <int DT, int B, int FMT>
-__global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs p) {
+__global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute_plain(QuantArgs p) {
     constexpr bool ONEBLK = (B >= 32);        // the thread owns exactly one block
     constexpr int G = brute_group_elems(B);     // elements per thread
     constexpr int NP = G / 2;                 // pairs per thread
@@ -400,7 +667,7 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs
     release_dependents();
     const float g = p.d_global_scale ? *p.d_global_scale : p.global_scale;
     const int first = (p.prevent_zero && FMT != kUE8M0) ? 1 : 0;
-    build_brute_tables<FMT>(T, g, first);
+    build_brute_tables<FMT, false>(T, g, first);
 
     const size_t stride = (size_t)gridDim.x * kThreads;
     double sse_sum = 0.0;                  // binary64 sum of the SSEs of this thread's blocks, in the order it stored them
@@ -445,8 +712,26 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs
                 search_list<B, FMT, false>(T, 2 * cls, 0, n0, v2, tb, best);
                 search_list<B, FMT, true>(T, 2 * cls + 1, 0, n1, v2, tb, best);
             }
-            // Dref = 1: the elements are their own quotients
-            search_list<B, FMT, false>(T, kFlatList, 0, T.cnt[kFlatList], v2, v2, best);
+            if (T.flat_min < 256) {   // codes outside the lists: the sum of squares of the elements, see search_group()
+                float2 s[NBL];
+                float s1 = 0.0f;
+#pragma unroll
+                for (int k = 0; k < NBL; ++k) s[k] = make_float2(0.0f, 0.0f);
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                    if constexpr (ONEBLK) {
+                        s1 = __fmaf_rn(v2[i].x, v2[i].x, s1);
+                        s1 = __fmaf_rn(v2[i].y, v2[i].y, s1);
+                    } else {
+                        s[i / BL] = __ffma2_rn(v2[i], v2[i], s[i / BL]);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < NBL; ++k) {
+                    merge_class_winner(best[k], __float_as_uint(ONEBLK ? s1 : s[k].x), T.flat_min);
+                    if constexpr (!ONEBLK) merge_class_winner(best[NBL + k], __float_as_uint(s[k].y), T.flat_min);
+                }
+            }
         }
 
         // general path (IEEE division), candidate by candidate: threads that hold a magnitude above
@@ -541,108 +826,234 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs
     }
 }
 
-// ------------------------------------------------------------------------------------------------
-// The blocks past the last whole per-thread group (block sizes up to 16 only): one block per
-// thread, general path.
-// ------------------------------------------------------------------------------------------------
+// One thread searches its elements under all codes; the warp stays together, lanes past the end idle.
 template <int DT, int B, int FMT>
-__global__ void k_brute_tail(QuantArgs p) {
-    const size_t b = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float my_sse = 0.0f;
-    if (b < p.n_items) {
-    const size_t blk = p.first_item + b;
+__global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs p) {
+    using S = BruteShape<B>;
+    __shared__ BruteTables T;
+    __shared__ unsigned long long key[kThreads / 32][32 * S::NBT];   // per warp: best of block k of lane l at k * 32 + l
+    wait_for_prior_grid();
+    release_dependents();
     const float g = p.d_global_scale ? *p.d_global_scale : p.global_scale;
     const int first = (p.prevent_zero && FMT != kUE8M0) ? 1 : 0;
-    float v[B];
-    load_elems<DT, B>(p.x, blk * B, v);
-    unsigned long long best = sse_key(__uint_as_float(0xFFFFFFFFu), first);
-    for (int c = first; c < num_codes(FMT); ++c) {
-        const float D = __fmul_rn(scale_value(FMT, c), g);
-        if (!(fabsf(D) <= 3.402823466e38f)) continue;
-        float s = 0.0f;
+    build_brute_tables<FMT, true>(T, g, first);
+    const float Rg = g >= kFastMin && g <= kFastMax ? __frcp_rn(g) : 0.0f;
+
+    const size_t n_groups = (p.n_items + S::NBT - 1) / S::NBT;
+    const size_t stride = (size_t)gridDim.x * kThreads;
+    const int lane = threadIdx.x & 31;
+    const SharedBest best = {&key[threadIdx.x >> 5][lane]};
+    double sse_sum = 0.0;                  // binary64 sum of the SSEs of this thread's blocks, in the order it stored them
+    for (size_t wbase = (size_t)blockIdx.x * kThreads + (threadIdx.x - lane); wbase < n_groups; wbase += stride) {
+        const size_t grp = wbase + lane;
+        const bool active = grp < n_groups;
+        const int blocks = active ? (int)min((size_t)S::NBT, p.n_items - grp * S::NBT) : 0;   // fewer in the last group
 #pragma unroll
-        for (int i = 0; i < B; i += 2) {
-            const float2 q = round_e2m1x2(quotient_general(v[i], D), quotient_general(v[i + 1], D));
-            const float e0 = __fmaf_rn(-q.x, D, v[i]);
-            s = __fmaf_rn(e0, e0, s);
-            const float e1 = __fmaf_rn(-q.y, D, v[i + 1]);
-            s = __fmaf_rn(e1, e1, s);
+        for (int k = 0; k < S::NBT; ++k) best[k] = sse_key(__uint_as_float(0xFFFFFFFFu), first);
+        float v[S::G];
+        {
+            float2 v2[S::NP];
+            load_group<DT, B>(v, p.x, grp * S::G, blocks * B);
+            const GroupRange gr = take_magnitudes<B>(v2, v);
+            search_group<B, FMT>(T, v2, gr, active, Rg, first, 0, 1, best);
         }
-        const unsigned long long k = sse_key(s, c);
-        if (k < best) best = k;
-    }
-    const int code = (int)(best & 0xFFu);
-    const float D = __fmul_rn(scale_value(FMT, code), g);
-    uint32_t packed[(B + 7) / 8];
+
+        // final encode with the winners; the elements are read again (from L2) rather than kept with their signs
+        load_group<DT, B>(v, p.x, grp * S::G, blocks * B);
+        float amax = 0.0f;
 #pragma unroll
-    for (int k = 0; k < (B + 7) / 8; ++k) packed[k] = 0;
+        for (int i = 0; i < S::G; ++i) amax = fmaxf(amax, fabsf(v[i]));
+        uint32_t packed[S::G / 8];
+        uint32_t sc[(S::NBT + 3) / 4];
+        uint32_t sw[S::NBT];
 #pragma unroll
-    for (int k = 0; k < B / 2; ++k)
-        packed[k / 4] |= pack_e2m1x2(quotient_general(v[2 * k], D), quotient_general(v[2 * k + 1], D)) << (8 * (k % 4));
-    store_bytes<B / 2>(p.codes + blk * (B / 2), packed);
-    p.scales[blk] = (uint8_t)code;
-    if (p.block_sse) p.block_sse[blk] = __uint_as_float((uint32_t)(best >> 32));
-    my_sse = __uint_as_float((uint32_t)(best >> 32));
+        for (int k = 0; k < (S::NBT + 3) / 4; ++k) sc[k] = 0;
+        float t[S::G];
+#pragma unroll
+        for (int kb = 0; kb < S::NBT; ++kb) {
+            const unsigned long long winner = best[kb];
+            const int code = (int)(winner & 0xFFu);
+            const float D = T.D[code];
+            const float R = T.R[code];
+            const bool fast = (R != 0.0f) && (amax <= kFastMax);
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                const int e = kb * B + i;
+                t[e] = fast ? quotient_corrected(v[e], D, R) : quotient_general(v[e], D);
+            }
+            sc[kb / 4] |= (uint32_t)code << (8 * (kb % 4));
+            sw[kb] = (uint32_t)(winner >> 32);
+        }
+#pragma unroll
+        for (int k = 0; k < S::G / 8; ++k)
+            packed[k] = pack_e2m1x8(t[8 * k], t[8 * k + 1], t[8 * k + 2], t[8 * k + 3], t[8 * k + 4], t[8 * k + 5], t[8 * k + 6], t[8 * k + 7]);
+        store_group<B>(p, grp, blocks, packed, sc, sw);
+#pragma unroll
+        for (int k = 0; k < S::NBT; ++k)
+            if (k < blocks) sse_sum = __dadd_rn(sse_sum, (double)__uint_as_float(sw[k]));
     }
-    // fused tensor-MSE partial sum: the kernel is one warp, every lane takes part (idle lanes add 0)
-    if (p.mse_partials != nullptr) warp_sum_to_partial(p, my_sse);
+    if (p.mse_partials != nullptr) {   // launch-uniform: fused tensor-MSE partial sum of this CTA
+        __syncthreads();               // the tables are no longer read: their memory serves as scratch
+        const double total = cta_sum_fixed_order(sse_sum, reinterpret_cast<double*>(&T));
+        if (threadIdx.x == 0) p.mse_partials[p.mse_first + blockIdx.x] = total;
+    }
+}
+
+// The same search for tensors that do not fill the chip with one thread per group: `slices` warps (2, 4 or 8) of a CTA share
+// 32 groups and take their part of the codes each (mantissa classes of the FP8 formats); the winners meet in shared
+// memory and the CTA encodes the elements together.
+template <int DT, int B, int FMT>
+__global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute_split(QuantArgs p, int slices) {
+    using S = BruteShape<B>;
+    constexpr int W = kThreads / 32;
+    constexpr int EPT = 32 * S::G / kThreads;      // elements of 32 groups that a thread encodes: at most one block
+    constexpr int NBW = 32 * S::NBT;               // blocks of 32 groups
+    __shared__ BruteTables T;
+    __shared__ unsigned long long key[W][NBW];     // per warp: best of block k of lane l at k * 32 + l
+    wait_for_prior_grid();
+    release_dependents();
+    const float g = p.d_global_scale ? *p.d_global_scale : p.global_scale;
+    const int first = (p.prevent_zero && FMT != kUE8M0) ? 1 : 0;
+    build_brute_tables<FMT, true>(T, g, first);
+    const float Rg = g >= kFastMin && g <= kFastMax ? __frcp_rn(g) : 0.0f;
+
+    const size_t n_groups = (p.n_items + S::NBT - 1) / S::NBT;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sets = W / slices;                   // sets of 32 groups the CTA works on
+    double sse_sum = 0.0;
+    for (size_t base = (size_t)blockIdx.x * (sets * 32); base < n_groups; base += (size_t)gridDim.x * (sets * 32)) {
+        {
+            const size_t grp = base + warp / slices * 32 + lane;
+            const int blocks = grp < n_groups ? (int)min((size_t)S::NBT, p.n_items - grp * S::NBT) : 0;
+            float v[S::G];
+            float2 v2[S::NP];
+            load_group<DT, B>(v, p.x, grp * S::G, blocks * B);
+            const GroupRange gr = take_magnitudes<B>(v2, v);
+            const SharedBest best = {&key[warp][lane]};
+#pragma unroll
+            for (int k = 0; k < S::NBT; ++k) best[k] = sse_key(__uint_as_float(0xFFFFFFFFu), first);
+            search_group<B, FMT>(T, v2, gr, grp < n_groups, Rg, first, warp % slices, slices, best);
+        }
+        __syncthreads();
+        for (int set = 0; set < sets; ++set) {
+            const size_t e0 = (base + set * 32) * S::G + threadIdx.x * EPT;
+            const int b = threadIdx.x * EPT / B;   // block of the set, in memory order
+            const size_t blk = e0 / B;
+            if (blk < p.n_items) {
+                const int at = (b % S::NBT) * 32 + b / S::NBT;
+                unsigned long long k = key[set * slices][at];
+                for (int w = 1; w < slices; ++w) k = min(k, key[set * slices + w][at]);
+                const int code = (int)(k & 0xFFu);
+                const float D = T.D[code], R = T.R[code];
+                float v[EPT];
+                load_elems<DT, EPT>(p.x, e0, v);
+                uint32_t packed = 0;
+#pragma unroll
+                for (int i = 0; i < EPT; i += 2) {
+                    const bool fast = R != 0.0f && fmaxf(fabsf(v[i]), fabsf(v[i + 1])) <= kFastMax;
+                    const float t0 = fast ? quotient_corrected(v[i], D, R) : quotient_general(v[i], D);
+                    const float t1 = fast ? quotient_corrected(v[i + 1], D, R) : quotient_general(v[i + 1], D);
+                    packed |= pack_e2m1x2(t0, t1) << (4 * i);
+                }
+                store_bytes<EPT / 2>(p.codes + e0 / 2, &packed);
+                if (e0 % B == 0) {
+                    const float sse = __uint_as_float((uint32_t)(k >> 32));
+                    p.scales[blk] = (uint8_t)code;
+                    if (p.block_sse) p.block_sse[blk] = sse;
+                    sse_sum = __dadd_rn(sse_sum, (double)sse);
+                }
+            }
+        }
+        __syncthreads();   // the keys have been read
+    }
+    if (p.mse_partials != nullptr) {
+        const double total = cta_sum_fixed_order(sse_sum, reinterpret_cast<double*>(&T));
+        if (threadIdx.x == 0) p.mse_partials[p.mse_first + blockIdx.x] = total;
+    }
+}
+
+// Resident CTAs per SM of a kernel (first use asks; racing threads store the same value).
+static cudaError_t resident_ctas(const void* kernel, size_t dynamic_bytes, int dev, std::atomic<int>* cache, size_t& ctas) {
+    int n = cache[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+        cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic_bytes);
+        if (err != cudaSuccess) return err;
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, dynamic_bytes);
+        if (err != cudaSuccess) return err;
+        if (n < 1) n = 1;
+        cache[dev].store(n, std::memory_order_relaxed);
+    }
+    ctas = (size_t)n;
+    return cudaSuccess;
 }
 
 template <int DT, int B, int FMT>
 static cudaError_t launch_brute_inst(const QuantArgs& a, cudaStream_t stream) {
-    static std::atomic<int> ctas_per_sm[kMaxDevices];   // first-use cache; racing threads store the same value
+    using S = BruteShape<B>;
+    static std::atomic<int> cache[3][kMaxDevices];
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    int resident = ctas_per_sm[dev].load(std::memory_order_relaxed);
-    if (resident == 0) {
-        int n = 0;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_brute<DT, B, FMT>, kThreads, 0);
-        if (err != cudaSuccess) return err;
-        resident = n > 0 ? n : 1;
-        ctas_per_sm[dev].store(resident, std::memory_order_relaxed);
+    const size_t n_groups = (a.n_items + S::NBT - 1) / S::NBT;
+    const size_t sms = (size_t)sm_count(dev);
+    const size_t per_sm = (n_groups + sms - 1) / sms;
+    // A tensor with fewer groups than threads that fit leaves SMs idle or with too few warps: its groups are split over 2 to 8
+    // warps.  (256, 384] per SM is the stretch in which some SMs would get a second CTA of 256 groups and the others one.
+    // fp32 Laplace under a tensor scale, UE4M3, B = 16, one warp per 32 groups -> split, us: 2^16 elements 41 -> 20 (8), 2^18 40 ->
+    // 24 (4), 2^19 40 -> 32 (2), 2^20.5 64 -> 57 (2); at 2^20 (221 per SM) 40 against 44, at 2^21 63 against 74: not split.
+    const int slices = per_sm <= 32 ? 8 : per_sm <= 64 ? 4 : (per_sm <= 128 || (per_sm > 256 && per_sm <= 384 && B <= 32)) ? 2 : 1;
+    // Under a tensor scale the codes of UE4M3 reach from the top of the tensor down by 17 binades only: next to none lies in
+    // the cheap stretches of search_group(), and the kernel without them is faster by the registers they take (16.8 M fp32
+    // Laplace elements, with -> without, us: B = 2 534 -> 499, 4 458 -> 440, 8 393 -> 371, 16 385 -> 367, 64 427 -> 420; B = 32
+    // 385 -> 391).  The other formats and unscaled UE4M3 gain (start -> with, B = 16): UE5M3 684 -> 543, UE8M0 660 ->
+    // 133, unscaled UE4M3 330 -> 273.
+    constexpr bool kHasPlain = FMT == kUE4M3 && B != 32;
+    const bool plain = kHasPlain && slices == 1 && (a.d_global_scale != nullptr || a.global_scale != 1.0f);
+    const void* kernel = reinterpret_cast<const void*>(k_brute<DT, B, FMT>);
+    if (slices > 1) kernel = reinterpret_cast<const void*>(k_brute_split<DT, B, FMT>);
+    if constexpr (kHasPlain) {
+        if (plain) kernel = reinterpret_cast<const void*>(k_brute_plain<DT, B, FMT>);
     }
-    constexpr size_t G = brute_group_elems(B);    // elements per thread of k_brute
-    const size_t n_blocks = a.n_items;
-    const size_t n_groups = n_blocks * B / G;
-    const size_t done = n_groups * G / B;
-    // The blocks past the last whole group go to the one-warp tail kernel.  With fused MSE partial sums it
-    // runs first and owns partial 0; the CTAs of the main kernel own the partials from 1 on.
-    auto launch_tail = [&]() -> cudaError_t {
-        if constexpr (B < 32) {
-            if (done < n_blocks) {
-                QuantArgs t = a;
-                t.first_item = done;
-                t.n_items = n_blocks - done;
-                t.mse_first = 0;
-                k_brute_tail<DT, B, FMT><<<1, 32, 0, stream>>>(t);
-                count_launch();
-                return cudaGetLastError();
-            }
-        }
-        return cudaSuccess;
+    size_t cap = 0;
+    err = resident_ctas(kernel, 0, dev, cache[slices > 1 ? 1 : plain ? 2 : 0], cap);
+    if (err != cudaSuccess) return err;
+    cap *= sms;
+    if (a.mse_partials && cap > (size_t)kMsePartials) cap = kMsePartials;
+    const unsigned per_cta = (unsigned)(kThreads / slices);
+    auto ctas = [&](size_t groups) {
+        const size_t want = (groups + per_cta - 1) / per_cta;
+        return (unsigned)(want < cap ? want : cap);
     };
-    if (a.mse_partials) {
-        err = launch_tail();
-        if (err != cudaSuccess) return err;
-    }
-    if (n_groups > 0) {
+    unsigned grid = ctas(n_groups), rest = 0;
+    if (slices > 1) {
+        err = launch_pdl(k_brute_split<DT, B, FMT>, grid, kThreads, 0, stream, a, slices);
+    } else if (!plain) {
+        err = launch_pdl(k_brute<DT, B, FMT>, grid, kThreads, 0, stream, a);
+    } else if constexpr (kHasPlain) {
+        // whole groups; the blocks past the last one go to the split kernel (one CTA, partial sum 0)
         QuantArgs m = a;
-        m.n_items = n_groups;
-        m.mse_first = (done < n_blocks) ? 1 : 0;
-        const size_t want = (n_groups + kThreads - 1) / kThreads;
-        size_t cap = (size_t)sm_count(dev) * (size_t)resident;
-        if (a.mse_partials && cap > (size_t)kMsePartials - 1) cap = kMsePartials - 1;
-        const unsigned grid = (unsigned)(want < cap ? want : cap);
-        err = launch_pdl(k_brute<DT, B, FMT>, grid, kThreads, 0, stream, m);
-        count_launch();
-        if (err != cudaSuccess) return err;
-        if (a.mse_n_partials) *a.mse_n_partials = (int)grid + m.mse_first;
-    } else if (a.mse_n_partials) {
-        *a.mse_n_partials = (done < n_blocks) ? 1 : 0;
+        m.n_items = a.n_items / S::NBT;
+        const size_t done = m.n_items * S::NBT;
+        if (done < a.n_items) {
+            QuantArgs t = a;
+            t.x = static_cast<const char*>(a.x) + done * B * elem_bytes(DT);
+            t.codes = a.codes + done * B / 2;
+            t.scales = a.scales + done;
+            if (a.block_sse) t.block_sse = a.block_sse + done;
+            t.n_items = a.n_items - done;
+            rest = 1;
+            err = launch_pdl(k_brute_split<DT, B, FMT>, 1u, kThreads, 0, stream, t, 8);
+            count_launch();
+            if (err != cudaSuccess) return err;
+        }
+        m.mse_first = (int)rest;
+        if (a.mse_partials && cap > (size_t)kMsePartials - rest) cap = kMsePartials - rest;
+        grid = ctas(m.n_items);
+        err = launch_pdl(k_brute_plain<DT, B, FMT>, grid, kThreads, 0, stream, m);
     }
-    if (!a.mse_partials) err = launch_tail();
+    count_launch();
+    if (err == cudaSuccess && a.mse_n_partials) *a.mse_n_partials = (int)(grid + rest);
     return err;
 }
 

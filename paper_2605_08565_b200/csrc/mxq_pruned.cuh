@@ -189,16 +189,6 @@ __device__ __forceinline__ float2 sse_two_candidates(const float2 (&v2)[pruned_v
     return s;
 }
 
-// Largest code whose value is at most S (0 if there is none), S >= 0.
-template <int FMT>
-__device__ __forceinline__ int floor_code(float S) {
-    const uint32_t b = __float_as_uint(S);
-    constexpr int bias = (FMT == kUE4M3) ? 7 : 15;
-    const int normal = (int)(b >> 20) - ((127 - bias) << 3);
-    const int sub = __float2int_rz(__fmul_rn(S, (float)(1 << (bias + 2))));
-    return min(normal < 8 ? sub : normal, num_codes(FMT) - 1);
-}
-
 __device__ __forceinline__ float sqrt_approx(float x) {
     float r;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -807,21 +797,6 @@ __global__ void __launch_bounds__(kThreads) k_pruned_pow2(QuantArgs p) {
         const double total = cta_sum_fixed_order(sse_sum, scratch);
         if (threadIdx.x == 0) p.mse_partials[p.mse_first + blockIdx.x] = total;
     }
-}
-
-// Resident CTAs per SM of a kernel (first use asks; racing threads store the same value).
-static cudaError_t resident_ctas(const void* kernel, size_t dynamic_bytes, int dev, std::atomic<int>* cache, size_t& ctas) {
-    int n = cache[dev].load(std::memory_order_relaxed);
-    if (n == 0) {
-        cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic_bytes);
-        if (err != cudaSuccess) return err;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, dynamic_bytes);
-        if (err != cudaSuccess) return err;
-        if (n < 1) n = 1;
-        cache[dev].store(n, std::memory_order_relaxed);
-    }
-    ctas = (size_t)n;
-    return cudaSuccess;
 }
 
 template <int DT, int B, int FMT>
