@@ -287,10 +287,9 @@ __device__ __forceinline__ int floor_code(float S) {
 // All members of one range of one list (one mantissa class, one residual kind) against the
 // thread's elements; the winner of every block is folded into best[].
 // Members first .. first + cnt_raw - 1 of the list are evaluated.
-template <int B, int FMT, bool HALF, int NP, typename Best>
+template <int B, int FMT, bool HALF, bool ONEBLK, int NP, typename Best>
 __device__ __forceinline__ void search_list(const BruteTables& T, int list, int first, int cnt_raw,
                                             const float2 (&v2)[NP], const float2 (&tb)[NP], Best& best) {
-    constexpr bool ONEBLK = (B >= 32);
     constexpr int BL = ONEBLK ? NP : B;
     constexpr int NBL = NP / BL;
     constexpr int NBT = ONEBLK ? 1 : 2 * NBL;
@@ -377,10 +376,9 @@ __device__ __forceinline__ void search_list(const BruteTables& T, int list, int 
 // size up to 32 -- the kernels sit within a few registers of that limit, and falling to one
 // resident CTA costs far more (measured: 8 % at B = 16) than the allocator's squeeze; B = 64 needs
 // about 170 registers and runs one CTA per SM.
-// Elements a thread of k_brute owns: one block for B >= 32, else 32; 16 for B = 2, whose 16
-// running minima per 32 elements otherwise leave room for one CTA per SM only (measured: 496 -> 452 us;
-// B = 4 and B = 8 lose with 16).
-__host__ __device__ constexpr int brute_group_elems(int B) { return B >= 32 ? B : (B == 2 ? 16 : 32); }
+// Elements a thread owns: one block for B >= 32, else 32; 16 for B = 2 and 4, whose 16 or 8 running minima per 32 elements
+// otherwise leave room for one CTA per SM only, or spill (16.8 M elements: B = 2 496 -> 452 us, B = 4 662 -> 632).
+__host__ __device__ constexpr int brute_group_elems(int B) { return B >= 32 ? B : (B <= 4 ? 16 : 32); }
 
 constexpr int brute_min_ctas(int B) { return B <= 32 ? 2 : 1; }
 
@@ -390,10 +388,11 @@ struct SharedBest {
     __device__ __forceinline__ unsigned long long& operator[](int k) const { return p[32 * k]; }
 };
 
-template <int B>
+// G: elements per thread.
+template <int B, int G_>
 struct BruteShape {
-    static constexpr bool ONEBLK = (B >= 32);       // the thread owns exactly one block
-    static constexpr int G = brute_group_elems(B);  // elements per thread
+    static constexpr int G = G_;
+    static constexpr bool ONEBLK = (G == B);        // the thread owns exactly one block
     static constexpr int NP = G / 2;                // pairs per thread
     static constexpr int BL = ONEBLK ? NP : B;      // elements of one block inside one half
     static constexpr int NBL = NP / BL;             // blocks per half (1 when ONEBLK)
@@ -409,9 +408,9 @@ struct GroupRange {
 
 // A thread's elements.  n_here: elements of the tensor in this group (a multiple of B, at most G); what is missing is taken
 // as zero.
-template <int DT, int B>
-__device__ __forceinline__ void load_group(float (&v)[BruteShape<B>::G], const void* x, size_t e0, int n_here) {
-    using S = BruteShape<B>;
+template <int DT, int B, int G>
+__device__ __forceinline__ void load_group(float (&v)[BruteShape<B, G>::G], const void* x, size_t e0, int n_here) {
+    using S = BruteShape<B, G>;
     if (n_here >= S::G) {
         load_elems<DT, S::G>(x, e0, v);
         return;
@@ -430,11 +429,21 @@ __device__ __forceinline__ void load_group(float (&v)[BruteShape<B>::G], const v
     }
 }
 
-// Stores a thread's results; blocks: how many of them the tensor has (fewer than NBT in its last group).
+// First group of a thread.  Sets of 32 groups go round the CTAs before they go round a CTA's warps, so that a tensor, or
+// its last trip, that does not occupy every warp is spread over all SMs (2^20.5 elements, B = 16: 64 -> 50 us).  Not for
+// B = 32, where a CTA's warps then run apart and 16.8 M elements take 565 us instead of 538.
+__host__ __device__ constexpr bool brute_spread(int B) { return B != 32; }
 template <int B>
-__device__ __forceinline__ void store_group(const QuantArgs& p, size_t grp, int blocks, const uint32_t (&packed)[BruteShape<B>::G / 8],
-                                            const uint32_t (&sc)[(BruteShape<B>::NBT + 3) / 4], const uint32_t (&sw)[BruteShape<B>::NBT]) {
-    using S = BruteShape<B>;
+__device__ __forceinline__ size_t first_group() {
+    if constexpr (!brute_spread(B)) return (size_t)blockIdx.x * kThreads + threadIdx.x;
+    return ((size_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+}
+
+// Stores a thread's results; blocks: how many of them the tensor has (fewer than NBT in its last group).
+template <int B, int G>
+__device__ __forceinline__ void store_group(const QuantArgs& p, size_t grp, int blocks, const uint32_t (&packed)[BruteShape<B, G>::G / 8],
+                                            const uint32_t (&sc)[(BruteShape<B, G>::NBT + 3) / 4], const uint32_t (&sw)[BruteShape<B, G>::NBT]) {
+    using S = BruteShape<B, G>;
     if (blocks == S::NBT) {
         store_bytes<S::G / 2>(p.codes + grp * (S::G / 2), packed);
         store_bytes<S::NBT>(p.scales + grp * S::NBT, sc);
@@ -460,9 +469,9 @@ __device__ __forceinline__ void store_group(const QuantArgs& p, size_t grp, int 
 
 // Their magnitudes (an SSE does not depend on signs): pair i = adjacent elements (one block per thread) or element i of
 // either half.
-template <int B>
-__device__ __forceinline__ GroupRange take_magnitudes(float2 (&v2)[BruteShape<B>::NP], float (&v)[BruteShape<B>::G]) {
-    using S = BruteShape<B>;
+template <int B, int G>
+__device__ __forceinline__ GroupRange take_magnitudes(float2 (&v2)[BruteShape<B, G>::NP], float (&v)[BruteShape<B, G>::G]) {
+    using S = BruteShape<B, G>;
     constexpr float kTiny = 2.168404344971009e-19f;  // 2^-62
     GroupRange r;
     r.amax = 0.0f;
@@ -482,10 +491,10 @@ __device__ __forceinline__ GroupRange take_magnitudes(float2 (&v2)[BruteShape<B>
 }
 
 // SSEs of all blocks of a thread when every element saturates, for the codes lo .. hi - 1: q = 6 and e = fma(6, -D, |v|).
-template <int B>
-__device__ __forceinline__ void search_saturated(const BruteTables& T, int lo, int hi, const float2 (&v2)[BruteShape<B>::NP],
+template <int B, int G>
+__device__ __forceinline__ void search_saturated(const BruteTables& T, int lo, int hi, const float2 (&v2)[BruteShape<B, G>::NP],
                                                  const SharedBest& best) {
-    using S = BruteShape<B>;
+    using S = BruteShape<B, G>;
     if (lo >= hi) return;
     uint32_t cbest[S::NBT];
     int ccode[S::NBT];
@@ -540,10 +549,10 @@ __device__ __forceinline__ void search_saturated(const BruteTables& T, int lo, i
 //                     smallest of these codes, which is how the full evaluation of each would end.
 //   D <= lo / 6       (no zero among the elements) every element saturates: the error is fl(|v| - 6 D), two packed FMAs
 //                     per pair of elements and code instead of quotient, rounding, widening and two FMAs.
-template <int B, int FMT>
-__device__ __forceinline__ void search_group(const BruteTables& T, const float2 (&v2)[BruteShape<B>::NP], const GroupRange& gr, bool live,
+template <int B, int G, int FMT>
+__device__ __forceinline__ void search_group(const BruteTables& T, const float2 (&v2)[BruteShape<B, G>::NP], const GroupRange& gr, bool live,
                                              float Rg, int first, int slice, int slices, const SharedBest& best) {
-    using S = BruteShape<B>;
+    using S = BruteShape<B, G>;
     constexpr int NCLS = (FMT == kUE8M0) ? 1 : 8;
     constexpr int NC = num_codes(FMT);
     constexpr uint32_t kFull = 0xFFFFFFFFu;
@@ -599,7 +608,7 @@ __device__ __forceinline__ void search_group(const BruteTables& T, const float2 
             }
         }
         const int n = c_sat - c_same;
-        search_saturated<B>(T, c_same + n * slice / slices, c_same + n * (slice + 1) / slices, v2, best);
+        search_saturated<B, G>(T, c_same + n * slice / slices, c_same + n * (slice + 1) / slices, v2, best);
         // the rest, one mantissa class after the other (slices share the classes, or the one class of the power-of-two format)
         for (int cls = NCLS == 1 ? 0 : slice; cls < NCLS; cls += NCLS == 1 ? 1 : slices) {
             int f0 = T.below[2 * cls][c_sat], n0 = T.below[2 * cls][c_zero] - f0;
@@ -617,8 +626,8 @@ __device__ __forceinline__ void search_group(const BruteTables& T, const float2 
             float2 tb[S::NP];
 #pragma unroll
             for (int i = 0; i < S::NP; ++i) tb[i] = quotient_pair(v2[i], nDr2, Rr2);
-            search_list<B, FMT, false>(T, 2 * cls, f0, n0, v2, tb, best);
-            search_list<B, FMT, true>(T, 2 * cls + 1, f1, n1, v2, tb, best);
+            search_list<B, FMT, false, S::ONEBLK>(T, 2 * cls, f0, n0, v2, tb, best);
+            search_list<B, FMT, true, S::ONEBLK>(T, 2 * cls + 1, f1, n1, v2, tb, best);
         }
     }
     // general path (IEEE division), candidate by candidate
@@ -651,10 +660,9 @@ __device__ __forceinline__ void search_group(const BruteTables& T, const float2 
 
 // One thread searches its elements under every code, all of them evaluated in full; whole groups only (n_items counts
 // groups here).
-template <int DT, int B, int FMT>
+template <int DT, int B, int G, int FMT>
 __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute_plain(QuantArgs p) {
-    constexpr bool ONEBLK = (B >= 32);        // the thread owns exactly one block
-    constexpr int G = brute_group_elems(B);     // elements per thread
+    constexpr bool ONEBLK = (G == B);         // the thread owns exactly one block
     constexpr int NP = G / 2;                 // pairs per thread
     constexpr int BL = ONEBLK ? NP : B;         // elements of one block inside one half
     constexpr int NBL = NP / BL;              // blocks per half (1 when ONEBLK)
@@ -671,7 +679,7 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute_plain(Qua
 
     const size_t stride = (size_t)gridDim.x * kThreads;
     double sse_sum = 0.0;                  // binary64 sum of the SSEs of this thread's blocks, in the order it stored them
-    for (size_t grp = (size_t)blockIdx.x * kThreads + threadIdx.x; grp < p.n_items; grp += stride) {
+    for (size_t grp = first_group<B>(); grp < p.n_items; grp += stride) {
         float2 v2[NP];
         float amax = 0.0f;
         bool tiny = false;   // a nonzero magnitude below 2^-62: its quotient by Dref may be inexact
@@ -709,8 +717,8 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute_plain(Qua
                 if (n0 + n1 == 0) continue;
                 float2 tb[NP];
                 class_quotients(cls, tb);
-                search_list<B, FMT, false>(T, 2 * cls, 0, n0, v2, tb, best);
-                search_list<B, FMT, true>(T, 2 * cls + 1, 0, n1, v2, tb, best);
+                search_list<B, FMT, false, ONEBLK>(T, 2 * cls, 0, n0, v2, tb, best);
+                search_list<B, FMT, true, ONEBLK>(T, 2 * cls + 1, 0, n1, v2, tb, best);
             }
             if (T.flat_min < 256) {   // codes outside the lists: the sum of squares of the elements, see search_group()
                 float2 s[NBL];
@@ -827,9 +835,9 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute_plain(Qua
 }
 
 // One thread searches its elements under all codes; the warp stays together, lanes past the end idle.
-template <int DT, int B, int FMT>
+template <int DT, int B, int G, int FMT>
 __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs p) {
-    using S = BruteShape<B>;
+    using S = BruteShape<B, G>;
     __shared__ BruteTables T;
     __shared__ unsigned long long key[kThreads / 32][32 * S::NBT];   // per warp: best of block k of lane l at k * 32 + l
     wait_for_prior_grid();
@@ -844,7 +852,7 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs
     const int lane = threadIdx.x & 31;
     const SharedBest best = {&key[threadIdx.x >> 5][lane]};
     double sse_sum = 0.0;                  // binary64 sum of the SSEs of this thread's blocks, in the order it stored them
-    for (size_t wbase = (size_t)blockIdx.x * kThreads + (threadIdx.x - lane); wbase < n_groups; wbase += stride) {
+    for (size_t wbase = first_group<B>() - lane; wbase < n_groups; wbase += stride) {
         const size_t grp = wbase + lane;
         const bool active = grp < n_groups;
         const int blocks = active ? (int)min((size_t)S::NBT, p.n_items - grp * S::NBT) : 0;   // fewer in the last group
@@ -853,13 +861,13 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs
         float v[S::G];
         {
             float2 v2[S::NP];
-            load_group<DT, B>(v, p.x, grp * S::G, blocks * B);
-            const GroupRange gr = take_magnitudes<B>(v2, v);
-            search_group<B, FMT>(T, v2, gr, active, Rg, first, 0, 1, best);
+            load_group<DT, B, G>(v, p.x, grp * S::G, blocks * B);
+            const GroupRange gr = take_magnitudes<B, G>(v2, v);
+            search_group<B, G, FMT>(T, v2, gr, active, Rg, first, 0, 1, best);
         }
 
         // final encode with the winners; the elements are read again (from L2) rather than kept with their signs
-        load_group<DT, B>(v, p.x, grp * S::G, blocks * B);
+        load_group<DT, B, G>(v, p.x, grp * S::G, blocks * B);
         float amax = 0.0f;
 #pragma unroll
         for (int i = 0; i < S::G; ++i) amax = fmaxf(amax, fabsf(v[i]));
@@ -887,7 +895,7 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs
 #pragma unroll
         for (int k = 0; k < S::G / 8; ++k)
             packed[k] = pack_e2m1x8(t[8 * k], t[8 * k + 1], t[8 * k + 2], t[8 * k + 3], t[8 * k + 4], t[8 * k + 5], t[8 * k + 6], t[8 * k + 7]);
-        store_group<B>(p, grp, blocks, packed, sc, sw);
+        store_group<B, G>(p, grp, blocks, packed, sc, sw);
 #pragma unroll
         for (int k = 0; k < S::NBT; ++k)
             if (k < blocks) sse_sum = __dadd_rn(sse_sum, (double)__uint_as_float(sw[k]));
@@ -902,9 +910,9 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs
 // The same search for tensors that do not fill the chip with one thread per group: `slices` warps (2, 4 or 8) of a CTA share
 // 32 groups and take their part of the codes each (mantissa classes of the FP8 formats); the winners meet in shared
 // memory and the CTA encodes the elements together.
-template <int DT, int B, int FMT>
+template <int DT, int B, int G, int FMT>
 __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute_split(QuantArgs p, int slices) {
-    using S = BruteShape<B>;
+    using S = BruteShape<B, G>;
     constexpr int W = kThreads / 32;
     constexpr int EPT = 32 * S::G / kThreads;      // elements of 32 groups that a thread encodes: at most one block
     constexpr int NBW = 32 * S::NBT;               // blocks of 32 groups
@@ -927,12 +935,12 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute_split(Qua
             const int blocks = grp < n_groups ? (int)min((size_t)S::NBT, p.n_items - grp * S::NBT) : 0;
             float v[S::G];
             float2 v2[S::NP];
-            load_group<DT, B>(v, p.x, grp * S::G, blocks * B);
-            const GroupRange gr = take_magnitudes<B>(v2, v);
+            load_group<DT, B, G>(v, p.x, grp * S::G, blocks * B);
+            const GroupRange gr = take_magnitudes<B, G>(v2, v);
             const SharedBest best = {&key[warp][lane]};
 #pragma unroll
             for (int k = 0; k < S::NBT; ++k) best[k] = sse_key(__uint_as_float(0xFFFFFFFFu), first);
-            search_group<B, FMT>(T, v2, gr, grp < n_groups, Rg, first, warp % slices, slices, best);
+            search_group<B, G, FMT>(T, v2, gr, grp < n_groups, Rg, first, warp % slices, slices, best);
         }
         __syncthreads();
         for (int set = 0; set < sets; ++set) {
@@ -987,9 +995,9 @@ static cudaError_t resident_ctas(const void* kernel, size_t dynamic_bytes, int d
     return cudaSuccess;
 }
 
-template <int DT, int B, int FMT>
-static cudaError_t launch_brute_inst(const QuantArgs& a, cudaStream_t stream) {
-    using S = BruteShape<B>;
+template <int DT, int B, int FMT, int G>
+static cudaError_t launch_brute_size(const QuantArgs& a, int slices, cudaStream_t stream) {
+    using S = BruteShape<B, G>;
     static std::atomic<int> cache[3][kMaxDevices];
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -997,12 +1005,6 @@ static cudaError_t launch_brute_inst(const QuantArgs& a, cudaStream_t stream) {
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     const size_t n_groups = (a.n_items + S::NBT - 1) / S::NBT;
     const size_t sms = (size_t)sm_count(dev);
-    const size_t per_sm = (n_groups + sms - 1) / sms;
-    // A tensor with fewer groups than threads that fit leaves SMs idle or with too few warps: its groups are split over 2 to 8
-    // warps.  (256, 384] per SM is the stretch in which some SMs would get a second CTA of 256 groups and the others one.
-    // fp32 Laplace under a tensor scale, UE4M3, B = 16, one warp per 32 groups -> split, us: 2^16 elements 41 -> 20 (8), 2^18 40 ->
-    // 24 (4), 2^19 40 -> 32 (2), 2^20.5 64 -> 57 (2); at 2^20 (221 per SM) 40 against 44, at 2^21 63 against 74: not split.
-    const int slices = per_sm <= 32 ? 8 : per_sm <= 64 ? 4 : (per_sm <= 128 || (per_sm > 256 && per_sm <= 384 && B <= 32)) ? 2 : 1;
     // Under a tensor scale the codes of UE4M3 reach from the top of the tensor down by 17 binades only: next to none lies in
     // the cheap stretches of search_group(), and the kernel without them is faster by the registers they take (16.8 M fp32
     // Laplace elements, with -> without, us: B = 2 534 -> 499, 4 458 -> 440, 8 393 -> 371, 16 385 -> 367, 64 427 -> 420; B = 32
@@ -1010,26 +1012,26 @@ static cudaError_t launch_brute_inst(const QuantArgs& a, cudaStream_t stream) {
     // 133, unscaled UE4M3 330 -> 273.
     constexpr bool kHasPlain = FMT == kUE4M3 && B != 32;
     const bool plain = kHasPlain && slices == 1 && (a.d_global_scale != nullptr || a.global_scale != 1.0f);
-    const void* kernel = reinterpret_cast<const void*>(k_brute<DT, B, FMT>);
-    if (slices > 1) kernel = reinterpret_cast<const void*>(k_brute_split<DT, B, FMT>);
+    const void* kernel = reinterpret_cast<const void*>(k_brute<DT, B, G, FMT>);
+    if (slices > 1) kernel = reinterpret_cast<const void*>(k_brute_split<DT, B, G, FMT>);
     if constexpr (kHasPlain) {
-        if (plain) kernel = reinterpret_cast<const void*>(k_brute_plain<DT, B, FMT>);
+        if (plain) kernel = reinterpret_cast<const void*>(k_brute_plain<DT, B, G, FMT>);
     }
     size_t cap = 0;
     err = resident_ctas(kernel, 0, dev, cache[slices > 1 ? 1 : plain ? 2 : 0], cap);
     if (err != cudaSuccess) return err;
     cap *= sms;
     if (a.mse_partials && cap > (size_t)kMsePartials) cap = kMsePartials;
-    const unsigned per_cta = (unsigned)(kThreads / slices);
+    const unsigned per_cta = slices > 1 ? (unsigned)(kThreads / slices) : brute_spread(B) ? 32u : (unsigned)kThreads;
     auto ctas = [&](size_t groups) {
         const size_t want = (groups + per_cta - 1) / per_cta;
         return (unsigned)(want < cap ? want : cap);
     };
     unsigned grid = ctas(n_groups), rest = 0;
     if (slices > 1) {
-        err = launch_pdl(k_brute_split<DT, B, FMT>, grid, kThreads, 0, stream, a, slices);
+        err = launch_pdl(k_brute_split<DT, B, G, FMT>, grid, kThreads, 0, stream, a, slices);
     } else if (!plain) {
-        err = launch_pdl(k_brute<DT, B, FMT>, grid, kThreads, 0, stream, a);
+        err = launch_pdl(k_brute<DT, B, G, FMT>, grid, kThreads, 0, stream, a);
     } else if constexpr (kHasPlain) {
         // whole groups; the blocks past the last one go to the split kernel (one CTA, partial sum 0)
         QuantArgs m = a;
@@ -1043,18 +1045,41 @@ static cudaError_t launch_brute_inst(const QuantArgs& a, cudaStream_t stream) {
             if (a.block_sse) t.block_sse = a.block_sse + done;
             t.n_items = a.n_items - done;
             rest = 1;
-            err = launch_pdl(k_brute_split<DT, B, FMT>, 1u, kThreads, 0, stream, t, 8);
+            err = launch_pdl(k_brute_split<DT, B, G, FMT>, 1u, kThreads, 0, stream, t, 8);
             count_launch();
             if (err != cudaSuccess) return err;
         }
         m.mse_first = (int)rest;
         if (a.mse_partials && cap > (size_t)kMsePartials - rest) cap = kMsePartials - rest;
         grid = ctas(m.n_items);
-        err = launch_pdl(k_brute_plain<DT, B, FMT>, grid, kThreads, 0, stream, m);
+        err = launch_pdl(k_brute_plain<DT, B, G, FMT>, grid, kThreads, 0, stream, m);
     }
     count_launch();
     if (err == cudaSuccess && a.mse_n_partials) *a.mse_n_partials = (int)(grid + rest);
     return err;
+}
+
+template <int DT, int B, int FMT>
+static cudaError_t launch_brute_inst(const QuantArgs& a, cudaStream_t stream) {
+    int dev = 0;
+    const cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    constexpr int G = brute_group_elems(B);
+    const size_t n_groups = (a.n_items * B + G - 1) / G;
+    const size_t sms = (size_t)sm_count(dev);
+    const size_t per_sm = (n_groups + sms - 1) / sms;
+    // A tensor with fewer groups than threads that fit leaves SMs idle or with too few warps.  Up to 32, 64, 128 groups per
+    // SM its groups are split over 8, 4, 2 warps.  Beside and beyond that groups of 16 help B = 8 up to four million elements,
+    // and B = 16 in a short stretch (a pair of lanes then holds two codes instead of two blocks; UE8M0, with few full
+    // evaluations, does not mind).  fp32 Laplace under a tensor scale, UE4M3, us, groups of 32 not split -> as chosen here: 2^16
+    // elements, B = 8 42 -> 19, B = 16 41 -> 18; 2^18 40 -> 23, 39 -> 23; 2^19 40 -> 28, 39 -> 28; 2^19.5 40 -> 32, 40 ->
+    // 33; 2^21.5 88 -> 81 (B = 8).
+    if constexpr (B == 8 || B == 16) {
+        const bool small = B == 8 ? (per_sm > 64 && per_sm <= 1024) : (per_sm > 128 && (per_sm <= 200 || FMT == kUE8M0));
+        if (small) return launch_brute_size<DT, B, FMT, 16>(a, 1, stream);
+    }
+    const int slices = per_sm <= 32 ? 8 : per_sm <= 64 ? 4 : per_sm <= 128 ? 2 : 1;
+    return launch_brute_size<DT, B, FMT, G>(a, slices, stream);
 }
 
 template <int DT, int B>

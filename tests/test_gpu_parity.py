@@ -151,14 +151,14 @@ def test_pruned_sweep_at_the_edges_of_its_bounds(dtype, B, fmt):
         mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 0)
 
 
-@pytest.mark.parametrize("B, fmt, g", [(2, mxq.MXQ_SF_UE4M3, 0.0131), (8, mxq.MXQ_SF_UE4M3, 0.0131), (16, mxq.MXQ_SF_UE5M3, 1.0), (32, mxq.MXQ_SF_UE8M0, 1.0),
+@pytest.mark.parametrize("B, fmt, g", [(2, mxq.MXQ_SF_UE4M3, 0.0131), (4, mxq.MXQ_SF_UE8M0, 0.0131), (8, mxq.MXQ_SF_UE4M3, 0.0131), (16, mxq.MXQ_SF_UE5M3, 1.0), (32, mxq.MXQ_SF_UE8M0, 1.0),
                                        (64, mxq.MXQ_SF_UE4M3, 1.0)])
 def test_full_sweep_around_the_limits_of_its_split(B, fmt, g):
     """The warps a group of elements is split over go down from eight to one as the tensor grows; sizes on either side of
     each limit, ending in part of a group, with zeros, large and small stretches among the elements."""
-    group = max(B, 16 if B == 2 else 32)
+    group = max(B, 16 if B <= 4 else 32)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    for k, groups in enumerate((32 * sms, 32 * sms + 1, 64 * sms + 1, 128 * sms + 1, 256 * sms + 33)):
+    for k, groups in enumerate((32 * sms, 32 * sms + 1, 64 * sms + 1, 128 * sms + 1, 200 * sms + 33)):
         n = groups * group - (group - B)
         x = inputs.student_t(n, 4, 0.05, 600 + B + k, torch.float32)
         x[::4099] = 0.0
