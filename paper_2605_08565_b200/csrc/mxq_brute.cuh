@@ -429,14 +429,14 @@ __device__ __forceinline__ void load_group(float (&v)[BruteShape<B, G>::G], cons
     }
 }
 
-// First group of a thread.  Sets of 32 groups go round the CTAs before they go round a CTA's warps, so that a tensor, or
+// Where a warp starts.  Sets of 32 groups go round the CTAs before they go round a CTA's warps, so that a tensor, or
 // its last trip, that does not occupy every warp is spread over all SMs (2^20.5 elements, B = 16: 64 -> 50 us).  Not for
 // B = 32, where a CTA's warps then run apart and 16.8 M elements take 565 us instead of 538.
 __host__ __device__ constexpr bool brute_spread(int B) { return B != 32; }
 template <int B>
-__device__ __forceinline__ size_t first_group() {
-    if constexpr (!brute_spread(B)) return (size_t)blockIdx.x * kThreads + threadIdx.x;
-    return ((size_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+__device__ __forceinline__ size_t first_set() {   // of the warp, in groups
+    if constexpr (!brute_spread(B)) return (size_t)blockIdx.x * kThreads + (threadIdx.x & ~31u);
+    return ((size_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32;
 }
 
 // Stores a thread's results; blocks: how many of them the tensor has (fewer than NBT in its last group).
@@ -679,7 +679,7 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute_plain(Qua
 
     const size_t stride = (size_t)gridDim.x * kThreads;
     double sse_sum = 0.0;                  // binary64 sum of the SSEs of this thread's blocks, in the order it stored them
-    for (size_t grp = first_group<B>(); grp < p.n_items; grp += stride) {
+    for (size_t grp = first_set<B>() + (threadIdx.x & 31); grp < p.n_items; grp += stride) {
         float2 v2[NP];
         float amax = 0.0f;
         bool tiny = false;   // a nonzero magnitude below 2^-62: its quotient by Dref may be inexact
@@ -852,7 +852,7 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs
     const int lane = threadIdx.x & 31;
     const SharedBest best = {&key[threadIdx.x >> 5][lane]};
     double sse_sum = 0.0;                  // binary64 sum of the SSEs of this thread's blocks, in the order it stored them
-    for (size_t wbase = first_group<B>() - lane; wbase < n_groups; wbase += stride) {
+    for (size_t wbase = first_set<B>(); wbase < n_groups; wbase += stride) {
         const size_t grp = wbase + lane;
         const bool active = grp < n_groups;
         const int blocks = active ? (int)min((size_t)S::NBT, p.n_items - grp * S::NBT) : 0;   // fewer in the last group
@@ -1078,7 +1078,8 @@ static cudaError_t launch_brute_inst(const QuantArgs& a, cudaStream_t stream) {
         const bool small = B == 8 ? (per_sm > 64 && per_sm <= 1024) : (per_sm > 128 && (per_sm <= 200 || FMT == kUE8M0));
         if (small) return launch_brute_size<DT, B, FMT, 16>(a, 1, stream);
     }
-    const int slices = per_sm <= 32 ? 8 : per_sm <= 64 ? 4 : per_sm <= 128 ? 2 : 1;
+    // (256, 384] at B = 32: without the spreading some SMs would get a second CTA of 256 groups and the others one (68 -> 58 us)
+    const int slices = per_sm <= 32 ? 8 : per_sm <= 64 ? 4 : (per_sm <= 128 || (!brute_spread(B) && per_sm > 256 && per_sm <= 384)) ? 2 : 1;
     return launch_brute_size<DT, B, FMT, G>(a, slices, stream);
 }
 
