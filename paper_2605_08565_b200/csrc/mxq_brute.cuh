@@ -980,21 +980,6 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute_split(Qua
     }
 }
 
-// Resident CTAs per SM of a kernel (first use asks; racing threads store the same value).
-static cudaError_t resident_ctas(const void* kernel, size_t dynamic_bytes, int dev, std::atomic<int>* cache, size_t& ctas) {
-    int n = cache[dev].load(std::memory_order_relaxed);
-    if (n == 0) {
-        cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic_bytes);
-        if (err != cudaSuccess) return err;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, dynamic_bytes);
-        if (err != cudaSuccess) return err;
-        if (n < 1) n = 1;
-        cache[dev].store(n, std::memory_order_relaxed);
-    }
-    ctas = (size_t)n;
-    return cudaSuccess;
-}
-
 template <int DT, int B, int FMT, int G>
 static cudaError_t launch_brute_size(const QuantArgs& a, int slices, cudaStream_t stream) {
     using S = BruteShape<B, G>;

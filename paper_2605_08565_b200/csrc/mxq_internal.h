@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace mxq {
 
 constexpr int kMaxDevices = 64;
@@ -70,6 +72,21 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned 
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+// Resident CTAs per SM of a kernel (first use asks; racing threads store the same value).
+inline cudaError_t resident_ctas(const void* kernel, size_t dynamic_bytes, int dev, std::atomic<int>* cache, size_t& ctas, int threads = 256) {
+    int n = cache[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+        cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic_bytes);
+        if (err != cudaSuccess) return err;
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, dynamic_bytes);
+        if (err != cudaSuccess) return err;
+        if (n < 1) n = 1;
+        cache[dev].store(n, std::memory_order_relaxed);
+    }
+    ctas = (size_t)n;
+    return cudaSuccess;
+}
+
 void count_launch();
 
 cudaError_t launch_quantize_f32(const QuantArgs& a, int B, int fmt, bool dual, cudaStream_t s);
