@@ -194,24 +194,45 @@ cudaError_t launch_histograms(const uint8_t* codes, const uint8_t* scales, size_
 
 // ------------------------------------------------------------------------------------------------
 // Segment MSE: out[s] = (sum of the block SSEs of segment s) / elems_per_segment.  One CTA per
-// segment (grid-stride over segments); thread t adds blocks t, t + 256, ... in order in binary64,
-// then a shared-memory halving tree: fixed shape, same bits on every run.
+// segment (grid-stride over segments), binary64 sums of a fixed shape: thread t adds the 16-byte pieces t, t + T, ... of the
+// segment's aligned part (and its share of what lies before and after it), then a shuffle tree per warp and the warps in
+// order: same bits on every run.  A long segment needs the bytes in flight of 1024 threads with four loads each (151 segments of
+// 50,000 blocks, 30 MB, with the launch 18 -> 15 us); many short ones are better off with four times the CTAs.
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_segment_mse(const float* sse, size_t n_segments, size_t blocks_per_segment,
-                                                          double elems_per_segment, double* out) {
-    __shared__ double sh[kThreads];
+template <int T>
+__global__ void __launch_bounds__(T) k_segment_mse(const float* sse, size_t n_segments, size_t blocks_per_segment,
+                                                   double elems_per_segment, double* out) {
+    __shared__ double sh[T / 32];
+    wait_for_prior_grid();
+    release_dependents();
     for (size_t seg = blockIdx.x; seg < n_segments; seg += gridDim.x) {
         const float* p = sse + seg * blocks_per_segment;
+        size_t head = ((16u - (unsigned)(reinterpret_cast<uintptr_t>(p) & 15u)) & 15u) / 4;
+        if (head > blocks_per_segment) head = blocks_per_segment;
+        const size_t n_vec = (blocks_per_segment - head) / 4;
+        const size_t tail = head + 4 * n_vec;
+        const float4* v = reinterpret_cast<const float4*>(p + head);
         double acc = 0.0;
-        for (size_t i = threadIdx.x; i < blocks_per_segment; i += kThreads) acc = __dadd_rn(acc, (double)p[i]);
-        sh[threadIdx.x] = acc;
-        __syncthreads();
+        if (threadIdx.x < head) acc = (double)p[threadIdx.x];
+        if (threadIdx.x < blocks_per_segment - tail) acc = __dadd_rn(acc, (double)p[tail + threadIdx.x]);
+        for (size_t i = threadIdx.x; i < n_vec; i += 4 * T) {
+            float4 w[4];
 #pragma unroll
-        for (int w = kThreads / 2; w > 0; w >>= 1) {
-            if (threadIdx.x < w) sh[threadIdx.x] = __dadd_rn(sh[threadIdx.x], sh[threadIdx.x + w]);
-            __syncthreads();
+            for (int u = 0; u < 4; ++u) w[u] = i + u * T < n_vec ? v[i + u * T] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                acc = __dadd_rn(acc, __dadd_rn(__dadd_rn((double)w[u].x, (double)w[u].y), __dadd_rn((double)w[u].z, (double)w[u].w)));
         }
-        if (threadIdx.x == 0) out[seg] = __ddiv_rn(sh[0], elems_per_segment);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc = __dadd_rn(acc, __shfl_down_sync(0xFFFFFFFFu, acc, o));
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            double t = threadIdx.x < T / 32 ? sh[threadIdx.x] : 0.0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t = __dadd_rn(t, __shfl_down_sync(0xFFFFFFFFu, t, o));
+            if (threadIdx.x == 0) out[seg] = __ddiv_rn(t, elems_per_segment);
+        }
         __syncthreads();
     }
 }
@@ -221,11 +242,13 @@ cudaError_t launch_segment_mse(const float* sse, size_t n_segments, size_t block
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
-    const size_t cap = (size_t)sm_count(dev) * 8;
+    const bool wide = blocks_per_segment >= 4096;
+    const size_t cap = (size_t)sm_count(dev) * (wide ? 2 : 8);
     const unsigned grid = (unsigned)(n_segments < cap ? n_segments : cap);
-    k_segment_mse<<<grid, kThreads, 0, s>>>(sse, n_segments, blocks_per_segment, (double)elems_per_segment, out);
+    if (wide) err = launch_pdl(k_segment_mse<1024>, grid, 1024u, 0, s, sse, n_segments, blocks_per_segment, (double)elems_per_segment, out);
+    else err = launch_pdl(k_segment_mse<256>, grid, 256u, 0, s, sse, n_segments, blocks_per_segment, (double)elems_per_segment, out);
     count_launch();
-    return cudaGetLastError();
+    return err;
 }
 
 // ------------------------------------------------------------------------------------------------
