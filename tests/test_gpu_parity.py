@@ -167,6 +167,22 @@ def test_full_sweep_around_the_limits_of_its_split(B, fmt, g):
         check_parity(x.to(torch.bfloat16 if k % 2 else torch.float32).contiguous(), B, fmt, mxq.MXQ_BRUTE, g)
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_tensor_amax_around_the_limit_of_one_cta(dtype):
+    """One launch of one CTA up to 256 KB, two kernels beyond: the largest magnitude at the first, the last and a middle
+    element, ragged ends, and a tensor of zeros (tensor scale 1)."""
+    limit = 256 * 1024 // (4 if dtype == torch.float32 else 2)
+    for n in (1, 7, 8, 4097, 16385, limit - 1, limit, limit + 1):
+        for at in {0, n // 2, n - 1}:
+            x = inputs.normal(n, 3 + n % 7, 0.1, torch.float32).to(dtype)
+            x[at] = -7.25
+            amax, g = (torch.full((1,), -1.0, device="cuda") for _ in range(2))
+            mxq.mxq_tensor_amax(x.cuda(), n, amax, g)
+            assert float(amax.cpu()) == 7.25 and float(g.cpu()) == np.float32(7.25) / np.float32(2688.0)
+    mxq.mxq_tensor_amax(torch.zeros(100, dtype=dtype, device="cuda"), 100, amax, g)
+    assert float(amax.cpu()) == 0.0 and float(g.cpu()) == 1.0
+
+
 def test_option_calls_reject_bad_arguments():
     with pytest.raises(mxq.MxqError):
         mxq.mxq_set_option(99, 1)
