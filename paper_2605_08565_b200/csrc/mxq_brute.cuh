@@ -993,7 +993,7 @@ static cudaError_t launch_brute_size(const QuantArgs& a, int slices, cudaStream_
     // Under a tensor scale the codes of UE4M3 reach from the top of the tensor down by 17 binades only: next to none lies in
     // the cheap stretches of search_group(), and the kernel without them is faster by the registers they take (16.8 M fp32
     // Laplace elements, with -> without, us: B = 2 534 -> 499, 4 458 -> 440, 8 393 -> 371, 16 385 -> 367, 64 427 -> 420; B = 32
-    // 385 -> 391).  The other formats and unscaled UE4M3 gain (start -> with, B = 16): UE5M3 684 -> 543, UE8M0 660 ->
+    // 385 -> 391).  The other formats and unscaled UE4M3 gain (all codes in full -> with, B = 16): UE5M3 684 -> 543, UE8M0 660 ->
     // 133, unscaled UE4M3 330 -> 273.
     constexpr bool kHasPlain = FMT == kUE4M3 && B != 32;
     const bool plain = kHasPlain && slices == 1 && (a.d_global_scale != nullptr || a.global_scale != 1.0f);
