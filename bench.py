@@ -519,16 +519,18 @@ def weight_set_report(torch, mxq, device, peaks, layers: int = 8):
 def search_lane_ops(torch, x, B: int, fmt: int) -> float:
     """Lane-ops that a full sweep of x under the tensor scale amax / 2688 performs: 4 per (element, code), except the codes under
     which every element of a warp's 32 groups saturates (2: residual and square) and those that leave or make
-    every element's error the element itself (one shared sum of squares, 1 per element).  UE4M3 evaluates every code in full."""
+    every element's error the element itself (one shared sum of squares, 1 per element).  UE4M3 evaluates every code in full
+    except at B = 32."""
     n = x.numel()
-    if fmt == UE4M3:
+    if fmt == UE4M3 and B != 32:
         return n * N_CODES[fmt] * 4.0
     c = torch.arange(N_CODES[fmt], device=x.device, dtype=torch.float64)
     if fmt == UE8M0:
         S = torch.exp2(c - 127)
     else:
         e, m = torch.div(c, 8, rounding_mode="floor"), c % 8
-        S = torch.where(e == 0, m * 2.0 ** -17, (1 + m / 8) * torch.exp2(e - 15))
+        bias = 7 if fmt == UE4M3 else 15
+        S = torch.where(e == 0, m * 2.0 ** (-2 - bias), (1 + m / 8) * torch.exp2(e - bias))
     span = 32 * (B if B >= 32 else (16 if B <= 4 else 32))
     inf = torch.tensor(float("inf"), device=x.device)
     ops, amax = 0.0, float(x.abs().max())
