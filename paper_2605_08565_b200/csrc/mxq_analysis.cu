@@ -193,35 +193,48 @@ cudaError_t launch_histograms(const uint8_t* codes, const uint8_t* scales, size_
 }
 
 // ------------------------------------------------------------------------------------------------
-// Segment MSE: out[s] = (sum of the block SSEs of segment s) / elems_per_segment.  One CTA per
-// segment (grid-stride over segments), binary64 sums of a fixed shape: thread t adds the 16-byte pieces t, t + T, ... of the
-// segment's aligned part (and its share of what lies before and after it), then a shuffle tree per warp and the warps in
-// order: same bits on every run.  A long segment needs the bytes in flight of 1024 threads with four loads each (151 segments of
-// 50,000 blocks, 30 MB, with the launch 18 -> 15 us); many short ones are better off with four times the CTAs.
+// Segment MSE: out[s] = (sum of the block SSEs of segment s) / elems_per_segment.  One CTA of T threads per
+// segment (grid-stride over segments), binary64 sums whose shape depends on the length of the segment alone: thread t adds
+// elements t, t + T, ..., four at a time as (a + b) + (c + d) with zeros past the end, then a shuffle tree per warp and one over
+// the warps.  The same values give the same bits wherever the segment lies.  Single floats are read, not vectors of four: a warp's
+// reads are whole lines at any alignment, and the conversions and additions to binary64 cost more than the wider loads save.
+// A long segment needs the bytes in flight of 1024 threads (151 segments of 50,000 blocks, 30 MB, with the launch, T = 256 / 1024: 7.3 /
+// 6.1 us); short ones are better off with four times the CTAs (10,000 segments of 64 blocks 9.8 / 37 us).
 // ------------------------------------------------------------------------------------------------
 template <int T>
-__global__ void __launch_bounds__(T) k_segment_mse(const float* sse, size_t n_segments, size_t blocks_per_segment,
+__global__ void __launch_bounds__(T, 2048 / T) k_segment_mse(const float* sse, size_t n_segments, size_t blocks_per_segment,
                                                    double elems_per_segment, double* out) {
     __shared__ double sh[T / 32];
     wait_for_prior_grid();
     release_dependents();
     for (size_t seg = blockIdx.x; seg < n_segments; seg += gridDim.x) {
         const float* p = sse + seg * blocks_per_segment;
-        size_t head = ((16u - (unsigned)(reinterpret_cast<uintptr_t>(p) & 15u)) & 15u) / 4;
-        if (head > blocks_per_segment) head = blocks_per_segment;
-        const size_t n_vec = (blocks_per_segment - head) / 4;
-        const size_t tail = head + 4 * n_vec;
-        const float4* v = reinterpret_cast<const float4*>(p + head);
         double acc = 0.0;
-        if (threadIdx.x < head) acc = (double)p[threadIdx.x];
-        if (threadIdx.x < blocks_per_segment - tail) acc = __dadd_rn(acc, (double)p[tail + threadIdx.x]);
-        for (size_t i = threadIdx.x; i < n_vec; i += 4 * T) {
-            float4 w[4];
+        auto add_four = [&](const float* w) {
+            acc = __dadd_rn(acc, __dadd_rn(__dadd_rn((double)w[0], (double)w[1]), __dadd_rn((double)w[2], (double)w[3])));
+        };
+        size_t i = threadIdx.x;
+        for (; i + 15 * T < blocks_per_segment; i += 16 * T) {
+            float w[16];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) w[u] = i + u * T < n_vec ? v[i + u * T] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (int u = 0; u < 16; ++u) w[u] = p[i + u * T];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                acc = __dadd_rn(acc, __dadd_rn(__dadd_rn((double)w[u].x, (double)w[u].y), __dadd_rn((double)w[u].z, (double)w[u].w)));
+            for (int u = 0; u < 16; u += 4) add_four(w + u);
+        }
+        const int rest = (int)(blocks_per_segment - (i - threadIdx.x));   // negative or below 16 T
+        const float* const q = p + (i - threadIdx.x);
+        if (rest > 4 * T) {
+            float w[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) w[u] = (int)threadIdx.x + u * T < rest ? q[u * T + threadIdx.x] : 0.0f;
+#pragma unroll
+            for (int u = 0; u < 16; u += 4)
+                if (u * T < rest) add_four(w + u);
+        } else if (rest > 0) {
+            float w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) w[u] = (int)threadIdx.x + u * T < rest ? q[u * T + threadIdx.x] : 0.0f;
+            add_four(w);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc = __dadd_rn(acc, __shfl_down_sync(0xFFFFFFFFu, acc, o));
@@ -242,11 +255,11 @@ cudaError_t launch_segment_mse(const float* sse, size_t n_segments, size_t block
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
-    const bool wide = blocks_per_segment >= 4096;
-    const size_t cap = (size_t)sm_count(dev) * (wide ? 2 : 8);
+    const int threads = blocks_per_segment < 4096 ? 256 : 1024;
+    const size_t cap = (size_t)sm_count(dev) * (2048 / threads);
     const unsigned grid = (unsigned)(n_segments < cap ? n_segments : cap);
-    if (wide) err = launch_pdl(k_segment_mse<1024>, grid, 1024u, 0, s, sse, n_segments, blocks_per_segment, (double)elems_per_segment, out);
-    else err = launch_pdl(k_segment_mse<256>, grid, 256u, 0, s, sse, n_segments, blocks_per_segment, (double)elems_per_segment, out);
+    auto* const kernel = threads == 256 ? k_segment_mse<256> : k_segment_mse<1024>;
+    err = launch_pdl(kernel, grid, (unsigned)threads, 0, s, sse, n_segments, blocks_per_segment, (double)elems_per_segment, out);
     count_launch();
     return err;
 }

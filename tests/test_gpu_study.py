@@ -51,6 +51,27 @@ def test_segment_mse_matches_oracle():
         assert torch.equal(out, out2)
 
 
+@pytest.mark.parametrize("per", [3, 50, 1001, 4095, 4097, 16383, 16385, 20002, 70001, 131073])
+def test_segment_mse_does_not_depend_on_where_a_segment_lies(per):
+    """Equal segments give equal bits at every offset from a 16-byte boundary, alone and as segments of one call; lengths on
+    either side of a full trip of the narrow kernel (4096) and of those of longer ones."""
+    rng = np.random.default_rng(per)
+    seg = (rng.random(per) * np.exp2(rng.integers(-30, 4, per))).astype(np.float32)
+    want = orc.segment_mse(seg, per, per * 8)[0]
+    d = torch.from_numpy(np.tile(seg, 5)).cuda()
+    out = torch.empty(5, dtype=torch.float64, device="cuda")
+    mxq.mxq_segment_mse(d, 5 * per, per, per * 8, out)
+    bits = set(out.cpu().numpy().view(np.uint64).tolist())
+    for offset in range(4):
+        buf = torch.full((per + 8,), 1e30, dtype=torch.float32, device="cuda")
+        buf[offset:offset + per] = d[:per]
+        one = torch.empty(1, dtype=torch.float64, device="cuda")
+        mxq.mxq_segment_mse(buf[offset:offset + per], per, per, per * 8, one)
+        bits.add(int(one.cpu().numpy().view(np.uint64)[0]))
+    assert len(bits) == 1
+    assert abs(float(out[0]) - want) <= 1e-12 * want
+
+
 def test_reduced_numerical_study_against_oracle():
     """16 sigmas x 2000 blocks, all five recipes, block sizes 4 and 16: every MSE and clipping-MSE
     point against the oracle on the very same samples."""
