@@ -198,8 +198,10 @@ cudaError_t launch_histograms(const uint8_t* codes, const uint8_t* scales, size_
 // elements t, t + T, ..., four at a time as (a + b) + (c + d) with zeros past the end, then a shuffle tree per warp and one over
 // the warps.  The same values give the same bits wherever the segment lies.  Single floats are read, not vectors of four: a warp's
 // reads are whole lines at any alignment, and the conversions and additions to binary64 cost more than the wider loads save.
-// A long segment needs the bytes in flight of 1024 threads (151 segments of 50,000 blocks, 30 MB, with the launch, T = 256 / 1024: 7.3 /
-// 6.1 us); short ones are better off with four times the CTAs (10,000 segments of 64 blocks 9.8 / 37 us).
+// What a segment needs is loads in flight, sixteen a thread at full occupancy (32 registers): short segments are better off
+// with many CTAs, long ones with wide ones.  151 segments, us with the launch, T = 256 / 512 / 1024: 1000 blocks 1.6 / 1.6 / 2.2, 8000
+// 2.4 / 2.2 / 2.9, 20,000 3.8 / 3.5 / 3.5, 50,000 7.3 / 6.0 / 6.1, 400,000 124 / 69 / 50; 10,000 segments of 64 9.8 / 19 / 37, 500 of 12,000
+// 4.0 / 4.4 / 5.0.
 // ------------------------------------------------------------------------------------------------
 template <int T>
 __global__ void __launch_bounds__(T, 2048 / T) k_segment_mse(const float* sse, size_t n_segments, size_t blocks_per_segment,
@@ -255,10 +257,10 @@ cudaError_t launch_segment_mse(const float* sse, size_t n_segments, size_t block
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
-    const int threads = blocks_per_segment < 4096 ? 256 : 1024;
+    const int threads = blocks_per_segment < 16384 ? 256 : blocks_per_segment < 131072 ? 512 : 1024;
     const size_t cap = (size_t)sm_count(dev) * (2048 / threads);
     const unsigned grid = (unsigned)(n_segments < cap ? n_segments : cap);
-    auto* const kernel = threads == 256 ? k_segment_mse<256> : k_segment_mse<1024>;
+    auto* const kernel = threads == 256 ? k_segment_mse<256> : threads == 512 ? k_segment_mse<512> : k_segment_mse<1024>;
     err = launch_pdl(kernel, grid, (unsigned)threads, 0, s, sse, n_segments, blocks_per_segment, (double)elems_per_segment, out);
     count_launch();
     return err;

@@ -54,7 +54,7 @@ def test_segment_mse_matches_oracle():
 @pytest.mark.parametrize("per", [3, 50, 1001, 4095, 4097, 16383, 16385, 20002, 70001, 131073])
 def test_segment_mse_does_not_depend_on_where_a_segment_lies(per):
     """Equal segments give equal bits at every offset from a 16-byte boundary, alone and as segments of one call; lengths on
-    either side of a full trip of the narrow kernel (4096) and of those of longer ones."""
+    either side of a full trip of the narrow kernel (4096) and of the limits between the three."""
     rng = np.random.default_rng(per)
     seg = (rng.random(per) * np.exp2(rng.integers(-30, 4, per))).astype(np.float32)
     want = orc.segment_mse(seg, per, per * 8)[0]
