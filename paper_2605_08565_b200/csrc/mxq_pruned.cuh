@@ -103,7 +103,7 @@ __device__ __forceinline__ float element(const float2 (&v)[pruned_values(B)], in
 // (-D, RN(1 / D)); holds for every decode scale in [2^-60, 2^60].  kModeHalf: -D is exact in f16 (and for bf16 input D
 // has at most four significant bits, so that the quotient is one multiply rounded toward zero): z holds f16(-D).
 // kModeChecked (bf16): the one-multiply quotient with the reciprocal that build_quant_tables() checked, which z holds.
-// kModeSlow: every code, with IEEE division.
+// kModeSlow: search_by_division().
 enum { kModeExact = 0, kModeHalf = 1, kModeChecked = 2, kModeSlow = 3 };
 struct PrunedTables {
     float nD[256], R[256], z[256];
@@ -213,6 +213,73 @@ __device__ __forceinline__ unsigned long long shl64(unsigned long long x, int n)
     return r;
 }
 
+// A block outside the ranges of the shortcuts, with IEEE division: the best (SSE bits, code) among codes first .. n_codes - 1.
+// decode(c): the decode scale, nondecreasing in c; pair(i): elements i and i + 1; a: the largest magnitude.  Codes are taken upwards from
+// the first with 6 D >= a, then downwards from there, until
+//   upwards     D >= 4 a: this and every larger D has the SSE of the all-zero quantization (ties go to the smaller code); or the
+//               elements that D sends to zero (4 |v| <= D) alone cost more than the best SSE so far: they do under every larger D;
+//   downwards   what the saturated elements leave, fl(|v| - 6 D) each, alone costs more: it does so under every smaller D.
+// The sums compared are taken in the order and arithmetic of the SSE.  Magnitudes of 1e-20 under their tensor scale, 4.2 M elements:
+// every code 1108 us for UE4M3 at B = 16 (fp32) and 1261 for UE5M3 at B = 2 (bf16), here 191 and 332.
+template <int B, int UNROLL, typename Decode, typename Pair>
+__device__ __forceinline__ unsigned long long search_by_division(Decode decode, Pair pair, float a, int first, int n_codes) {
+    int c0 = first, end = n_codes;
+    while (c0 < end) {
+        const int mid = (c0 + end) >> 1;
+        if (__fmul_rn(6.0f, decode(mid)) < a) c0 = mid + 1;
+        else end = mid;
+    }
+    unsigned long long best = sse_key(__uint_as_float(0xFFFFFFFFu), first);
+    bool up = true;
+    int c = c0;
+    while (up || c >= first) {
+        const float D = c < n_codes ? decode(c) : __uint_as_float(0x7F800000u);
+        if (!(fabsf(D) <= 3.402823466e38f)) {   // overflowed: not usable, nor is any larger code
+            c = up ? c0 - 1 : c - 1;
+            up = false;
+            continue;
+        }
+        float s = 0.0f, z = 0.0f;
+#pragma unroll UNROLL
+        for (int i = 0; i < B; i += 2) {
+            const float2 v = pair(i);
+            const float2 q = round_e2m1x2(quotient_general(v.x, D), quotient_general(v.y, D));
+            const float e0 = __fmaf_rn(-q.x, D, v.x), e1 = __fmaf_rn(-q.y, D, v.y);
+            s = __fmaf_rn(e0, e0, s);
+            s = __fmaf_rn(e1, e1, s);
+            const float a0 = fabsf(v.x), a1 = fabsf(v.y);
+            const float z0 = up ? (__fmul_rn(4.0f, a0) <= D ? a0 : 0.0f) : fmaxf(__fmaf_rn(-6.0f, D, a0), 0.0f);
+            const float z1 = up ? (__fmul_rn(4.0f, a1) <= D ? a1 : 0.0f) : fmaxf(__fmaf_rn(-6.0f, D, a1), 0.0f);
+            z = __fmaf_rn(z0, z0, z);
+            z = __fmaf_rn(z1, z1, z);
+        }
+        best = min(best, sse_key(s, c));
+        const bool rest_is_out = __float_as_uint(z) > (uint32_t)(best >> 32) || (up && D >= __fmul_rn(4.0f, a));
+        if (!rest_is_out) {
+            c += up ? 1 : -1;
+        } else if (up) {
+            up = false;
+            c = c0 - 1;
+        } else {
+            break;
+        }
+    }
+    return best;
+}
+
+// The same for block b of a tile; out of line, to leave the registers of the search proper alone.
+template <int B>
+__device__ __noinline__ unsigned long long search_tile_block(const float* tile, int b, const float* nD, int first, int n_codes) {
+    auto pair = [&](int i) {
+        if constexpr (B == 2) return *reinterpret_cast<const float2*>(tile + b * 2);
+        else return *reinterpret_cast<const float2*>(tile + PrunedTile<B>::piece(b, i / 4) + (i & 3));
+    };
+    float a = 0.0f;
+#pragma unroll 1
+    for (int i = 0; i < B; i += 2) a = fmaxf(a, fmaxf(fabsf(pair(i).x), fabsf(pair(i).y)));
+    return search_by_division<B, 1>([&](int c) { return -nD[c]; }, pair, a, first, n_codes);
+}
+
 // The first n blocks of a unit of eight elements (B = 2 or 4), from block blk on.
 template <int B, int UB>
 __device__ __forceinline__ void store_whole_blocks(const QuantArgs& p, size_t blk, size_t n, uint32_t packed, uint32_t sc, const uint32_t (&sw)[UB]) {
@@ -273,9 +340,12 @@ __global__ void __launch_bounds__(kThreads, pruned_min_ctas(B)) k_pruned(QuantAr
     __syncthreads();
     const int fast_mode = checked ? kModeChecked : kModeHalf;
     const int fast_end = checked ? NC : (DT == kF32 ? short_end : first_bad);   // codes below it may be evaluated in fast_mode
-    // every nonzero code of both formats then has its decode scale in [2^-60, 2^60]
+    // The shortcuts need decode scales in [2^-60, 2^60].  For g within kMaxG of 1 every nonzero code has one.  Beyond, the codes from a / 12
+    // to 4 a do (a within [2^-55, 2^57], codes are at most a factor of two apart), which are all that a block with r < a / 2 looks at
+    // (magnitudes of 1e-12 under their tensor scale, UE5M3, B = 8, 4.2 M elements: 2166 -> 36 us).
     constexpr float kMaxG = FMT == kUE4M3 ? 2.251799813685248e15f /* 2^51 */ : 8.796093022208e12f /* 2^43 */;
-    const bool g_ok = g >= 1.0f / kMaxG && g <= kMaxG;
+    const bool g_ok = g >= kFastMin && g <= kFastMax;
+    const bool all_in_range = g >= 1.0f / kMaxG && g <= kMaxG;
     const float Rg = g_ok ? __frcp_rn(g) : 1.0f;
     // fast_mode for the blocks all of whose codes, up to the first with D >= 4 a, lie below fast_end
     const float fast_below = fast_end == NC ? 3.402823466e38f : (fast_end >= 8 ? __fmul_rn(-0.25f, tab.nD[fast_end - 1]) : 0.0f);
@@ -336,7 +406,7 @@ __global__ void __launch_bounds__(kThreads, pruned_min_ctas(B)) k_pruned(QuantAr
             int base = 0, mode = kModeExact;
             if (a == 0.0f) {
                 best = sse_key(0.0f, first);   // every code reproduces the zeros
-            } else if (!(g_ok && a <= kFastMax && a >= 6.938893903907228e-18f /* 2^-57 */)) {
+            } else if (!(g_ok && a <= 1.44115188075855872e17f /* 2^57 */ && a >= 2.77555756156289135e-17f /* 2^-55 */)) {
                 mode = kModeSlow;
             } else {
                 const float u = __fmul_rn(a, Rg);
@@ -358,6 +428,7 @@ __global__ void __launch_bounds__(kThreads, pruned_min_ctas(B)) k_pruned(QuantAr
                 float r = __fmaf_rn(sqrt_approx(__uint_as_float(ubits)), 1.0009765625f, 2.168404344971009e-19f /* 2^-62 */);
                 // zero rule; with r < a / 2 the all-zero quantization (at least a^2) cannot be the best
                 if (!(r < 0.5f * a)) {
+                    if (!all_in_range) mode = kModeSlow;
                     const int zc = first == 0 ? 0 : floor_code<FMT>(__fmul_rn(4.0f * kUp, u)) + 1;
                     if (zc < NC) best = min(best, sse_key(sum_of_squares([](float v) { return v; }), zc));
                     ubits = (uint32_t)(best >> 32);
@@ -481,25 +552,7 @@ __global__ void __launch_bounds__(kThreads, pruned_min_ctas(B)) k_pruned(QuantAr
             const int b = perm[at];
             const int mode = info[b] >> 8;
             if (mode == kModeSlow) {
-                unsigned long long best = sse_key(__uint_as_float(0xFFFFFFFFu), first);
-                for (int c = first; c < NC; ++c) {
-                    const float D = -tab.nD[c];
-                    if (!(fabsf(D) <= 3.402823466e38f)) continue;   // decode scale overflowed: not usable
-                    float s = 0.0f;
-#pragma unroll 1
-                    for (int from = 0; from < B; from += 2) {
-                        float2 v2[1];
-                        if constexpr (B == 2) v2[0] = *reinterpret_cast<const float2*>(tile + b * 2);
-                        else v2[0] = *reinterpret_cast<const float2*>(tile + Tile::piece(b, from / 4) + (from & 3));
-                        const float2 q = round_e2m1x2(quotient_general(v2[0].x, D), quotient_general(v2[0].y, D));
-                        const float e0 = __fmaf_rn(-q.x, D, v2[0].x);
-                        s = __fmaf_rn(e0, e0, s);
-                        const float e1 = __fmaf_rn(-q.y, D, v2[0].y);
-                        s = __fmaf_rn(e1, e1, s);
-                    }
-                    best = min(best, sse_key(s, c));
-                }
-                key[b] = best;
+                key[b] = search_tile_block<B>(tile, b, tab.nD, first, NC);
                 continue;
             }
             const unsigned long long m64 = mask[b];
@@ -653,25 +706,9 @@ __device__ __forceinline__ unsigned long long pow2_search(const float2 (&v2)[B /
 #pragma unroll
     for (int i = 0; i < B / 2; ++i) a = fmaxf(a, fmaxf(fabsf(v2[i].x), fabsf(v2[i].y)));
     fast = g_ok && a <= 1.44115188075855872e17f /* 2^57 */ && a >= 2.77555756156289135e-17f /* 2^-55 */;
-    unsigned long long best = sse_key(__uint_as_float(0xFFFFFFFFu), 0);
     if (a == 0.0f) return sse_key(0.0f, 0);   // every code reproduces the zeros
-    if (!fast) {
-        for (int c = 0; c < num_codes(kUE8M0); ++c) {
-            const float D = __fmul_rn(scale_value(kUE8M0, c), g);
-            if (!(fabsf(D) <= 3.402823466e38f)) continue;   // decode scale overflowed: not usable
-            float s = 0.0f;
-#pragma unroll
-            for (int i = 0; i < B / 2; ++i) {
-                const float2 q = round_e2m1x2(quotient_general(v2[i].x, D), quotient_general(v2[i].y, D));
-                const float e0 = __fmaf_rn(-q.x, D, v2[i].x);
-                s = __fmaf_rn(e0, e0, s);
-                const float e1 = __fmaf_rn(-q.y, D, v2[i].y);
-                s = __fmaf_rn(e1, e1, s);
-            }
-            best = min(best, sse_key(s, c));
-        }
-        return best;
-    }
+    if (!fast) return search_by_division<B, B / 2>([g](int c) { return __fmul_rn(scale_value(kUE8M0, c), g); }, [&](int i) { return v2[i / 2]; }, a, 0, num_codes(kUE8M0));
+    unsigned long long best = sse_key(__uint_as_float(0xFFFFFFFFu), 0);
     // a / g lies within [2^-98, 2^100]: every code below is far from either end of the format, and every D and 1 / D
     // within [2^-60, 2^60]
     const float u = __fmul_rn(a, Rg);

@@ -151,6 +151,26 @@ def test_pruned_sweep_at_the_edges_of_its_bounds(dtype, B, fmt):
         mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 0)
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B", BLOCKS)
+@pytest.mark.parametrize("fmt", FMTS)
+def test_searches_of_tiny_and_huge_tensors_under_their_tensor_scale(dtype, B, fmt, sweep_mode):
+    """Gradient-like magnitudes and smaller, down to where squares and elements are denormal, and large ones up to where
+    squares overflow: the tensor scale leaves the range of every shortcut while the codes stay ordinary."""
+    for k in (-34, -43, -52, -66, -90, -126, -140, 44, 62, 90, 118):
+        x = inputs.student_t(261 * B, 4, 0.3, 900 + B - k, torch.float32) * 2.0 ** k
+        x[3 * B:5 * B] = 0.0
+        x[7 * B:8 * B] *= 2.0 ** -8
+        x = x.clamp(-2.0 ** 124, 2.0 ** 124).to(dtype).contiguous()
+        g = max(float(np.float32(x.float().abs().max()) / np.float32(2688.0)), 2.0 ** -149)
+        recipe = mxq.MXQ_BRUTE_PZ if k % 4 else mxq.MXQ_BRUTE
+        got = gpu_quantize(x, B, fmt, recipe, g)
+        want = orc.quantize(inputs.to_numpy_bits(x), B, fmt, recipe, g, threads=8)
+        for have, should in zip(got, want):     # codes, scale bytes, block SSE (infinite where squares overflow)
+            bad = np.flatnonzero(have.view(np.uint8) != should.view(np.uint8))
+            assert bad.size == 0, (k, bad[:8])
+
+
 @pytest.mark.parametrize("B, fmt, g", [(2, mxq.MXQ_SF_UE4M3, 0.0131), (4, mxq.MXQ_SF_UE8M0, 0.0131), (8, mxq.MXQ_SF_UE4M3, 0.0131), (16, mxq.MXQ_SF_UE5M3, 1.0), (32, mxq.MXQ_SF_UE8M0, 1.0),
                                        (64, mxq.MXQ_SF_UE4M3, 1.0)])
 def test_full_sweep_around_the_limits_of_its_split(B, fmt, g):
