@@ -4,6 +4,7 @@
 // numerical study per segment).  None of them is on the bandwidth-critical path; they are written
 // for exactness and determinism first.
 #include <atomic>
+#include <type_traits>
 
 #include "mxq_device.cuh"
 #include "mxq_internal.h"
@@ -20,7 +21,8 @@ namespace mxq {
 // rounds to 6, so fl32(v / D) > 6  <=>  v / D > 6 + 2^-22  <=>  |v| - 6 D > 2^-22 D.  The difference is formed by one FMA: near
 // the limit it is a multiple of 2^(e - 22) below 2^(e - 20), D in [2^e, 2^(e+1)), and therefore exact, as is 2^-22 D; away
 // from the limit its rounding cannot change the outcome.  It is also the residual.  Bound by the reads of x: fp32, B = 8,
-// 60.4 M elements (279 MB) 62 -> 53 us, B = 4 72 -> 58.
+// 60.4 M elements (279 MB) 62 -> 53 us, B = 4 72 -> 58.  The last block of a thread goes alone: a second load that is not needed
+// (the tensor's last block, for every thread of a small tensor) cost bf16, B = 2 1.05 -> 1.28 us at 4096 elements.
 // ------------------------------------------------------------------------------------------------
 template <int B>
 __device__ __forceinline__ float clip_sse(const float (&v)[B], int c, int fmt, float gs) {
@@ -54,21 +56,24 @@ __global__ void __launch_bounds__(kThreads) k_block_clip_sse(const void* x, size
     wait_for_prior_grid();
     release_dependents();
     const float gs = d_g ? *d_g : g;
-    constexpr int U = B <= 16 ? 2 : 1;
     const size_t stride = (size_t)gridDim.x * kThreads;
-    for (size_t b = (size_t)blockIdx.x * kThreads + threadIdx.x; b < n_blocks; b += U * stride) {
+    auto do_blocks = [&](auto count, size_t b) {   // blocks b, b + stride, ...: all loads first
+        constexpr int U = decltype(count)::value;
         float v[U][B];
         int c[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const size_t bu = u == 0 ? b : min(b + u * stride, n_blocks - 1);
-            load_elems<DT, B>(x, bu * B, v[u]);      // vector loads: a block is 4 .. 256 contiguous bytes
-            c[u] = scales[bu];
+            load_elems<DT, B>(x, (b + u * stride) * B, v[u]);      // vector loads: a block is 4 .. 256 contiguous bytes
+            c[u] = scales[b + u * stride];
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (b + u * stride < n_blocks) out[b + u * stride] = clip_sse<B>(v[u], c[u], fmt, gs);
+        for (int u = 0; u < U; ++u) out[b + u * stride] = clip_sse<B>(v[u], c[u], fmt, gs);
+    };
+    size_t b = (size_t)blockIdx.x * kThreads + threadIdx.x;
+    if constexpr (B <= 16) {
+        for (; b + stride < n_blocks; b += 2 * stride) do_blocks(std::integral_constant<int, 2>{}, b);
     }
+    for (; b < n_blocks; b += stride) do_blocks(std::integral_constant<int, 1>{}, b);
 }
 
 template <int DT>

@@ -51,6 +51,49 @@ def test_segment_mse_matches_oracle():
         assert torch.equal(out, out2)
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B", [2, 4, 8, 16, 32])
+def test_clip_sse_of_more_blocks_than_threads(dtype, B):
+    """More blocks than the grid has threads, and not a multiple: a thread's second block (in flight with the first for
+    B <= 16), its third, and none at all for the last threads."""
+    threads = 8 * torch.cuda.get_device_properties(0).multi_processor_count * 256
+    nb = 2 * threads + threads // 3 + 17
+    n = nb * B
+    x = (inputs.student_t(n, 4, 0.05, 50 + B, torch.float32, "cuda") * 3.0).to(dtype)
+    scales = torch.randint(0, 127, (nb,), dtype=torch.uint8, device="cuda", generator=torch.Generator("cuda").manual_seed(B))
+    clip = torch.empty(nb, dtype=torch.float32, device="cuda")
+    for g in (1.0, 0.0131):
+        mxq.mxq_block_clip_sse(x, n, B, mxq.MXQ_SF_UE4M3, g, None, scales, clip)
+        want = orc.block_clip_sse(inputs.to_numpy_bits(x.cpu()), scales.cpu().numpy(), B, mxq.MXQ_SF_UE4M3, g)
+        assert np.array_equal(clip.cpu().numpy().view(np.uint32), want.view(np.uint32))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B", [2, 4, 8, 16, 32, 64])
+def test_clip_sse_next_to_the_clipping_limit(dtype, B):
+    """Elements at 6 D and on either side of it (the quotient that still rounds to 6 lies up to 2^-22 D beyond), for decode
+    scales of many significands, and for decode scales on either side of 2^-100 and 2^100."""
+    rng = np.random.default_rng(B)
+    cases = [(mxq.MXQ_SF_UE4M3, np.float32(g), np.arange(1, 127)) for g in np.exp2(rng.uniform(-40, 40, 12))]
+    cases += [(mxq.MXQ_SF_UE5M3, np.float32(1.0), np.arange(1, 255))]
+    for e in (np.float32(1.0), np.nextafter(np.float32(1.0), np.float32(0.0)), np.nextafter(np.float32(1.0), np.float32(2.0))):
+        cases += [(mxq.MXQ_SF_UE8M0, e, np.arange(20, 34)), (mxq.MXQ_SF_UE8M0, e, np.arange(220, 234))]
+    for fmt, g, codes in cases:
+        scales = np.resize(codes, 700).astype(np.uint8)
+        D = (np.array([orc.scale_value(fmt, int(c)) for c in scales], dtype=np.float32) * g).astype(np.float32)
+        six = (np.float32(6.0) * D).astype(np.float32)
+        if dtype == torch.float32:
+            bits = six.view(np.uint32)[:, None].astype(np.int64) + rng.integers(-4, 6, (700, B))
+        else:
+            bits = (six.view(np.uint32)[:, None].astype(np.int64) & ~0xFFFF) + 0x10000 * rng.integers(-1, 3, (700, B))
+        v = bits.astype(np.uint32).view(np.float32) * rng.choice(np.array([-1.0, 1.0], dtype=np.float32), (700, B))
+        x = torch.from_numpy(v.reshape(-1).copy()).to(dtype)
+        clip = torch.empty(700, dtype=torch.float32, device="cuda")
+        mxq.mxq_block_clip_sse(x.cuda(), 700 * B, B, fmt, float(g), None, torch.from_numpy(scales).cuda(), clip)
+        want = orc.block_clip_sse(inputs.to_numpy_bits(x), scales, B, fmt, float(g))
+        assert np.array_equal(clip.cpu().numpy().view(np.uint32), want.view(np.uint32)), (fmt, g)
+
+
 @pytest.mark.parametrize("per", [3, 50, 1001, 4095, 4097, 16383, 16385, 20002, 70001, 131073])
 def test_segment_mse_does_not_depend_on_where_a_segment_lies(per):
     """Equal segments give equal bits at every offset from a 16-byte boundary, alone and as segments of one call; lengths on
