@@ -94,6 +94,24 @@ def test_clip_sse_next_to_the_clipping_limit(dtype, B):
         assert np.array_equal(clip.cpu().numpy().view(np.uint32), want.view(np.uint32)), (fmt, g)
 
 
+@pytest.mark.parametrize("B, codes_at, scales_at", [(2, 0, 0), (8, 4, 1), (16, 12, 7)])
+def test_histograms_around_the_limit_of_one_cta_per_sm(B, codes_at, scales_at):
+    """Up to 24 loads of 16 bytes per thread one CTA per SM counts, beyond that three; buffers off the 16-byte boundary."""
+    limit = torch.cuda.get_device_properties(0).multi_processor_count * 512 * 16 * 24     # bytes of codes and scales
+    gen = torch.Generator("cuda").manual_seed(B)
+    for blocks in (limit // (B // 2 + 1), limit // (B // 2 + 1) + 1, 3 * 1000 + 1):
+        n = blocks * B
+        c = torch.randint(0, 256, (n // 2 + 16,), dtype=torch.uint8, device="cuda", generator=gen)[codes_at:codes_at + n // 2]
+        s = torch.randint(0, 256, (blocks + 16,), dtype=torch.uint8, device="cuda", generator=gen)[scales_at:scales_at + blocks]
+        s[:blocks // 3] = 77
+        ch = torch.zeros(16, dtype=torch.int64, device="cuda")
+        sh = torch.zeros(256, dtype=torch.int64, device="cuda")
+        mxq.mxq_histograms(c, s, n, B, ch, sh)
+        och, osh = orc.histograms(c.cpu().numpy(), s.cpu().numpy(), n, B)
+        assert np.array_equal(ch.cpu().numpy().astype(np.uint64), och)
+        assert np.array_equal(sh.cpu().numpy().astype(np.uint64), osh)
+
+
 @pytest.mark.parametrize("per", [3, 50, 1001, 4095, 4097, 16383, 16385, 20002, 70001, 131073])
 def test_segment_mse_does_not_depend_on_where_a_segment_lies(per):
     """Equal segments give equal bits at every offset from a 16-byte boundary, alone and as segments of one call; lengths on
