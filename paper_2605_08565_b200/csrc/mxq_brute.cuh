@@ -31,6 +31,7 @@
 #pragma once
 
 #include <atomic>
+#include <type_traits>
 
 #include "mxq_device.cuh"
 #include "mxq_internal.h"
@@ -382,10 +383,25 @@ __host__ __device__ constexpr int brute_group_elems(int B) { return B >= 32 ? B 
 
 constexpr int brute_min_ctas(int B) { return B <= 32 ? 2 : 1; }
 
-// The best (SSE bits, code) keys of a thread's blocks in shared memory, 32 lanes apart.
+// Where k_brute keeps the best (SSE bits, code) key of each of a thread's blocks: in registers, except at B = 32, B = 8 in groups of 32
+// and UE8M0 at B = 64, which pay for the registers (16.8 M fp32 elements, shared memory -> registers, us: unscaled UE4M3 of N(0, 300),
+// B = 2 476 -> 451, 64 349 -> 337, but 8 336 -> 343; UE5M3 under a tensor scale, B = 16 539 -> 532, 64 589 -> 578, but 32 527 -> 559; UE8M0,
+// B = 2 171 -> 168, but 64 144 -> 145).
+__host__ __device__ constexpr bool brute_keys_in_registers(int B, int G, int fmt) {
+    return B != 32 && !(B == 8 && G == 32) && !(B == 64 && fmt == kUE8M0);
+}
+
+// Keys in shared memory, 32 lanes apart.
 struct SharedBest {
     unsigned long long* p;
     __device__ __forceinline__ unsigned long long& operator[](int k) const { return p[32 * k]; }
+};
+
+// Keys in registers.
+template <int N>
+struct RegisterBest {
+    unsigned long long k[N];
+    __device__ __forceinline__ unsigned long long& operator[](int i) { return k[i]; }
 };
 
 // G: elements per thread.
@@ -491,9 +507,9 @@ __device__ __forceinline__ GroupRange take_magnitudes(float2 (&v2)[BruteShape<B,
 }
 
 // SSEs of all blocks of a thread when every element saturates, for the codes lo .. hi - 1: q = 6 and e = fma(6, -D, |v|).
-template <int B, int G>
+template <int B, int G, typename Best>
 __device__ __forceinline__ void search_saturated(const BruteTables& T, int lo, int hi, const float2 (&v2)[BruteShape<B, G>::NP],
-                                                 const SharedBest& best) {
+                                                 Best& best) {
     using S = BruteShape<B, G>;
     if (lo >= hi) return;
     uint32_t cbest[S::NBT];
@@ -538,8 +554,8 @@ __device__ __forceinline__ void search_saturated(const BruteTables& T, int lo, i
     for (int k = 0; k < S::NBT; ++k) merge_class_winner(best[k], cbest[k], ccode[k]);
 }
 
-// The SSE of every code on every block of the warp's threads; best[k] (shared memory: registers are what these kernels
-// are short of) receives the smallest of block k, ties to the smaller code.  Rg = RN(1 / g), or 0 for g beyond 2^+-60.
+// The SSE of every code on every block of the warp's threads; best[k] receives the smallest of block k, ties to the smaller
+// code.  Rg = RN(1 / g), or 0 for g beyond 2^+-60.
 // Called by whole warps; `live` lanes take part.  Slice `slice` of `slices` covers its share of the codes.
 //
 // Three stretches of the codes need less than the full evaluation, and are the same for the whole warp (decode scales rise
@@ -549,9 +565,9 @@ __device__ __forceinline__ void search_saturated(const BruteTables& T, int lo, i
 //                     smallest of these codes, which is how the full evaluation of each would end.
 //   D <= lo / 6       (no zero among the elements) every element saturates: the error is fl(|v| - 6 D), two packed FMAs
 //                     per pair of elements and code instead of quotient, rounding, widening and two FMAs.
-template <int B, int G, int FMT>
+template <int B, int G, int FMT, typename Best>
 __device__ __forceinline__ void search_group(const BruteTables& T, const float2 (&v2)[BruteShape<B, G>::NP], const GroupRange& gr, bool live,
-                                             float Rg, int first, int slice, int slices, const SharedBest& best) {
+                                             float Rg, int first, int slice, int slices, Best& best) {
     using S = BruteShape<B, G>;
     constexpr int NCLS = (FMT == kUE8M0) ? 1 : 8;
     constexpr int NC = num_codes(FMT);
@@ -839,7 +855,8 @@ template <int DT, int B, int G, int FMT>
 __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs p) {
     using S = BruteShape<B, G>;
     __shared__ BruteTables T;
-    __shared__ unsigned long long key[kThreads / 32][32 * S::NBT];   // per warp: best of block k of lane l at k * 32 + l
+    constexpr bool kKeysInRegisters = brute_keys_in_registers(B, G, FMT);
+    __shared__ unsigned long long key[kKeysInRegisters ? 1 : kThreads / 32][kKeysInRegisters ? 1 : 32 * S::NBT];   // per warp: block k of lane l at k * 32 + l
     wait_for_prior_grid();
     release_dependents();
     const float g = p.d_global_scale ? *p.d_global_scale : p.global_scale;
@@ -850,7 +867,10 @@ __global__ void __launch_bounds__(kThreads, brute_min_ctas(B)) k_brute(QuantArgs
     const size_t n_groups = (p.n_items + S::NBT - 1) / S::NBT;
     const size_t stride = (size_t)gridDim.x * kThreads;
     const int lane = threadIdx.x & 31;
-    const SharedBest best = {&key[threadIdx.x >> 5][lane]};
+    typename std::conditional<kKeysInRegisters, RegisterBest<S::NBT>, const SharedBest>::type best = [&] {
+        if constexpr (kKeysInRegisters) return RegisterBest<S::NBT>{};
+        else return SharedBest{&key[threadIdx.x >> 5][lane]};
+    }();
     double sse_sum = 0.0;                  // binary64 sum of the SSEs of this thread's blocks, in the order it stored them
     for (size_t wbase = first_set<B>(); wbase < n_groups; wbase += stride) {
         const size_t grp = wbase + lane;
@@ -993,8 +1013,10 @@ static cudaError_t launch_brute_size(const QuantArgs& a, int slices, cudaStream_
     // Under a tensor scale the codes of UE4M3 reach from the top of the tensor down by 17 binades only: next to none lies in
     // the cheap stretches of search_group(), and the kernel without them is faster by the registers they take (16.8 M fp32
     // Laplace elements, with -> without, us: B = 2 534 -> 499, 4 458 -> 440, 8 393 -> 371, 16 385 -> 367, 64 427 -> 420; B = 32
-    // 385 -> 391).  The other formats and unscaled UE4M3 gain (all codes in full -> with, B = 16): UE5M3 684 -> 543, UE8M0 660 ->
-    // 133, unscaled UE4M3 330 -> 273.
+    // 385 -> 391).  The other formats gain (all codes in full -> with, B = 16): UE5M3 678 -> 532, UE8M0 650 -> 115.  So does unscaled
+    // UE4M3 of weights (322 -> 167) and of N(0, 1) (322 -> 242).  Where its elements lie at the top of the codes or all over them
+    // there is little to skip, which only the kernel can see: N(0, 300) 322 -> 318, activations with outlier columns 322 -> 323; bf16
+    // loses most, outlier columns at B = 8 and 16 3 % (317 -> 326, 302 -> 311), exponents drawn from 22 binades 5 %.
     constexpr bool kHasPlain = FMT == kUE4M3 && B != 32;
     const bool plain = kHasPlain && slices == 1 && (a.d_global_scale != nullptr || a.global_scale != 1.0f);
     const void* kernel = reinterpret_cast<const void*>(k_brute<DT, B, G, FMT>);

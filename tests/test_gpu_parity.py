@@ -128,10 +128,11 @@ def test_brute_force_on_warps_of_unlike_blocks(B, fmt, sweep_mode):
 @pytest.mark.parametrize("B", BLOCKS)
 @pytest.mark.parametrize("fmt", FMTS)
 def test_pruned_sweep_at_the_edges_of_its_bounds(dtype, B, fmt):
-    """Tensors of one block, of part of a store unit and of one tile and a bit; blocks whose bounds leave nearly every code
-    (several elements far above the largest decode scale), whose codes are subnormal, whose elements are exact grid
-    multiples of a scale (the bounds are met with equality), and blocks and tensor scales outside the shortcuts' ranges."""
-    tile = 512 if B == 16 else max(256, 4096 // B)     # blocks the kernel sorts together
+    """Tensors of one block, of part of a store unit and of a few thousand blocks (in tiles of 32 to 64, which is what tensors of
+    this size are cut into); blocks whose bounds leave nearly every code (several elements far above the largest decode
+    scale), whose codes are subnormal, whose elements are exact grid multiples of a scale (the bounds are met with equality),
+    and blocks and tensor scales outside the shortcuts' ranges."""
+    tile = 512 if B == 16 else max(256, 4096 // B)     # blocks of a full tile
     gen = torch.Generator().manual_seed(77 + B + fmt)
     mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 1)
     try:
@@ -149,6 +150,73 @@ def test_pruned_sweep_at_the_edges_of_its_bounds(dtype, B, fmt):
                 check_parity(xd, B, fmt, recipe, g)
     finally:
         mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 0)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B", BLOCKS)
+@pytest.mark.parametrize("fmt", FMTS)
+def test_both_searches_on_tensors_that_fill_the_chip(dtype, B, fmt):
+    """5.2 million elements on 148 SMs: the full sweep's kernels without a split, their last group partial, and more full tiles of
+    the pruned search than CTAs, the last one partial.  Hard blocks dense at the start, in the middle and at the end and
+    sprinkled over the rest.  The two searches give the same bytes everywhere (but for blocks with a NaN or an infinity);
+    the hard blocks and the end agree with the oracle, and the fused MSE with the block SSEs."""
+    nb = torch.cuda.get_device_properties(0).multi_processor_count * 35200 // B + 13
+    n = nb * B
+    gen = torch.Generator().manual_seed(5 + B + fmt)
+    x = inputs.student_t(n, 4, 0.05, 331 + B, torch.float32, "cuda").cpu().view(nb, B)
+    dense = torch.zeros(nb, dtype=torch.bool)
+    for at in (0, nb // 2, nb - 300):
+        dense[at:at + 300] = True
+    dense[torch.randperm(nb, generator=gen)[:400]] = True
+    hard = torch.nonzero(dense).reshape(-1)
+    kind = torch.arange(hard.numel()) % 12
+    grid = torch.tensor([0.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, 6.0])
+    x[hard[kind == 1]] *= 2.0 ** 26                     # above 6 times the top scale
+    x[hard[kind == 2]] = x[hard[kind == 2]].sign() * 2.0 ** 24
+    x[hard[kind == 3]] *= 2.0 ** -12                    # subnormal scale codes of UE4M3, code 0
+    steps = torch.randint(0, 8, (int((kind == 4).sum()), B), generator=gen)
+    x[hard[kind == 4]] = grid[steps] * (1 + torch.arange(steps.shape[0]).view(-1, 1) % 8 / 8) * 0.0625
+    x[hard[kind == 5], 0] *= 2.0 ** 62                  # one huge element
+    x[hard[kind == 6]] *= 2.0 ** -60
+    x[hard[kind == 7]] = 0.0
+    x[hard[kind == 8], 1:] = 0.0
+    x[hard[kind == 9], 0] = 2.0 ** -140                 # one denormal
+    x[hard[kind == 10], B - 1] = float("nan")
+    x[hard[kind == 11], 0] = float("inf")
+    finite = torch.isfinite(x).all(1)
+    xd = x.reshape(-1).to(dtype).cuda()
+    sample = torch.cat([hard[finite[hard]], torch.arange(nb - 70, nb)[finite[nb - 70:]]])
+    xs = inputs.to_numpy_bits(xd.view(nb, B)[sample.cuda()].reshape(-1))
+    elems, keep = finite.cuda().repeat_interleave(B // 2), finite.cuda()
+    mse = torch.empty(1, dtype=torch.float64, device="cuda")
+    ws = torch.empty(mxq.mxq_tensor_mse_workspace_bytes(nb) // 8, dtype=torch.float64, device="cuda")
+    for recipe, g in ((mxq.MXQ_BRUTE, 1.0), (mxq.MXQ_BRUTE_PZ, 1.0), (mxq.MXQ_BRUTE_PZ, 0.0173), (mxq.MXQ_BRUTE, 2.0 ** -45),
+                      (mxq.MXQ_BRUTE, 1.5 * 2.0 ** -64), (mxq.MXQ_BRUTE_PZ, 1.5 * 2.0 ** 62)):
+        out = []
+        for prune in (0, 1):
+            mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, prune)
+            try:
+                codes, scales, sse = mxq.alloc_outputs(n, B, xd.device)
+                mxq.mxq_quantize_mse(xd, n, B, fmt, recipe, g, None, codes, scales, sse, mse, ws)
+                out.append((codes, scales, sse))
+            finally:
+                mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 0)
+            total = float(sse.double().sum() / n)      # infinite or NaN with the non-finite blocks
+            assert float(mse) == total or abs(float(mse) - total) <= 1e-12 * total or (total != total and float(mse) != float(mse))
+        for full, pruned, where in zip(out[0], out[1], (elems, keep, keep)):
+            assert torch.equal(full.view(torch.uint8).view(where.numel(), -1)[where], pruned.view(torch.uint8).view(where.numel(), -1)[where]), (recipe, g)
+        oc, os_, oe = orc.quantize(xs, B, fmt, recipe, g, threads=8)
+        codes, scales, sse = out[0]
+        assert np.array_equal(codes.view(nb, B // 2)[sample.cuda()].reshape(-1).cpu().numpy(), oc), (recipe, g)
+        assert np.array_equal(scales[sample.cuda()].cpu().numpy(), os_), (recipe, g)
+        assert np.array_equal(sse[sample.cuda()].cpu().numpy().view(np.uint32), oe.view(np.uint32)), (recipe, g)
+    # the same without the non-finite blocks, so that the fused sum is a number
+    xd = torch.where(torch.isfinite(xd), xd, torch.zeros_like(xd)).clamp(-1e6, 1e6)
+    for g in (1.0, 0.0173):
+        codes, scales, sse = mxq.alloc_outputs(n, B, xd.device)
+        mxq.mxq_quantize_mse(xd, n, B, fmt, mxq.MXQ_BRUTE, g, None, codes, scales, sse, mse, ws)
+        total = float(sse.double().sum() / n)
+        assert total > 0.0 and abs(float(mse) - total) <= 1e-12 * total
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
