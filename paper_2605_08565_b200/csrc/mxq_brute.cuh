@@ -2,19 +2,23 @@
 // scale values and keeping the one with the least error): every finite scale code of the format
 // is tried on every block and the code with the smallest SSE is kept (equal SSE: the smaller code).
 //
-// Work layout.  A thread keeps its elements in registers as float pairs and the candidate loop
-// works on float pairs with the packed binary32 instructions of sm_100 (fma.rn.f32x2 /
+// Work layout.  A thread owns a group of G consecutive elements, whole blocks: G = B for B >= 32; 16 for B = 2 and 4; 32 for B = 8 and
+// 16, or 16 where the tensor is too small to fill the chip with groups of 32 (launch_brute_inst()).  They stay in registers as float
+// pairs and the candidate loop works on pairs with the packed binary32 instructions of sm_100 (fma.rn.f32x2 /
 // mul.rn.f32x2, FP4 pack and unpack two at a time):
-//   B <= 16   the thread owns G = 32 consecutive elements (16 for B = 2), pair i = (element i,
-//             element G/2 + i): the two halves of a pair belong to different blocks, so one instruction serves two
-//             elements of one candidate and the two SSE chains are independent.  Two candidates
+//   G > B     pair i = (element i, element G/2 + i): the two halves of a pair belong to different blocks, so one
+//             instruction serves two elements of one candidate and the two SSE chains are independent.  Two candidates
 //             per trip.
-//   B >= 32   the thread owns one block, pair i = (element 2i, element 2i + 1).  Its SSE is one
+//   G = B     the thread owns one block, pair i = (element 2i, element 2i + 1).  Its SSE is one
 //             sequential chain over all elements, so the two lanes of the SSE pair are two
 //             CANDIDATES: the scaling multiplies run on element pairs, the FP4 rounding and the
 //             residuals on candidate pairs of one element, and the elements are walked in order.
-// The candidate loop is uniform across the CTA: decode scales come from shared memory as
-// broadcasts.
+// The candidate loop is uniform across a warp (not across the CTA: a warp's ranges depend on its elements, its slice of the codes on
+// its place): decode scales come from shared memory as broadcasts, and no barrier may stand inside.
+//
+// Three kernels: k_brute leaves the cheap stretches of the codes out of the full evaluation, any number of blocks; k_brute_plain
+// evaluates every code in full, whole groups only (k_brute_split takes the blocks behind them); k_brute_split shares a group
+// between 2, 4 or 8 warps, any number of blocks.
 //
 // One exact quotient per mantissa, not per candidate.  The decode scale of code c is
 // D_c = fl(S_c * g).  All codes whose S_c share a mantissa (eight classes for the FP8 scale
@@ -22,8 +26,8 @@
 // D_c = Dref * 2^k, as long as D_c is a normal number.  Hence fl(v / D_c) = fl(v / Dref) * 2^-k
 // exactly: the correctly rounded quotient is formed once per class and element, and a candidate
 // costs one multiply by a power of two, the FP4 rounding, and the two FMAs of the SSE.  Codes under
-// which every element of the warp rounds to zero or saturates cost less (search_group()).  Threads holding a magnitude above 2^60
-// or a nonzero one below 2^-62 take the general path (IEEE division), candidate by candidate.
+// which every element of the warp rounds to zero or saturates cost less (search_group()).  Threads holding a magnitude above
+// 2^60 or a nonzero one below 2^-62 take the general path (IEEE division), candidate by candidate.
 //
 // Inside a class the members are visited in ascending code order and the smallest SSE bit pattern
 // is kept with a strict compare (SSE >= 0, so integer order is float order and the first of equals

@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, pruned_min_ctas(B)) k_pruned(QuantAr
                                 constexpr float kW = 1.0f / 262144.0f;
                                 const int l6 = first_code(__fmul_rn(ul, (1.0f - kW) / 6.0f)), h6 = last_code(__fmul_rn(uh, (1.0f + kW) / 6.0f));
                                 const int l4 = first_code(__fmul_rn(ul, (1.0f - kW) / 4.0f)), h4 = last_code(__fmul_rn(uh, (1.0f + kW) / 4.0f));
-                                // r < a / 2: a window spans at most 1.6 binades, 13 codes
+                                // r < a / 2: a window reaches from u - r to u + r, a factor of at most 3 (1.6 binades), 14 codes
                                 const uint32_t w6 = (1u << (h6 - l6 + 1)) - 1u, w4 = (1u << (h4 - l4 + 1)) - 1u;
                                 const uint32_t p6 = w6 | (w6 << 8) | (w6 << 16);                       // q = 6, 3, 3/2
                                 const unsigned long long p4 = (unsigned long long)(w4 >> 8) << 32 |    // q = 4, 2, 1, 1/2
