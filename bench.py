@@ -735,7 +735,7 @@ def run_gpu(args) -> None:
                 "peak_source": f"{n_sm} SMs x 128 lanes x {peaks['sm_max_mhz']:.0f} MHz (max SM clock, {peaks['source']})",
                 "launches_per_step": len(per_inst), "ms_per_launch": tot_ms / len(per_inst),
                 "ms_all_launches_per_step": tot_ms, "share_of_step_time": tot_ms / step_ms,
-                "largest_share": largest, "per_instantiation": per_inst}
+                "largest_share": largest}
     legs = {leg: {"ms_per_step": wl.mean_ms(evs),
                   "gelem_s": sum(p[2] for p in wl.passes if p[0] == leg) / (wl.mean_ms(evs) * 1e-3) / 1e9}
             for leg, evs in wl.leg_events.items()}
@@ -758,14 +758,19 @@ def run_gpu(args) -> None:
 
     names = [f"{leg}:{key}:B{B}:{FMT_NAME[fmt]}:{RECIPE_NAME[r]}" + (":g" if hier else "")
              for leg, key, _, B, fmt, r, hier in wl.passes]
+    # the tables of the single kernels and passes go to stderr: the result line has to stay short enough to be read whole
+    print("details " + json.dumps({
+        "roofline_per_instantiation": per_inst, "roofline_hbm": hbm, "roofline_hbm_streaming": streaming,
+        "brute_pruned_sweep": pruned, "weight_set_8_layers": weight_set,
+        "mse": {nm: float(mse_host[i]) for i, nm in enumerate(names)},
+    }), file=sys.stderr)
     print(json.dumps({
         "metric": METRIC, "value": value / 1e9, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": step_ms, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": WORKLOAD_NAME, "elements_per_step": wl.elems_per_step, "passes_per_step": len(wl.passes),
                    "l2": "search tensor 1 GiB > 126 MB L2; the legs walk their tensors round-robin (277 MB and 201 MB sets)"},
-        "roofline": roofline, "legs": legs, "roofline_hbm": hbm, "roofline_hbm_streaming": streaming,
-        "brute_pruned_sweep": pruned, "weight_set_8_layers": weight_set, "cpu_baseline": cpu_baseline,
+        "roofline": roofline, "legs": legs, "cpu_baseline": cpu_baseline,
         "e2e": {"value": e2e_value / 1e9, "unit": UNIT, "h2d_bytes_per_step": int(h2d_bytes),
                 "d2h_bytes_per_step": int(host_out.numel() * 8), "steps": e2e_steps,
                 "what": "the same step with all inputs copied from pinned host memory every step (overlapped with the "
@@ -775,7 +780,6 @@ def run_gpu(args) -> None:
                                  "what": "one abs-max pass (14336x4096 bf16, B=16, UE4M3): input from pinned host memory, "
                                          "codes and scale bytes back to pinned host memory, one stream, no overlap"},
         "gpu_launches": int(launches), "clocks": clocks,
-        "mse": {nm: float(mse_host[i]) for i, nm in enumerate(names)},
     }))
     dist.shutdown()
 
@@ -1073,6 +1077,10 @@ def run_single_kernel(args) -> None:
         sh = torch.zeros(256, dtype=torch.int64, device=dev)
         fn = lambda: mxq.mxq_histograms(codes, scales, n, B, ch, sh)
         nbytes = n * (0.5 + 1.0 / B)
+    elif args.kernel == "clip":
+        mxq.mxq_quantize_ex(x, n, B, fmt, 0, g, None, codes, scales, sse)
+        fn = lambda: mxq.mxq_block_clip_sse(x, n, B, fmt, g, None, scales, sse)
+        nbytes = n * (eb + 5.0 / B)
     else:
         raise SystemExit(f"unknown --kernel {args.kernel}")
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev) if n * eb < (256 << 20) else None
@@ -1097,7 +1105,7 @@ def run_single_kernel(args) -> None:
 
 def main() -> None:
     ap = argparse.ArgumentParser()
-    ap.add_argument("--kernel", default=None, help="time one kernel alone: absmax|absmax_pz|4o6|4o6_pz|brute|brute_pz|amax|mse|dequant|hist")
+    ap.add_argument("--kernel", default=None, help="time one kernel alone: absmax|absmax_pz|4o6|4o6_pz|brute|brute_pz|amax|mse|dequant|hist|clip")
     ap.add_argument("--config", default=None, help="time one benchmark configuration (1..5, comma list, or all), one recipe at a time")
     ap.add_argument("--hash-inputs", action="store_true", help="with --config: record the SHA-256 of every configuration's input bytes")
     ap.add_argument("--block", type=int, default=16)
@@ -1112,7 +1120,7 @@ def main() -> None:
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--skip-extras", action="store_true",
                     help="leave out the measurements taken outside the timed step (roofline_hbm, roofline_hbm_streaming, "
-                         "brute_pruned_sweep = null)")
+                         "brute_pruned_sweep = null in the details)")
     ap.add_argument("--impl", default="mxq", choices=["mxq", "reference"])
     args = ap.parse_args()
     if args.kernel:
