@@ -202,57 +202,64 @@ cudaError_t launch_histograms(const uint8_t* codes, const uint8_t* scales, size_
 }
 
 // ------------------------------------------------------------------------------------------------
-// Segment MSE: out[s] = (sum of the block SSEs of segment s) / elems_per_segment.  One CTA of T threads per
-// segment (grid-stride over segments), binary64 sums whose shape depends on the length of the segment alone: thread t adds
-// elements t, t + T, ..., four at a time as (a + b) + (c + d) with zeros past the end, then a shuffle tree per warp and one over
-// the warps.  The same values give the same bits wherever the segment lies.  Single floats are read, not vectors of four: a warp's
-// reads are whole lines at any alignment, and the conversions and additions to binary64 cost more than the wider loads save.
-// What a segment needs is loads in flight, sixteen a thread at full occupancy (32 registers): short segments are better off
-// with many CTAs, long ones with wide ones.  151 segments, us with the launch, T = 256 / 512 / 1024: 1000 blocks 1.6 / 1.6 / 2.2, 8000
-// 2.4 / 2.2 / 2.9, 20,000 3.8 / 3.5 / 3.5, 50,000 7.3 / 6.0 / 6.1, 400,000 124 / 69 / 50; 10,000 segments of 64 9.8 / 19 / 37, 500 of 12,000
-// 4.0 / 4.4 / 5.0.
+// Segment MSE: out[s] = (sum of the block SSEs of segment s) / elems_per_segment.  One CTA per segment (grid-stride over
+// segments), binary64 sums whose shape depends on the length of the segment alone: L lanes (256 below 4096 blocks, 512 below 8192, else 1024),
+// lane i adds elements i, i + L, ..., four at a time as (a + b) + (c + d) with zeros past the end, then a shuffle tree over 32
+// lanes and one over their sums.  The same values give the same bits wherever the segment lies and however many threads share the
+// lanes.  Single floats are read, not vectors of four: a warp's reads are whole lines at any alignment.  What a segment needs is
+// loads in flight, sixteen a thread (with full occupancy at 32 registers).
 // ------------------------------------------------------------------------------------------------
-template <int T>
+template <int T, int L>
 __global__ void __launch_bounds__(T, 2048 / T) k_segment_mse(const float* sse, size_t n_segments, size_t blocks_per_segment,
-                                                   double elems_per_segment, double* out) {
-    __shared__ double sh[T / 32];
+                                                             double elems_per_segment, double* out) {
+    constexpr int A = L / T;             // lanes per thread: t, t + T, ...
+    static_assert(A == 1 || A == 2 || A == 4, "sixteen elements of a thread are whole groups of four of its lanes");
+    __shared__ double sh[L / 32];
     wait_for_prior_grid();
     release_dependents();
     for (size_t seg = blockIdx.x; seg < n_segments; seg += gridDim.x) {
         const float* p = sse + seg * blocks_per_segment;
-        double acc = 0.0;
-        auto add_four = [&](const float* w) {
-            acc = __dadd_rn(acc, __dadd_rn(__dadd_rn((double)w[0], (double)w[1]), __dadd_rn((double)w[2], (double)w[3])));
+        double acc[A];
+#pragma unroll
+        for (int a = 0; a < A; ++a) acc[a] = 0.0;
+        // element m * T + t belongs to lane m % A of the thread: group r of a lane is m = (4 r + 0 .. 3) A + a
+        auto add_four = [&](const float* w, int r, int a) {
+            const float* const x = w + 4 * r * A + a;
+            acc[a] = __dadd_rn(acc[a], __dadd_rn(__dadd_rn((double)x[0], (double)x[A]), __dadd_rn((double)x[2 * A], (double)x[3 * A])));
         };
         size_t i = threadIdx.x;
         for (; i + 15 * T < blocks_per_segment; i += 16 * T) {
             float w[16];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) w[u] = p[i + u * T];
+            for (int m = 0; m < 16; ++m) w[m] = p[i + m * T];
 #pragma unroll
-            for (int u = 0; u < 16; u += 4) add_four(w + u);
+            for (int k = 0; k < 4; ++k) add_four(w, k / A, k % A);
         }
         const int rest = (int)(blocks_per_segment - (i - threadIdx.x));   // negative or below 16 T
         const float* const q = p + (i - threadIdx.x);
         if (rest > 4 * T) {
             float w[16];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) w[u] = (int)threadIdx.x + u * T < rest ? q[u * T + threadIdx.x] : 0.0f;
+            for (int m = 0; m < 16; ++m) w[m] = (int)threadIdx.x + m * T < rest ? q[m * T + threadIdx.x] : 0.0f;
 #pragma unroll
-            for (int u = 0; u < 16; u += 4)
-                if (u * T < rest) add_four(w + u);
+            for (int k = 0; k < 4; ++k)
+                if (4 * (k / A) * L < rest) add_four(w, k / A, k % A);
         } else if (rest > 0) {
-            float w[4];
+            float w[4 * A];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) w[u] = (int)threadIdx.x + u * T < rest ? q[u * T + threadIdx.x] : 0.0f;
-            add_four(w);
+            for (int m = 0; m < 4 * A; ++m) w[m] = m < 4 && (int)threadIdx.x + m * T < rest ? q[m * T + threadIdx.x] : 0.0f;
+#pragma unroll
+            for (int a = 0; a < A; ++a) add_four(w, 0, a);
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc = __dadd_rn(acc, __shfl_down_sync(0xFFFFFFFFu, acc, o));
-        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+        for (int a = 0; a < A; ++a) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc[a] = __dadd_rn(acc[a], __shfl_down_sync(0xFFFFFFFFu, acc[a], o));
+            if ((threadIdx.x & 31) == 0) sh[a * (T / 32) + (threadIdx.x >> 5)] = acc[a];
+        }
         __syncthreads();
         if (threadIdx.x < 32) {
-            double t = threadIdx.x < T / 32 ? sh[threadIdx.x] : 0.0;
+            double t = threadIdx.x < L / 32 ? sh[threadIdx.x] : 0.0;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) t = __dadd_rn(t, __shfl_down_sync(0xFFFFFFFFu, t, o));
             if (threadIdx.x == 0) out[seg] = __ddiv_rn(t, elems_per_segment);
@@ -266,10 +273,21 @@ cudaError_t launch_segment_mse(const float* sse, size_t n_segments, size_t block
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
-    const int threads = blocks_per_segment < 16384 ? 256 : blocks_per_segment < 131072 ? 512 : 1024;
-    const size_t cap = (size_t)sm_count(dev) * (2048 / threads);
+    const size_t sms = (size_t)sm_count(dev);
+    // Few segments need wide CTAs, many of them small ones; what counts is the pass right after the one that wrote the SSEs, which
+    // finds part of them in L2 only.  us added to that pass, T = 256 / 512 / 1024: 151 segments of 6000 blocks 4.5 / 3.2 / 3.1, 10,000 6.2 /
+    // 3.9 / 3.4, 50,000 25 / 15 / 10; 500 of 4096 3.9 / 2.7 / 4.4, of 20,000 22 / 15 / 18; 10,000 of 64, from L2, 9.8 / 19 / 37.
+    int threads = 256;
+    auto* kernel = k_segment_mse<256, 256>;
+    if (blocks_per_segment >= 8192) {
+        threads = n_segments <= 3 * sms ? 1024 : 512;
+        kernel = threads == 1024 ? k_segment_mse<1024, 1024> : k_segment_mse<512, 1024>;
+    } else if (blocks_per_segment >= 4096) {
+        threads = n_segments <= 4 * sms ? 512 : 256;
+        kernel = threads == 512 ? k_segment_mse<512, 512> : k_segment_mse<256, 512>;
+    }
+    const size_t cap = sms * (2048 / threads);
     const unsigned grid = (unsigned)(n_segments < cap ? n_segments : cap);
-    auto* const kernel = threads == 256 ? k_segment_mse<256> : threads == 512 ? k_segment_mse<512> : k_segment_mse<1024>;
     err = launch_pdl(kernel, grid, (unsigned)threads, 0, s, sse, n_segments, blocks_per_segment, (double)elems_per_segment, out);
     count_launch();
     return err;
