@@ -20,9 +20,10 @@ namespace mxq {
 // No division for decode scales within [2^-100, 2^100]: floats are 2^-21 apart above 6, and half way to the next one a tie
 // rounds to 6, so fl32(v / D) > 6  <=>  v / D > 6 + 2^-22  <=>  |v| - 6 D > 2^-22 D.  The difference is formed by one FMA: near
 // the limit it is a multiple of 2^(e - 22) below 2^(e - 20), D in [2^e, 2^(e+1)), and therefore exact, as is 2^-22 D; away
-// from the limit its rounding cannot change the outcome.  It is also the residual.  Bound by the reads of x: fp32, B = 8,
-// 60.4 M elements (279 MB) 62 -> 53 us, B = 4 72 -> 58.  The last block of a thread goes alone: a second load that is not needed
-// (the tensor's last block, for every thread of a small tensor) cost bf16, B = 2 1.05 -> 1.28 us at 4096 elements.
+// from the limit its rounding cannot change the outcome.  It is also the residual.  Bound by the reads of x: fp32,
+// B = 8, from memory, 16.8 M elements (77 MB) 16.8 -> 13.2 us against a division per element and one block at a time; 60.4 M 45 us.  The
+// last block of a thread goes alone: a second load that is not needed (the tensor's last block, for every thread of a small
+// tensor) cost bf16, B = 2 1.05 -> 1.28 us at 4096 elements.
 // ------------------------------------------------------------------------------------------------
 template <int B>
 __device__ __forceinline__ float clip_sse(const float (&v)[B], int c, int fmt, float gs) {
@@ -112,7 +113,8 @@ cudaError_t launch_block_clip_sse(const void* x, int dtype, size_t n, int B, int
 // per lane and bank, so that no two lanes of a warp meet at an address or in a bank (one table per warp
 // with all lanes in it: three to five lanes a bank, and every repeated value the same address).  16-byte loads, no per-code
 // compares.  Per-CTA counts are 32-bit (a CTA sees far fewer than 2^32 bytes), flushed with 64-bit integer atomics --
-// integer sums are order-free, so the result is deterministic.  Bound by the shared-memory atomics: 60.4 M codes and 7.5 M scales 29 -> 23 us with the launch.
+// integer sums are order-free, so the result is deterministic.  60.4 M codes and 7.5 M scales 29 -> 23 us with the launch; bound by the
+// latency of the one load that a thread has in flight in front of sixteen atomics, then by the atomics (LSU pipe 46 %).
 // ------------------------------------------------------------------------------------------------
 constexpr int kHistThreads = 512;
 constexpr size_t kHistBytes = 2 * 256 * 32 * sizeof(unsigned int);
