@@ -299,13 +299,13 @@ int mxq_mask_interval(const void* x, int dtype, size_t n, float lo, float hi, vo
  * code, as the search is stated (Experimental Setup), and keep the smallest; nothing depends on the SSEs of
  * other codes.  (Codes under which the same sum of squares arises by definition -- every element rounds
  * to zero, or the scale is too small to change any element -- share one evaluation.)  With 1 the kernel leaves out the
- * codes that provably cannot change an output of the block, given the better SSE of two codes tried first:
- *   - decode scales of at least four times the block maximum: every element quantizes to zero
- *     (|v|/D <= 1/4 rounds to the grid value 0), so all of them have the SSE of the all-zero
- *     quantization, which is entered once with the smallest such code;
- *   - decode scales so large that the elements they send to zero alone already cost more;
- *   - decode scales so small that the saturation error of the largest element alone already costs more;
- *   - decode scales none of whose multiples by an FP4 grid value comes near enough to the largest element.
+ * codes that provably cannot change an output of the block:
+ *   - twice a decode scale D with 7 D > max |v|: the FP4 grid times 2 D has no point near an element that the grid
+ *     times D lacks, so no element's error is smaller than under D (and the smaller code wins a tie);
+ *   - decode scales so small that the saturation error of the largest element, or of all of them, alone already
+ *     costs more than the best SSE so far;
+ *   - among the odd ones of the fifteen smallest codes, which have no half: decode scales so large that the
+ *     elements they send to zero, or the error of the largest element, alone already cost more.
  * The bounds hold for the kernel's own binary32 arithmetic, so the outputs (codes, scale bytes, block
  * SSE; ties to the smaller code) are bit-identical to the full sweep; only the time differs, by an
  * amount that depends on the data.  The paper states no such shortcut.

@@ -155,6 +155,37 @@ def test_pruned_sweep_at_the_edges_of_its_bounds(dtype, B, fmt):
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("B", BLOCKS)
 @pytest.mark.parametrize("fmt", FMTS)
+def test_pruned_search_around_its_first_and_last_code(dtype, B, fmt):
+    """Block maxima at 3.5, 6 and 7 times a decode scale and one unit either side (the code the search starts from is 2 / 7 of the
+    maximum), over subnormal and normal scale codes; beside the maximum ordinary elements, zeros only (several codes tie), equal
+    elements, and elements just above a grid midpoint; blocks whose other elements are all as large as they can be without
+    saturating, under which the search runs on below its eight codes."""
+    gen = torch.Generator().manual_seed(3 * B + fmt)
+    scales = torch.tensor([orc.scale_value(fmt, c) for c in (range(100, 140) if fmt == mxq.MXQ_SF_UE8M0 else range(1, 64))], dtype=torch.float64)
+    for g in (1.0, 0.0131):
+        D = (scales * g).float()
+        peak = torch.cat([D * k for k in (3.5, 6.0, 7.0)])
+        peak = torch.cat([peak, torch.nextafter(peak, torch.zeros(1)), torch.nextafter(peak, torch.full((1,), 1e38))])
+        nb = 5 * peak.numel()
+        x = torch.rand(nb, B, generator=gen)
+        x[0::5] = 0.0
+        x[1::5] = 1.0
+        x[2::5] = (2.5 + 2.0 ** -20) / 6.0
+        x[3::5] = 0.8 + 0.2 * x[3::5]
+        x[:, B - 1] = 1.0
+        x = x * peak.repeat_interleave(5).view(nb, 1) * torch.where(torch.rand(nb, B, generator=gen) < 0.5, -1.0, 1.0)
+        xd = x.reshape(-1).to(dtype).contiguous()
+        for recipe in (mxq.MXQ_BRUTE, mxq.MXQ_BRUTE_PZ):
+            mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 1)
+            try:
+                check_parity(xd, B, fmt, recipe, g)
+            finally:
+                mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 0)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B", BLOCKS)
+@pytest.mark.parametrize("fmt", FMTS)
 def test_both_searches_on_tensors_that_fill_the_chip(dtype, B, fmt):
     """5.2 million elements on 148 SMs: the full sweep's kernels without a split, their last group partial, and more full tiles of
     the pruned search than CTAs, the last one partial.  Hard blocks dense at the start, in the middle and at the end and

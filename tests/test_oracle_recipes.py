@@ -381,3 +381,31 @@ def test_block_maxima_next_to_a_scale_midpoint_follow_two_divisions(g):
                 one_div = ex.round_scale_exact(orc.UE4M3, ex.f32_div(a, ex.f32_mul(f32(g), f32(M))))
                 differ += int(one_div != want)
     assert differ > 0
+
+
+@pytest.mark.parametrize("fmt", FMTS)
+@pytest.mark.parametrize("g", [1.0, 0.0131, 1.37 * 2.0 ** -45])
+def test_twice_a_decode_scale_above_a_seventh_of_the_maximum_is_never_better(fmt, g):
+    """What the pruned search rests on: with 7 D > max |v|, no block has a smaller SSE under 2 D than under D, in the binary32
+    arithmetic of the SSE.  Elements at the rounding midpoints of both grids and one unit either side, zeros, and random
+    ones; the maximum a few units below 7 D."""
+    rng = np.random.default_rng(17 + fmt)
+    codes = range(1, 254) if fmt == orc.UE8M0 else range(1, orc.num_codes(fmt) - 8)
+    for c in codes:
+        twice = c + 1 if fmt == orc.UE8M0 else (2 * c if c < 8 else c + 8)
+        D, D2 = f32(orc.scale_value(fmt, c)) * f32(g), f32(orc.scale_value(fmt, twice)) * f32(g)
+        if not (2.0 ** -126 <= float(D) and float(D2) < 2.0 ** 100):
+            continue
+        assert D2 == 2 * D
+        mid = (np.array([0.25, 0.75, 1.25, 1.75, 2.5, 3.5, 5.0, 0.5, 1.5, 3.0, 4.0, 6.0, 7.0]) * float(D)).astype(f32)
+        v = np.concatenate([mid, np.nextafter(mid, f32(0.0)), np.nextafter(mid, f32(np.inf)), np.zeros(3, f32),
+                            (rng.random(22) * 7.0 * float(D)).astype(f32)])
+        v = np.minimum(v, f32(7.0 * float(D) * (1.0 - 2.0 ** -19)))
+        rng.shuffle(v)
+        v = v * rng.choice(np.array([-1.0, 1.0], dtype=f32), v.size)
+        for B in (2, 8, 64):
+            for k in range(0, v.size - B + 1, B):
+                blk = np.ascontiguousarray(v[k:k + B])
+                s1, s2 = orc.block_sse(blk, fmt, c, g), orc.block_sse(blk, fmt, twice, g)
+                s1, s2 = (s1[0] if isinstance(s1, tuple) else s1), (s2[0] if isinstance(s2, tuple) else s2)
+                assert s2 >= s1, (c, twice, blk)
