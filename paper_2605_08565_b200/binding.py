@@ -1,4 +1,7 @@
-"""Thin ctypes binding of libmxq (argument marshalling only; every step runs in the CUDA kernels).
+"""Thin binding of libmxq (argument marshalling only; every step runs in the CUDA kernels).
+
+The calls of an inner loop go through the extension module ``_native`` (csrc/mxq_python.cpp), which unpacks the usual
+arguments in C++; everything else, and whatever ``_native`` does not take, goes through ctypes.
 
 The functions carry the names of the C-ABI declared in ``include/mxq.h`` and take torch CUDA
 tensors (torch supplies device memory and streams, nothing else).  There is no CPU fallback: if
@@ -39,11 +42,12 @@ class TensorDesc(ctypes.Structure):
 
 
 _lib = None
+_native = None
 
 
 def load_library() -> ctypes.CDLL:
     """dlopen libmxq.so (built by ``paper_2605_08565_b200.build``); raises if it is missing."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -96,6 +100,12 @@ def load_library() -> ctypes.CDLL:
     L.mxq_last_cuda_error.argtypes = []
     L.mxq_version.restype = i32
     L.mxq_version.argtypes = []
+    try:
+        from . import _native as native
+    except ImportError as e:
+        raise MxqError(f"extension module _native not found ({e}): build it with `python -m paper_2605_08565_b200.build`") from e
+    native.bind({name: c.cast(getattr(L, name), vp).value for name in EXPORTS})
+    _native = native
     _lib = L
     return L
 
@@ -107,6 +117,11 @@ def _check(status: int) -> None:
         if status == 7:
             msg += f" [cudaError {L.mxq_last_cuda_error()}]"
         raise MxqError(f"libmxq status {status}: {msg}")
+
+
+def _load_native():
+    load_library()
+    return _native
 
 
 def _ptr(t) -> int:
@@ -149,6 +164,12 @@ def mxq_quantize(x, n, block_size, scale_fmt, recipe, global_scale, out_codes, o
 
 def mxq_quantize_ex(x, n, block_size, scale_fmt, recipe, global_scale, d_global_scale, out_codes, out_scales,
                     out_block_sse, stream=None) -> None:
+    st = (_native or _load_native()).quantize_ex(x, n, block_size, scale_fmt, recipe, global_scale, d_global_scale,
+                                                 out_codes, out_scales, out_block_sse, stream)
+    if st == 0:
+        return
+    if st > 0:
+        _check(st)
     _check(load_library().mxq_quantize_ex(_ptr(x), _dtype_id(x), n, block_size, scale_fmt, recipe, global_scale,
                                           _ptr(d_global_scale), _ptr(out_codes), _ptr(out_scales),
                                           _ptr(out_block_sse), _stream(stream, x)))
@@ -157,6 +178,13 @@ def mxq_quantize_ex(x, n, block_size, scale_fmt, recipe, global_scale, d_global_
 def mxq_quantize_mse(x, n, block_size, scale_fmt, recipe, global_scale, d_global_scale, out_codes, out_scales,
                      out_block_sse, d_out_mse, d_workspace, stream=None) -> None:
     """Quantize and score in one call: the tensor MSE comes from partial sums formed inside the quantization kernel."""
+    st = (_native or _load_native()).quantize_mse(x, n, block_size, scale_fmt, recipe, global_scale, d_global_scale,
+                                                  out_codes, out_scales, out_block_sse, d_out_mse, d_workspace,
+                                                  stream)
+    if st == 0:
+        return
+    if st > 0:
+        _check(st)
     ws_bytes = d_workspace.numel() * d_workspace.element_size() if d_workspace is not None else 0
     _check(load_library().mxq_quantize_mse(_ptr(x), _dtype_id(x), n, block_size, scale_fmt, recipe, global_scale,
                                            _ptr(d_global_scale), _ptr(out_codes), _ptr(out_scales), _ptr(out_block_sse),
@@ -179,17 +207,35 @@ def make_tensor_descs(items):
 def mxq_quantize_batch(h_descs, d_descs, n_tensors, dtype_id, block_size, scale_fmt, recipe, global_scale=1.0,
                        d_global_scale=None, stream=None) -> None:
     """One launch over a list of tensors; h_descs / d_descs from ``make_tensor_descs``."""
+    st = (_native or _load_native()).quantize_batch(ctypes.addressof(h_descs), d_descs, n_tensors, dtype_id,
+                                                    block_size, scale_fmt, recipe, global_scale, d_global_scale,
+                                                    stream)
+    if st == 0:
+        return
+    if st > 0:
+        _check(st)
     _check(load_library().mxq_quantize_batch(ctypes.addressof(h_descs), _ptr(d_descs), n_tensors, dtype_id, block_size,
                                              scale_fmt, recipe, global_scale, _ptr(d_global_scale),
                                              _stream(stream, d_descs)))
 
 
 def mxq_fake_quantize(x, n, block_size, scale_fmt, recipe, global_scale, d_global_scale, d_out, stream=None) -> None:
+    st = (_native or _load_native()).fake_quantize(x, n, block_size, scale_fmt, recipe, global_scale, d_global_scale,
+                                                   d_out, stream)
+    if st == 0:
+        return
+    if st > 0:
+        _check(st)
     _check(load_library().mxq_fake_quantize(_ptr(x), _dtype_id(x), n, block_size, scale_fmt, recipe, global_scale,
                                             _ptr(d_global_scale), _ptr(d_out), _dtype_id(d_out), _stream(stream, x)))
 
 
 def mxq_tensor_amax(x, n, d_out_amax, d_out_global_scale=None, stream=None) -> None:
+    st = (_native or _load_native()).tensor_amax(x, n, d_out_amax, d_out_global_scale, stream)
+    if st == 0:
+        return
+    if st > 0:
+        _check(st)
     _check(load_library().mxq_tensor_amax(_ptr(x), _dtype_id(x), n, _ptr(d_out_amax), _ptr(d_out_global_scale),
                                           _stream(stream, x)))
 
@@ -203,6 +249,11 @@ def mxq_tensor_mse_workspace_bytes(n_blocks: int) -> int:
 
 
 def mxq_tensor_mse(d_block_sse, n_blocks, n, d_out_mse, d_workspace, stream=None) -> None:
+    st = (_native or _load_native()).tensor_mse(d_block_sse, n_blocks, n, d_out_mse, d_workspace, stream)
+    if st == 0:
+        return
+    if st > 0:
+        _check(st)
     ws_bytes = d_workspace.numel() * d_workspace.element_size() if d_workspace is not None else 0
     _check(load_library().mxq_tensor_mse(_ptr(d_block_sse), n_blocks, n, _ptr(d_out_mse), _ptr(d_workspace),
                                          ws_bytes, _stream(stream, d_block_sse)))
@@ -219,23 +270,46 @@ def mxq_dequantize(d_codes, d_scales, n, block_size, scale_fmt, global_scale, d_
 
 
 def mxq_dequantize_ex(d_codes, d_scales, n, block_size, scale_fmt, global_scale, d_global_scale, d_out, stream=None) -> None:
+    st = (_native or _load_native()).dequantize_ex(d_codes, d_scales, n, block_size, scale_fmt, global_scale,
+                                                   d_global_scale, d_out, stream)
+    if st == 0:
+        return
+    if st > 0:
+        _check(st)
     _check(load_library().mxq_dequantize_ex(_ptr(d_codes), _ptr(d_scales), n, block_size, scale_fmt, global_scale,
                                             _ptr(d_global_scale), _ptr(d_out), _dtype_id(d_out), _stream(stream, d_out)))
 
 
 def mxq_block_clip_sse(x, n, block_size, scale_fmt, global_scale, d_global_scale, d_scales, out_clip_sse,
                        stream=None) -> None:
+    st = (_native or _load_native()).block_clip_sse(x, n, block_size, scale_fmt, global_scale, d_global_scale,
+                                                    d_scales, out_clip_sse, stream)
+    if st == 0:
+        return
+    if st > 0:
+        _check(st)
     _check(load_library().mxq_block_clip_sse(_ptr(x), _dtype_id(x), n, block_size, scale_fmt, global_scale,
                                              _ptr(d_global_scale), _ptr(d_scales), _ptr(out_clip_sse), _stream(stream, x)))
 
 
 def mxq_histograms(d_codes, d_scales, n, block_size, d_code_hist, d_scale_hist, stream=None) -> None:
     """d_code_hist: 16 and d_scale_hist: 256 int64/uint64 CUDA counters; counts are added to them."""
+    st = (_native or _load_native()).histograms(d_codes, d_scales, n, block_size, d_code_hist, d_scale_hist, stream)
+    if st == 0:
+        return
+    if st > 0:
+        _check(st)
     _check(load_library().mxq_histograms(_ptr(d_codes), _ptr(d_scales), n, block_size, _ptr(d_code_hist),
                                          _ptr(d_scale_hist), _stream(stream, d_codes)))
 
 
 def mxq_segment_mse(d_block_sse, n_blocks, blocks_per_segment, elems_per_segment, d_out_mse, stream=None) -> None:
+    st = (_native or _load_native()).segment_mse(d_block_sse, n_blocks, blocks_per_segment, elems_per_segment,
+                                                 d_out_mse, stream)
+    if st == 0:
+        return
+    if st > 0:
+        _check(st)
     _check(load_library().mxq_segment_mse(_ptr(d_block_sse), n_blocks, blocks_per_segment, elems_per_segment,
                                           _ptr(d_out_mse), _stream(stream, d_block_sse)))
 
@@ -245,7 +319,7 @@ def mxq_mask_interval(x, n, lo, hi, d_out, stream=None) -> None:
 
 
 def mxq_set_option(option: int, value: int) -> None:
-    _check(load_library().mxq_set_option(int(option), int(value)))
+    _check((_native or _load_native()).set_option(int(option), int(value)))
 
 
 def mxq_get_option(option: int) -> int:

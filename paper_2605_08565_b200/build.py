@@ -1,10 +1,11 @@
-"""Build libmxq.so (hand-written CUDA for sm_100a) in-tree with nvcc.
+"""Build libmxq.so (hand-written CUDA for sm_100a) in-tree with nvcc, and the extension module _native with g++.
 
 ``python -m paper_2605_08565_b200.build [--force] [--verbose]``
 
 Every ``csrc/*.cu`` is compiled to an object file in ``_build/`` (in parallel) and linked into
 ``paper_2605_08565_b200/libmxq.so``.  No fast-math, no flush-to-zero, no FMA contraction: the
-kernels must reproduce IEEE binary32 results bit for bit.
+kernels must reproduce IEEE binary32 results bit for bit.  ``csrc/mxq_python.cpp``, which unpacks the arguments of the
+binding's inner-loop calls, is compiled against the installed torch to ``paper_2605_08565_b200/_native.so``.
 """
 from __future__ import annotations
 
@@ -19,6 +20,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmxq.so")
+NATIVE = os.path.join(HERE, "_native.so")
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -40,8 +42,33 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_native(force: bool = False, verbose: bool = False) -> str:
+    src = os.path.join(CSRC, "mxq_python.cpp")
+    if not force and not _stale(NATIVE, [src, os.path.join(os.path.dirname(HERE), "include", "mxq.h"), os.path.abspath(__file__)]):
+        return NATIVE
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+               os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
+    tmp = NATIVE + f".{os.getpid()}.tmp"
+    cmd = [shutil.which("g++") or "g++", "-O2", "-std=c++17", "-fPIC", "-shared",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(f"-I{d}" for d in include), src, "-o", tmp,
+           "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode != 0:
+        sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+    if r.returncode != 0:
+        raise RuntimeError("build of the extension module _native failed")
+    os.replace(tmp, NATIVE)
+    return NATIVE
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
+    build_native(force, verbose)
     headers = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
         [os.path.join(os.path.dirname(HERE), "include", "mxq.h"), os.path.abspath(__file__)]
     sources = sorted(glob.glob(os.path.join(CSRC, "*.cu")))

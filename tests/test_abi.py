@@ -84,3 +84,31 @@ def test_binding_refuses_cpu_tensors():
     x = torch.zeros(64)
     with pytest.raises(binding.MxqError):
         binding.quantize(x, 16, binding.MXQ_SF_UE4M3, binding.MXQ_ABSMAX)
+
+
+def test_native_calls_hand_on_what_they_do_not_know(lib):
+    """The extension module answers -1 to anything but contiguous CUDA tensors (or None), ints and floats, and the library's status
+    otherwise; the binding then raises what its ctypes call raises."""
+    import torch
+
+    from paper_2605_08565_b200 import binding
+    native = binding._native
+
+    class Stream:
+        cuda_stream = 0
+    s = Stream()
+    x = torch.zeros(64)
+    assert native.quantize_ex(x, 64, 16, 1, 0, 1.0, None, x, x, None, s) == -1       # a CPU tensor
+    assert native.segment_mse(None, 1, 1, 1, None, s) == 1                           # the library: a pointer is missing
+    assert native.segment_mse(None, 1, 1, 1.0, None, s) == -1
+    assert native.segment_mse(None, -1, 1, 1, None, s) == -1
+    assert native.segment_mse(None, 1, 1, 1, None, None) == -1                       # no tensor to take the stream from
+    assert native.segment_mse(None, 1, 1, 1) == -1
+    assert native.segment_mse(object(), 1, 1, 1, None, s) == -1
+    with pytest.raises(binding.MxqError, match="CUDA tensors only"):
+        binding.mxq_quantize_ex(x, 64, 16, 1, 0, 1.0, None, x, x, None)
+    with pytest.raises(binding.MxqError, match="status 1"):
+        binding.mxq_segment_mse(None, 1, 1, 1, None, stream=s)
+    with pytest.raises(binding.MxqError, match="status 2"):
+        binding.mxq_set_option(7, 1)
+    assert binding.mxq_get_option(binding.MXQ_OPT_BRUTE_PRUNE) == 0

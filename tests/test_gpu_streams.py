@@ -180,3 +180,39 @@ def test_entry_points_called_from_four_host_threads_at_once():
     fl.join()
     mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 0)
     assert not errors, errors
+
+
+def test_native_and_ctypes_calls_agree():
+    """The same call through the extension module (plain tensors, current or given stream) and through ctypes (a tensor subclass, an int
+    for the tensor scale), and the errors of both."""
+    class Sub(torch.Tensor):
+        pass
+
+    n = 64 * 100
+    x = inputs.normal(n, 3, 1.0, torch.bfloat16, "cuda")
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    outs = []
+    for kind in range(4):
+        codes, scales, sse = mxq.alloc_outputs(n, 16, x.device)
+        if kind == 0:
+            mxq.mxq_quantize_ex(x, n, 16, mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6, 1.0, None, codes, scales, sse)
+        elif kind == 1:
+            mxq.mxq_quantize_ex(x.as_subclass(Sub), n, 16, mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6, 1, None, codes, scales, sse)
+        elif kind == 2:
+            side.wait_stream(torch.cuda.current_stream())
+            mxq.mxq_quantize_ex(x, n, 16, mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6, 1.0, None, codes, scales, sse, stream=side)
+        else:
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(side):
+                mxq.mxq_quantize_ex(x, n, 16, mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6, 1.0, None, codes, scales, sse)
+        outs.append((codes, scales, sse))
+    torch.cuda.synchronize()
+    for o in outs[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(o, outs[0]))
+    with pytest.raises(mxq.MxqError, match="contiguous"):
+        mxq.mxq_quantize_ex(x[::2], n // 2, 16, mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6, 1.0, None, *outs[0])
+    with pytest.raises(mxq.MxqError, match="unsupported dtype"):
+        mxq.mxq_quantize_ex(x.half(), n, 16, mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6, 1.0, None, *outs[0])
+    with pytest.raises(mxq.MxqError, match="status 3"):
+        mxq.mxq_quantize_ex(x, n, 3, mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6, 1.0, None, *outs[0])
