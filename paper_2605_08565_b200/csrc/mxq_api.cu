@@ -60,7 +60,7 @@ static int quantize_common(const void* x, int dtype, size_t n, int block_size, i
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     QuantArgs a;
     a.x = x;
-    a.first_item = 0;
+    a.n_tail = a.tail_first = 0;
     a.global_scale = d_global_scale ? 1.0f : global_scale;
     a.d_global_scale = d_global_scale;
     a.codes = out_codes;
@@ -158,7 +158,7 @@ int mxq_quantize_batch(const mxq_tensor_desc* h_descs, const mxq_tensor_desc* d_
     QuantArgs a;
     a.x = nullptr;
     a.n_items = 0;
-    a.first_item = 0;
+    a.n_tail = a.tail_first = 0;
     a.global_scale = d_global_scale ? 1.0f : global_scale;
     a.d_global_scale = d_global_scale;
     a.codes = nullptr;

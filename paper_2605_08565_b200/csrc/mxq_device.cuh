@@ -44,15 +44,6 @@ __device__ __forceinline__ double cta_sum_fixed_order(double v, double* scratch)
     return t;
 }
 
-// Tail kernels (one warp): the binary64 sum of one SSE per lane, shuffle tree in fixed order, stored
-// as the call's partial number p.mse_first.  Every lane of the warp calls it (0 for an idle lane).
-__device__ __forceinline__ void warp_sum_to_partial(const QuantArgs& p, float sse) {
-    double v = (double)sse;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_down_sync(0xFFFFFFFFu, v, o));
-    if ((threadIdx.x & 31) == 0) p.mse_partials[p.mse_first] = v;
-}
-
 __host__ __device__ constexpr int num_codes(int fmt) { return fmt == kUE4M3 ? 127 : 255; }
 __host__ __device__ constexpr int elem_bytes(int dt) { return dt == kF32 ? 4 : 2; }
 

@@ -29,7 +29,7 @@ constexpr int kMaxBatch = 1024;   // tensors per multi-tensor launch
 struct QuantArgs {
     const void* x;
     size_t n_items;
-    size_t first_item;            // tail kernel only: index of the first block it handles
+    unsigned n_tail, tail_first;  // one-pass kernels: blocks past the last whole chunk, and the thread of the grid that takes the first of them
     float global_scale;
     const float* d_global_scale;  // overrides global_scale when non-NULL
     uint8_t* codes;
@@ -40,8 +40,8 @@ struct QuantArgs {
     void* xhat;                   // fused fake-quantize output (codes / scales may then be NULL), or NULL
     int xhat_dtype;
     // fused tensor-MSE partial sums (mxq_quantize_mse), or NULL: CTA i of the main kernel stores the
-    // binary64 sum of the block SSEs it produced in mse_partials[mse_first + i]; the tail kernel (one
-    // warp) stores its sum in mse_partials[mse_first]
+    // binary64 sum of the block SSEs it produced in mse_partials[mse_first + i] (a kernel launched before it may own those
+    // below mse_first)
     double* mse_partials;
     int mse_first;
     int* mse_n_partials;          // host: receives how many partials the launches of this call write (or NULL)
@@ -103,8 +103,6 @@ cudaError_t launch_brute_f32(const QuantArgs& a, int B, int fmt, cudaStream_t s)
 cudaError_t launch_brute_bf16(const QuantArgs& a, int B, int fmt, cudaStream_t s);
 cudaError_t launch_brute_pruned_f32(const QuantArgs& a, int B, int fmt, cudaStream_t s);
 cudaError_t launch_brute_pruned_bf16(const QuantArgs& a, int B, int fmt, cudaStream_t s);
-// Scalar kernel for the few blocks that do not fill a whole chunk (abs-max and 4-over-6 only).
-cudaError_t launch_quantize_tail(const QuantArgs& a, int dtype, int B, int fmt, bool dual, cudaStream_t s);
 
 cudaError_t launch_tensor_amax(const void* x, int dtype, size_t n, float* d_amax, float* d_g, cudaStream_t s);
 cudaError_t launch_tensor_mse(const float* d_sse, size_t n_blocks, size_t n, double* d_out, double* d_partials,

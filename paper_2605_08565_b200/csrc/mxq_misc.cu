@@ -180,41 +180,36 @@ cudaError_t launch_tensor_amax(const void* x, int dtype, size_t n, float* d_amax
 }
 
 // ------------------------------------------------------------------------------------------------
-// Tensor MSE: two-level tree of fixed shape in binary64.  Level 1: P = min(1024, ceil(nb/256))
+// Tensor MSE: two levels of fixed shape in binary64.  Level 1: P = min(1024, ceil(nb/256))
 // CTAs, CTA p sums the contiguous slice [p*L, (p+1)*L), L = ceil(nb/P): thread t adds elements
-// t, t+256, ... in order, then a shared-memory halving tree.  Level 2: one CTA, halving tree over
-// the P partials, divided by n.
+// t, t+256, ... in order, then cta_sum_fixed_order().  Level 2: one CTA of 256 threads, sum_partials() over the P partials, divided by
+// n (1024 threads and a halving tree of ten barriers: 0.5 us more; the last CTA of the first level in its place: 0.8 us more).
 // ------------------------------------------------------------------------------------------------
-template <int T>
-__device__ __forceinline__ double cta_tree_sum(double v, double* sh) {
-    sh[threadIdx.x] = v;
-    __syncthreads();
-#pragma unroll
-    for (int w = T / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] = __dadd_rn(sh[threadIdx.x], sh[threadIdx.x + w]);
-        __syncthreads();
-    }
-    return sh[0];
-}
-
 __global__ void __launch_bounds__(kThreads) k_mse_partial(const float* sse, size_t nb, size_t slice, double* partials) {
-    __shared__ double sh[kThreads];
+    __shared__ double scratch[kThreads / 32];
     wait_for_prior_grid();
     release_dependents();
     const size_t lo = (size_t)blockIdx.x * slice;
     const size_t hi = (lo + slice < nb) ? lo + slice : nb;
     double acc = 0.0;
     for (size_t i = lo + threadIdx.x; i < hi; i += kThreads) acc = __dadd_rn(acc, (double)__ldcs(sse + i));
-    const double total = cta_tree_sum<kThreads>(acc, sh);
+    const double total = cta_sum_fixed_order(acc, scratch);
     if (threadIdx.x == 0) partials[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(kMsePartials) k_mse_final(const double* partials, int n_partials, double n, double* out) {
-    __shared__ double sh[kMsePartials];
+// The second level of a tensor MSE: sum of n partials over a CTA of kThreads threads in a fixed order (thread t those at t, t + 256,
+// ..., then cta_sum_fixed_order()), valid in thread 0.  Read from L2: other CTAs have just written them.
+__device__ __forceinline__ double sum_partials(const double* partials, int n, double* scratch) {
+    double v = 0.0;
+    for (int i = threadIdx.x; i < n; i += kThreads) v = __dadd_rn(v, __ldcg(partials + i));
+    return cta_sum_fixed_order(v, scratch);
+}
+
+__global__ void __launch_bounds__(kThreads) k_mse_final(const double* partials, int n_partials, double n, double* out) {
+    __shared__ double scratch[kThreads / 32];
     wait_for_prior_grid();
     release_dependents();
-    const double v = (int)threadIdx.x < n_partials ? partials[threadIdx.x] : 0.0;
-    const double total = cta_tree_sum<kMsePartials>(v, sh);
+    const double total = sum_partials(partials, n_partials, scratch);
     if (threadIdx.x == 0) *out = __ddiv_rn(total, n);
 }
 
@@ -227,13 +222,11 @@ cudaError_t launch_tensor_mse(const float* d_sse, size_t n_blocks, size_t n, dou
     cudaError_t err = launch_pdl(k_mse_partial, (unsigned)P, kThreads, 0, s, d_sse, n_blocks, slice, d_partials);
     count_launch();
     if (err != cudaSuccess) return err;
-    err = launch_pdl(k_mse_final, 1u, (unsigned)kMsePartials, 0, s, (const double*)d_partials, (int)P, (double)n, d_out);
-    count_launch();
-    return err;
+    return launch_mse_final(d_partials, (int)P, n, d_out, s);
 }
 
 cudaError_t launch_mse_final(const double* d_partials, int n_partials, size_t n, double* d_out, cudaStream_t s) {
-    cudaError_t err = launch_pdl(k_mse_final, 1u, (unsigned)kMsePartials, 0, s, d_partials, n_partials, (double)n, d_out);
+    cudaError_t err = launch_pdl(k_mse_final, 1u, (unsigned)kThreads, 0, s, d_partials, n_partials, (double)n, d_out);
     count_launch();
     return err;
 }
@@ -353,87 +346,6 @@ cudaError_t launch_dequantize(const uint8_t* codes, const uint8_t* scales, size_
     else err = launch_pdl(k_dequantize<kBF16>, grid, kThreads, 0, s, codes, scales, n, log2B, fmt, g, d_g, out);
     count_launch();
     return err;
-}
-
-// ------------------------------------------------------------------------------------------------
-// Scalar abs-max / 4-over-6 for the blocks past the last whole per-thread chunk (block sizes up to
-// 16, fewer than 16 blocks).
-// Same arithmetic as the one-pass kernels, general quotient only.
-// ------------------------------------------------------------------------------------------------
-template <int FMT>
-__device__ float tail_eval(const float* v, int B, int c, float g, uint8_t* codes_out) {
-    const float D = __fmul_rn(scale_value(FMT, c), g);
-    float s = 0.0f;
-    for (int i = 0; i < B; i += 2) {
-        const float t0 = quotient_general(v[i], D), t1 = quotient_general(v[i + 1], D);
-        if (codes_out) codes_out[i >> 1] = (uint8_t)pack_e2m1x2(t0, t1);
-        const float2 q = round_e2m1x2(t0, t1);
-        const float e0 = __fmaf_rn(-q.x, D, v[i]);
-        s = __fmaf_rn(e0, e0, s);
-        const float e1 = __fmaf_rn(-q.y, D, v[i + 1]);
-        s = __fmaf_rn(e1, e1, s);
-    }
-    return s;
-}
-
-template <int FMT>
-__global__ void k_quantize_tail(QuantArgs p, int dtype, int B, int dual) {
-    const size_t b = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float my_sse = 0.0f;
-    if (b < p.n_items) {
-    const size_t blk = p.first_item + b;
-    const float g = p.d_global_scale ? *p.d_global_scale : p.global_scale;
-    float v[16];
-    float amax = 0.0f;
-    for (int i = 0; i < B; ++i) {
-        const size_t e = blk * B + i;
-        v[i] = dtype == kF32 ? static_cast<const float*>(p.x)[e]
-                             : __uint_as_float((uint32_t) static_cast<const uint16_t*>(p.x)[e] << 16);
-        amax = fmaxf(amax, fabsf(v[i]));
-    }
-    const bool pz = p.prevent_zero && FMT != kUE8M0;
-    const float u = __fdiv_rn(amax, g);
-    int c = (FMT == kUE8M0 && p.pow2_rule != kPow2Eq1) ? pow2_rule_code(u, p.pow2_rule) : round_scale<FMT>(__fdiv_rn(u, 6.0f));
-    if (pz) c = max(c, 1);
-    float s = tail_eval<FMT>(v, B, c, g, nullptr);
-    if (dual) {
-        int c4 = round_scale<FMT>(__fdiv_rn(u, 4.0f));
-        if (pz) c4 = max(c4, 1);
-        const float s4 = tail_eval<FMT>(v, B, c4, g, nullptr);
-        if (s4 < s) { s = s4; c = c4; }
-    }
-    uint8_t packed[8];
-    tail_eval<FMT>(v, B, c, g, packed);
-    if (p.codes)
-        for (int i = 0; i < B / 2; ++i) p.codes[blk * (B / 2) + i] = packed[i];
-    if (p.scales) p.scales[blk] = (uint8_t)c;
-    if (p.block_sse) p.block_sse[blk] = s;
-    if (p.xhat) {
-        const float D = __fmul_rn(scale_value(FMT, c), g);
-        for (int i = 0; i < B; ++i) {
-            float q[8];
-            unpack_e2m1x8((uint32_t)((packed[i >> 1] >> ((i & 1) ? 4 : 0)) & 15u), q);
-            const float xh = __fmul_rn(q[0], D);
-            if (p.xhat_dtype == kF32) static_cast<float*>(p.xhat)[blk * B + i] = xh;
-            else static_cast<__nv_bfloat16*>(p.xhat)[blk * B + i] = __float2bfloat16_rn(xh);
-        }
-    }
-    my_sse = s;
-    }
-    // fused tensor-MSE partial sum: the kernel is one warp, every lane takes part (idle lanes add 0)
-    if (p.mse_partials != nullptr) warp_sum_to_partial(p, my_sse);
-}
-
-cudaError_t launch_quantize_tail(const QuantArgs& a, int dtype, int B, int fmt, bool dual, cudaStream_t s) {
-    if (B > 16) return cudaErrorInvalidValue;
-    const unsigned grid = (unsigned)((a.n_items + 31) / 32);
-    switch (fmt) {
-    case kUE8M0: k_quantize_tail<kUE8M0><<<grid, 32, 0, s>>>(a, dtype, B, dual ? 1 : 0); break;
-    case kUE4M3: k_quantize_tail<kUE4M3><<<grid, 32, 0, s>>>(a, dtype, B, dual ? 1 : 0); break;
-    default: k_quantize_tail<kUE5M3><<<grid, 32, 0, s>>>(a, dtype, B, dual ? 1 : 0); break;
-    }
-    count_launch();
-    return cudaGetLastError();
 }
 
 }  // namespace mxq

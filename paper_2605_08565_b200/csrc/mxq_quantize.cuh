@@ -34,8 +34,8 @@
 // Variants of the chunk loop inside one kernel, chosen once per launch after the table is built: the
 // lean loop (see quantize_chunk) when no block can leave the shortcuts, the general loop otherwise.
 // Every thread also adds the SSEs of its blocks in binary64; a launch that was given a partial-sum
-// array (mxq_quantize_mse) ends with a fixed-order sum over the CTA.  The BATCH instantiation walks a
-// list of tensors in one launch (quantize_batch_body()).
+// array (mxq_quantize_mse) ends with a fixed-order sum over the CTA.  k_quantize_batch walks a
+// list of tensors in one launch.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -862,7 +862,67 @@ __device__ __forceinline__ void stage_chunk(uint32_t slot_addr, const void* src,
 // is faster with the whole block in registers (33.5 M bf16 elements: 0.775 against 0.711 of the copy bandwidth).
 __host__ __device__ constexpr bool long_block_path(int B, bool dual) { return B > 16 && !(dual && B == 32); }
 
-// Body of the multi-tensor kernel (see k_quantize, BATCH).
+// One block past the last whole chunk (a chunk of several blocks, B <= 16; fewer blocks than a chunk holds), by the general quotient; the
+// elements are read again for each candidate.  Out of line, to leave the registers of the kernel alone.  Returns its SSE.
+template <int DT, int B, int FMT, bool DUAL, bool FAKE>
+__device__ __noinline__ float quantize_tail_block(const QuantArgs& p, size_t blk, float g, int c_min, int pow2_rule) {
+    auto pair = [&](int i) {
+        float v[2];
+        load_elems<DT, 2>(p.x, blk * B + i, v);
+        return make_float2(v[0], v[1]);
+    };
+    float a = 0.0f;
+#pragma unroll 1
+    for (int i = 0; i < B; i += 2) {
+        const float2 v = pair(i);
+        a = fmaxf(a, fmaxf(fabsf(v.x), fabsf(v.y)));
+    }
+    auto evaluate = [&](int c, bool store) {
+        const float D = __fmul_rn(scale_value(FMT, c), g);
+        float s = 0.0f;
+#pragma unroll 1
+        for (int i = 0; i < B; i += 2) {
+            const float2 v = pair(i);
+            const float t0 = quotient_general(v.x, D), t1 = quotient_general(v.y, D);
+            const float2 q = round_e2m1x2(t0, t1);
+            const float e0 = __fmaf_rn(-q.x, D, v.x), e1 = __fmaf_rn(-q.y, D, v.y);
+            s = __fmaf_rn(e0, e0, s);
+            s = __fmaf_rn(e1, e1, s);
+            if (store) {
+                const size_t e = blk * B + i;
+                if constexpr (!FAKE) {
+                    p.codes[e / 2] = (uint8_t)pack_e2m1x2(t0, t1);
+                } else {   // x_hat = fl32(grid(code) * D), q with the sign of a zero
+                    const float x0 = __fmul_rn(q.x, D), x1 = __fmul_rn(q.y, D);
+                    if (p.xhat_dtype == kF32) {
+                        static_cast<float*>(p.xhat)[e] = x0;
+                        static_cast<float*>(p.xhat)[e + 1] = x1;
+                    } else {
+                        static_cast<__nv_bfloat16*>(p.xhat)[e] = __float2bfloat16_rn(x0);
+                        static_cast<__nv_bfloat16*>(p.xhat)[e + 1] = __float2bfloat16_rn(x1);
+                    }
+                }
+            }
+        }
+        return s;
+    };
+    const float u = __fdiv_rn(a, g);
+    int c = max(target6_code<FMT, true>(u, pow2_rule), c_min);
+    float s = DUAL ? evaluate(c, false) : 0.0f;
+    if constexpr (DUAL) {
+        const int c4 = max(round_scale<FMT>(__fmul_rn(u, 0.25f)), c_min);
+        const float s4 = evaluate(c4, false);
+        if (s4 < s) c = c4;
+    }
+    s = evaluate(c, true);
+    if constexpr (!FAKE) {
+        p.scales[blk] = (uint8_t)c;
+        if (p.block_sse) p.block_sse[blk] = s;
+    }
+    return s;
+}
+
+// Body of the multi-tensor kernel (k_quantize_batch).
 template <int DT, int B, int FMT, bool DUAL>
 __device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, QuantTables& T, uint4* ring) {
     using S = QuantShape<DT, B>;
@@ -1018,7 +1078,7 @@ __device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, QuantTab
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// BATCH: one launch over a list of tensors (same dtype, block size, format, recipe and tensor scale).
+// k_quantize_batch: one launch over a list of tensors (same dtype, block size, format, recipe and tensor scale).
 // The unit of distribution is a ROW of 32 consecutive chunks of one tensor (what a warp handles in one
 // trip); tensor t owns ceil(chunks_t / 32) rows of a common index space whose prefix sums every CTA
 // forms in shared memory; a warp walks rows first, first + 8 * gridDim.x, ... and moves its tensor
@@ -1029,15 +1089,28 @@ __device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, QuantTab
 // multi-tensor instantiations carry a cursor and a row loop on top of the chunk arithmetic; without a bound
 // some of them (B = 16) land a few registers above the 85 that three CTAs per SM allow and lose a third of
 // their loads in flight.
-__host__ __device__ constexpr int quantize_min_ctas(int B, bool batch) { return (batch && B >= 4 && B <= 16) ? 3 : 0; }
+__host__ __device__ constexpr int quantize_batch_min_ctas(int B) { return B >= 4 && B <= 16 ? 3 : 0; }
 
-template <int DT, int B, int FMT, bool DUAL, bool FAKE, bool BATCH = false>
-__global__ void __launch_bounds__(kThreads, quantize_min_ctas(B, BATCH)) k_quantize(QuantArgs p) {
+template <int DT, int B, int FMT, bool DUAL>
+__global__ void __launch_bounds__(kThreads, quantize_batch_min_ctas(B)) k_quantize_batch(QuantArgs p) {
     using S = QuantShape<DT, B>;
     static_assert(S::C == quantize_chunk_elems(DT, B), "host and kernel agree on the chunk size");
     extern __shared__ uint4 ring[];
     __shared__ QuantTables T;
-    if constexpr (!BATCH) {
+    wait_for_prior_grid();
+    release_dependents();
+    quantize_batch_body<DT, B, FMT, DUAL>(p, T, ring);
+}
+
+// TAIL: with blocks past the last whole chunk.  An instantiation of its own: the call that takes care of them costs the chunk loop of some
+// others registers (fp32, B = 16, abs-max, 16.8 M elements 15.7 -> 16.0 us without a single such block).
+template <int DT, int B, int FMT, bool DUAL, bool FAKE, bool TAIL>
+__global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ QuantArgs p) {
+    using S = QuantShape<DT, B>;
+    static_assert(S::C == quantize_chunk_elems(DT, B), "host and kernel agree on the chunk size");
+    extern __shared__ uint4 ring[];
+    __shared__ QuantTables T;
+    {
         // While the kernel before this one in the stream drains: ask L2 for this thread's first chunk.
         // A prefetch changes no architectural state and L2 is the point of coherence, so this is safe
         // even if that kernel is still writing x; the loads themselves come after the wait below.
@@ -1047,10 +1120,6 @@ __global__ void __launch_bounds__(kThreads, quantize_min_ctas(B, BATCH)) k_quant
     }
     wait_for_prior_grid();
     release_dependents();
-    if constexpr (BATCH) {
-        quantize_batch_body<DT, B, FMT, DUAL>(p, T, ring);
-        return;
-    }
     // request the first chunks before anything else: their latency hides behind the table build
     const size_t stride = (size_t)gridDim.x * kThreads;
     const int lane = threadIdx.x & 31;
@@ -1103,9 +1172,9 @@ __global__ void __launch_bounds__(kThreads, quantize_min_ctas(B, BATCH)) k_quant
     // Thread-private staging: a thread leaves when its chunks are done (no barrier follows).
     // Cooperative staging: the warp stays together, lanes past the end only take part in the copies.
     // (with fused MSE partial sums every thread stays for the CTA-wide sum at the end)
-    const bool has_work = (S::COOP ? wchunk0 : chunk) < p.n_items;
-    if (!has_work && (FAKE || p.mse_partials == nullptr)) return;
     double sse_sum = 0.0;   // binary64 sum of the SSEs of this thread's blocks, in the order it produced them
+    const bool has_work = (S::COOP ? wchunk0 : chunk) < p.n_items;
+    if (!has_work && (FAKE || p.mse_partials == nullptr) && !TAIL) return;
     // The chunk loop, instantiated with and without the lean per-block path (see quantize_chunk);
     // which one runs is the same for every thread of the launch.
     auto chunk_loop = [&](auto lean_tag) {
@@ -1154,6 +1223,13 @@ __global__ void __launch_bounds__(kThreads, quantize_min_ctas(B, BATCH)) k_quant
             chunk_loop(std::integral_constant<int, 0>{});
         }
     }
+    if constexpr (TAIL) {
+        // The blocks past the last whole chunk, one thread each: those that the round of the chunks would come to next.
+        const unsigned threads = gridDim.x * kThreads, t = blockIdx.x * kThreads + threadIdx.x;
+        const unsigned b = t >= p.tail_first ? t - p.tail_first : t + threads - p.tail_first;
+        if (b < p.n_tail)
+            sse_sum = __dadd_rn(sse_sum, (double)quantize_tail_block<DT, B, FMT, DUAL, FAKE>(p, p.n_items * S::NBC + b, k.g, k.c_min, k.pow2_rule));
+    }
     if constexpr (!FAKE) {
         if (p.mse_partials != nullptr) {   // launch-uniform: every thread of the CTA is here
             asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -1165,9 +1241,8 @@ __global__ void __launch_bounds__(kThreads, quantize_min_ctas(B, BATCH)) k_quant
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// Host side: pick the instantiation, launch a persistent grid over the whole chunks and hand the
-// blocks past the last whole chunk to the scalar tail kernel.
-template <int DT, int B, int FMT, bool DUAL, bool FAKE>
+// Host side: pick the instantiation and launch a persistent grid over the whole chunks and the blocks behind them.
+template <int DT, int B, int FMT, bool DUAL, bool FAKE, bool TAIL>
 static cudaError_t launch_quantize_inst(const QuantArgs& a, cudaStream_t stream) {
     using S = QuantShape<DT, B>;
     static std::atomic<int> ctas_per_sm[kMaxDevices];   // first-use cache; racing threads store the same value
@@ -1177,54 +1252,36 @@ static cudaError_t launch_quantize_inst(const QuantArgs& a, cudaStream_t stream)
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     int resident = ctas_per_sm[dev].load(std::memory_order_relaxed);
     if (resident == 0) {
-        err = cudaFuncSetAttribute(k_quantize<DT, B, FMT, DUAL, FAKE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        err = cudaFuncSetAttribute(k_quantize<DT, B, FMT, DUAL, FAKE, TAIL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)S::RING_BYTES);
         if (err != cudaSuccess) return err;
         int n = 0;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_quantize<DT, B, FMT, DUAL, FAKE>, kThreads, S::RING_BYTES);
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_quantize<DT, B, FMT, DUAL, FAKE, TAIL>, kThreads, S::RING_BYTES);
         if (err != cudaSuccess) return err;
         resident = n > 0 ? n : 1;
         ctas_per_sm[dev].store(resident, std::memory_order_relaxed);
     }
-    const size_t n_blocks = a.n_items;
-    const size_t n_chunks = n_blocks / S::NBC;
-    const size_t done = n_chunks * S::NBC;
-    // The blocks past the last whole chunk go to the one-warp tail kernel.  With fused MSE partial sums it
-    // runs first and owns partial 0; the CTAs of the main kernel own the partials from 1 on.
-    auto launch_tail = [&]() -> cudaError_t {
-        if (done == n_blocks) return cudaSuccess;
-        QuantArgs t = a;
-        t.first_item = done;
-        t.n_items = n_blocks - done;
-        t.mse_first = 0;
-        return launch_quantize_tail(t, DT, B, FMT, DUAL, stream);
-    };
-    if (a.mse_partials) {
-        err = launch_tail();
-        if (err != cudaSuccess) return err;
-    }
-    if (n_chunks > 0) {
-        QuantArgs m = a;
-        m.n_items = n_chunks;
-        m.mse_first = (done < n_blocks) ? 1 : 0;
-        const size_t want = (n_chunks + kThreads - 1) / kThreads;
-        size_t cap = (size_t)sm_count(dev) * (size_t)resident;
-        if (a.mse_partials && cap > (size_t)kMsePartials - 1) cap = kMsePartials - 1;
-        const unsigned grid = (unsigned)(want < cap ? want : cap);
-        err = launch_pdl(k_quantize<DT, B, FMT, DUAL, FAKE>, grid, kThreads, S::RING_BYTES, stream, m);
-        count_launch();
-        if (err != cudaSuccess) return err;
-        if (a.mse_n_partials) *a.mse_n_partials = (int)grid + m.mse_first;
-    } else if (a.mse_n_partials) {
-        *a.mse_n_partials = (done < n_blocks) ? 1 : 0;
-    }
-    if (!a.mse_partials) err = launch_tail();
+    QuantArgs m = a;
+    m.n_items = a.n_items / S::NBC;                          // whole chunks
+    m.n_tail = (unsigned)(a.n_items - m.n_items * S::NBC);      // the blocks behind them
+    const size_t want = (m.n_items + m.n_tail + kThreads - 1) / kThreads;
+    size_t cap = (size_t)sm_count(dev) * (size_t)resident;
+    if (a.mse_partials && cap > (size_t)kMsePartials) cap = kMsePartials;
+    const unsigned grid = (unsigned)(want < cap ? want : cap);
+    m.tail_first = (unsigned)(m.n_items % ((size_t)grid * kThreads));
+    err = launch_pdl(k_quantize<DT, B, FMT, DUAL, FAKE, TAIL>, grid, kThreads, S::RING_BYTES, stream, m);
+    count_launch();
+    if (err == cudaSuccess && a.mse_n_partials) *a.mse_n_partials = (int)grid;
     return err;
 }
 
 template <int DT, int B, int FMT, bool FAKE>
 static cudaError_t launch_quantize_kind(const QuantArgs& a, bool dual, cudaStream_t s) {
-    return dual ? launch_quantize_inst<DT, B, FMT, true, FAKE>(a, s) : launch_quantize_inst<DT, B, FMT, false, FAKE>(a, s);
+    using S = QuantShape<DT, B>;
+    if constexpr (S::NBC > 1) {
+        if (a.n_items % S::NBC != 0) return dual ? launch_quantize_inst<DT, B, FMT, true, FAKE, true>(a, s) : launch_quantize_inst<DT, B, FMT, false, FAKE, true>(a, s);
+    }
+    return dual ? launch_quantize_inst<DT, B, FMT, true, FAKE, false>(a, s) : launch_quantize_inst<DT, B, FMT, false, FAKE, false>(a, s);
 }
 
 template <int DT, int B, bool FAKE>
@@ -1260,11 +1317,11 @@ static cudaError_t launch_quantize_batch_inst(const QuantArgs& a, size_t total_r
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     int resident = ctas_per_sm[dev].load(std::memory_order_relaxed);
     if (resident == 0) {
-        err = cudaFuncSetAttribute(k_quantize<DT, B, FMT, DUAL, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        err = cudaFuncSetAttribute(k_quantize_batch<DT, B, FMT, DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)S::RING_BYTES);
         if (err != cudaSuccess) return err;
         int n = 0;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_quantize<DT, B, FMT, DUAL, false, true>, kThreads, S::RING_BYTES);
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_quantize_batch<DT, B, FMT, DUAL>, kThreads, S::RING_BYTES);
         if (err != cudaSuccess) return err;
         resident = n > 0 ? n : 1;
         ctas_per_sm[dev].store(resident, std::memory_order_relaxed);
@@ -1272,7 +1329,7 @@ static cudaError_t launch_quantize_batch_inst(const QuantArgs& a, size_t total_r
     const size_t want = (total_rows + kThreads / 32 - 1) / (kThreads / 32);
     const size_t cap = (size_t)sm_count(dev) * (size_t)resident;
     const unsigned grid = (unsigned)(want < cap ? want : cap);
-    err = launch_pdl(k_quantize<DT, B, FMT, DUAL, false, true>, grid, kThreads, S::RING_BYTES, stream, a);
+    err = launch_pdl(k_quantize_batch<DT, B, FMT, DUAL>, grid, kThreads, S::RING_BYTES, stream, a);
     count_launch();
     return err;
 }
