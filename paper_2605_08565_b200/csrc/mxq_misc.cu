@@ -3,12 +3,43 @@
 // that do not fill a whole per-thread chunk.
 #include <cuda_bf16.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "mxq_device.cuh"
 #include "mxq_internal.h"
 
 namespace mxq {
+
+// ------------------------------------------------------------------------------------------------
+// Slots in which the CTAs of a launch leave their maximum and count themselves, so that no kernel has to initialise those words: zero
+// between launches, the last CTA puts them back.  A ring of them per device, 2 MB that every GPU which loads the library holds until
+// exit, handed out in turn: a slot comes round again 2^18 calls later, where a stream holds about a thousand launches in flight.
+// ------------------------------------------------------------------------------------------------
+struct DoneSlot {
+    unsigned arrived, max_bits;
+};
+constexpr unsigned kDoneSlots = 1u << 18;
+static __device__ DoneSlot g_done_slots[kDoneSlots];
+
+// A slot for one launch on the current device, or NULL while the stream is being captured (a graph replays with the same slot at any
+// later time, beside launches that were given it meanwhile): the launch then takes the route with the initialising kernel.
+static DoneSlot* done_slot(cudaStream_t s) {
+    static std::atomic<DoneSlot*> ring_of_device[kMaxDevices];   // first-use cache; racing threads store the same value
+    static std::atomic<unsigned> next{0};
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return nullptr;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    DoneSlot* ring = ring_of_device[dev].load(std::memory_order_relaxed);
+    if (ring == nullptr) {
+        void* p = nullptr;
+        if (cudaGetSymbolAddress(&p, g_done_slots) != cudaSuccess) return nullptr;
+        ring = static_cast<DoneSlot*>(p);
+        ring_of_device[dev].store(ring, std::memory_order_relaxed);
+    }
+    return ring + next.fetch_add(1, std::memory_order_relaxed) % kDoneSlots;
+}
 
 // ------------------------------------------------------------------------------------------------
 // Tensor abs-max: max is exact and order-independent, so the cross-CTA step is an integer
@@ -20,8 +51,8 @@ __device__ __forceinline__ float warp_max(float m) {
     return m;
 }
 
-// Zeroes the running maximum and, when a tensor scale is wanted, the word that first counts the CTAs
-// that have finished and then receives the scale.
+// Without a slot (under capture): zeroes the running maximum and, when a tensor scale is wanted, the word that first counts the
+// CTAs that have finished and then receives the scale.
 __global__ void k_amax_init(uint32_t* amax_bits, uint32_t* g_word) {
     wait_for_prior_grid();
     release_dependents();
@@ -29,14 +60,17 @@ __global__ void k_amax_init(uint32_t* amax_bits, uint32_t* g_word) {
     if (g_word) *g_word = 0u;
 }
 
-// One CTA reads tiles of U x 256 sixteen-byte vectors (U independent loads per thread in flight).  The
-// last CTA to finish (a count in g_word) turns the maximum into g = amax / (6 * 448), the tensor
-// maximum mapped to the top of FP4 times the top of E4M3, and stores it over the count.  Loads are
+__device__ __forceinline__ float scale_of_amax(float a) { return (a > 0.0f && a <= 3.402823466e38f) ? __fdiv_rn(a, 2688.0f) : 1.0f; }
+
+// One CTA reads tiles of U x 256 sixteen-byte vectors (U independent loads per thread in flight).  The running maximum and the
+// count of CTAs that have finished lie in the launch's slot, or, without one, in out_bits and g_word.  The
+// last CTA to finish turns the maximum into g = amax / (6 * 448), the tensor
+// maximum mapped to the top of FP4 times the top of E4M3, and stores both.  Loads are
 // streaming (evict-first): reading with the default policy, so that the quantize pass that follows finds
 // the tensor in L2, was measured on 33 to 117 MB tensors and gains nothing (that pass is not DRAM-bound
 // enough at those sizes), while it slows this kernel by 5 %.
 template <int DT>
-__global__ void __launch_bounds__(kThreads) k_tensor_amax(const void* x, size_t n, uint32_t* out_bits, uint32_t* g_word) {
+__global__ void __launch_bounds__(kThreads) k_tensor_amax(const void* x, size_t n, uint32_t* out_bits, uint32_t* g_word, DoneSlot* done) {
     constexpr int VEC = 16 / elem_bytes(DT);
     constexpr int U = 4;
     const size_t n_vec = n / VEC;
@@ -85,13 +119,19 @@ __global__ void __launch_bounds__(kThreads) k_tensor_amax(const void* x, size_t 
         m = threadIdx.x < kThreads / 32 ? warp_m[threadIdx.x] : 0.0f;
         m = warp_max(m);
         if (threadIdx.x == 0) {
-            atomicMax(out_bits, __float_as_uint(m));
-            if (g_word) {
+            unsigned* const run = done ? &done->max_bits : out_bits;
+            unsigned* const count = done ? &done->arrived : g_word;
+            atomicMax(run, __float_as_uint(m));
+            if (count) {
                 __threadfence();
-                if (atomicAdd(g_word, 1u) == gridDim.x - 1) {   // every CTA's maximum is in: this one writes the scale
+                if (atomicAdd(count, 1u) == gridDim.x - 1) {   // every CTA's maximum is in
                     __threadfence();
-                    const float a = __uint_as_float(atomicMax(out_bits, 0u));
-                    *reinterpret_cast<float*>(g_word) = (a > 0.0f && a <= 3.402823466e38f) ? __fdiv_rn(a, 2688.0f) : 1.0f;
+                    const uint32_t bits = done ? atomicExch(run, 0u) : atomicMax(run, 0u);
+                    if (done) {
+                        done->arrived = 0;
+                        *out_bits = bits;
+                    }
+                    if (g_word) *reinterpret_cast<float*>(g_word) = scale_of_amax(__uint_as_float(bits));
                 }
             }
         }
@@ -148,7 +188,7 @@ __global__ void __launch_bounds__(kOneCtaThreads) k_tensor_amax_one(const void* 
         m = warp_max(warp_m[threadIdx.x]);
         if (threadIdx.x == 0) {
             *out = m;
-            if (out_g) *out_g = (m > 0.0f && m <= 3.402823466e38f) ? __fdiv_rn(m, 2688.0f) : 1.0f;
+            if (out_g) *out_g = scale_of_amax(m);
         }
     }
 }
@@ -162,9 +202,13 @@ cudaError_t launch_tensor_amax(const void* x, int dtype, size_t n, float* d_amax
     }
     uint32_t* amax_bits = reinterpret_cast<uint32_t*>(d_amax);
     uint32_t* g_word = reinterpret_cast<uint32_t*>(d_g);
-    cudaError_t err = launch_pdl(k_amax_init, 1u, 1u, 0, s, amax_bits, g_word);
-    count_launch();
-    if (err != cudaSuccess) return err;
+    DoneSlot* const done = done_slot(s);
+    cudaError_t err = cudaSuccess;
+    if (!done) {
+        err = launch_pdl(k_amax_init, 1u, 1u, 0, s, amax_bits, g_word);
+        count_launch();
+        if (err != cudaSuccess) return err;
+    }
     int dev = 0;
     err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
@@ -173,8 +217,8 @@ cudaError_t launch_tensor_amax(const void* x, int dtype, size_t n, float* d_amax
     if (want == 0) want = 1;
     const size_t cap = (size_t)sm_count(dev) * 8;
     const unsigned grid = (unsigned)(want < cap ? want : cap);
-    if (dtype == kF32) err = launch_pdl(k_tensor_amax<kF32>, grid, (unsigned)kThreads, 0, s, x, n, amax_bits, g_word);
-    else err = launch_pdl(k_tensor_amax<kBF16>, grid, (unsigned)kThreads, 0, s, x, n, amax_bits, g_word);
+    if (dtype == kF32) err = launch_pdl(k_tensor_amax<kF32>, grid, (unsigned)kThreads, 0, s, x, n, amax_bits, g_word, done);
+    else err = launch_pdl(k_tensor_amax<kBF16>, grid, (unsigned)kThreads, 0, s, x, n, amax_bits, g_word, done);
     count_launch();
     return err;
 }

@@ -216,3 +216,38 @@ def test_native_and_ctypes_calls_agree():
         mxq.mxq_quantize_ex(x.half(), n, 16, mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6, 1.0, None, *outs[0])
     with pytest.raises(mxq.MxqError, match="status 3"):
         mxq.mxq_quantize_ex(x, n, 3, mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6, 1.0, None, *outs[0])
+
+
+def test_tensor_amax_on_many_streams_at_once_and_in_a_graph():
+    """Beyond 256 KB the CTAs of a launch meet in a slot of their own: launches on several streams at once, their results and those of
+    a graph that holds the same calls (which take the route without a slot), replayed beside direct calls."""
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    sizes = [131073, 200001, 1 << 18, (1 << 20) + 5]
+    xs = [[inputs.normal(n, 31 * k + j, 2.0 ** (j - 2), torch.float32, "cuda") for j in range(6)] for k, n in enumerate(sizes)]
+    want = [[np.float32(x.abs().max().item()) for x in row] for row in xs]
+    out = torch.zeros(4, 2, 6, device="cuda")
+    torch.cuda.synchronize()
+    graphs = []
+    for st, row, o in zip(streams, xs, out):
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            for j, x in enumerate(row):
+                mxq.mxq_tensor_amax(x, x.numel(), o[0, j], o[1, j])
+        graphs.append(g)
+    for trip in range(30):
+        out.zero_()
+        torch.cuda.synchronize()
+        for k, (st, row, o) in enumerate(zip(streams, xs, out)):
+            with torch.cuda.stream(st):
+                if (trip + k) % 3 == 0:
+                    graphs[k].replay()
+                else:
+                    for j, x in enumerate(row):
+                        mxq.mxq_tensor_amax(x, x.numel(), o[0, j], o[1, j] if (trip + j) % 2 else None)
+        torch.cuda.synchronize()
+        got = out.cpu().numpy()
+        for k, row in enumerate(want):
+            for j, a in enumerate(row):
+                assert got[k, 0, j] == a
+                if (trip + k) % 3 == 0 or (trip + j) % 2:
+                    assert got[k, 1, j] == a / np.float32(2688.0)
