@@ -493,6 +493,92 @@ __device__ __forceinline__ int target6_code(float u, int pow2_rule) {
     return round_scale<FMT>(EXACT ? __fdiv_rn(u, 6.0f) : div6_fast(u));
 }
 
+// What a chunk leaves for the fake-quantize store.
+template <int DT, int B>
+struct FakeChunk {
+    using S = QuantShape<DT, B>;
+    uint32_t codes[S::C / 8];
+    uint32_t scales[(S::NBC + 3) / 4];
+    float D[S::NBC];
+};
+
+// Fake-quantize: x_hat = fl32(grid(code) * D), optionally rounded to bf16, of the warp's n_valid chunks from chunk wchunk on.  A
+// thread's own x_hat is a run of 32 to 256 bytes; stored by the thread that made it, every 16-byte store of a warp would touch 16 or
+// 32 cache lines and write half sectors (33.5 M bf16 elements, B = 32, UE8M0, bf16 out: 26.7 us, here 22.2;
+// 16.8 M bf16 elements, B = 8, 4-over-6, fp32 out 33.4, here 17.7).  So the packed codes and the decode scales (for bf16 blocks of 2, where these
+// would not fit, the scale bytes) go through the ring slot that the chunk came from, and the warp forms and stores 512 contiguous bytes at a time.
+// Every lane of the warp calls it.
+template <int DT, int B>
+__device__ __forceinline__ void store_fake_chunks(const QuantArgs& p, const QuantTables& T, const FakeChunk<DT, B>& f, size_t wchunk, int n_valid,
+                                                  uint4* slot_warp, int lane) {
+    using S = QuantShape<DT, B>;
+    constexpr int ROW = 512, ROW_STRIDE = kThreads * 16;   // a row of the slot: 16 bytes per lane of the warp
+    constexpr int CODE_ROWS = (32 * S::C / 2 + ROW - 1) / ROW;
+    constexpr bool BY_CODE = (B == 2 && DT == kBF16);
+    constexpr int D_BYTES = BY_CODE ? S::NBC : 4 * S::NBC;   // per lane
+    static_assert(CODE_ROWS + (32 * D_BYTES + ROW - 1) / ROW <= S::PIECES, "fits the slot");
+    unsigned char* const base = reinterpret_cast<unsigned char*>(slot_warp);
+    auto at = [&](int o) { return base + o / ROW * ROW_STRIDE + o % ROW; };
+    auto dat = [&](int o) { return at(CODE_ROWS * ROW + o); };
+    __syncwarp();   // every lane has read its chunk
+    if constexpr (S::C / 2 == 8) *reinterpret_cast<uint2*>(at(lane * 8)) = make_uint2(f.codes[0], f.codes[1]);
+    else {
+#pragma unroll
+        for (int i = 0; i < S::C / 32; ++i)
+            *reinterpret_cast<uint4*>(at(lane * (S::C / 2) + 16 * i)) = make_uint4(f.codes[4 * i], f.codes[4 * i + 1], f.codes[4 * i + 2], f.codes[4 * i + 3]);
+    }
+    if constexpr (BY_CODE) {
+#pragma unroll
+        for (int i = 0; i < S::NBC / 4; ++i) *reinterpret_cast<uint32_t*>(dat(lane * D_BYTES + 4 * i)) = f.scales[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < S::NBC; ++i) *reinterpret_cast<float*>(dat(lane * D_BYTES + 4 * i)) = f.D[i];
+    }
+    __syncwarp();
+    auto store_units = [&](auto bf16_tag) {
+        constexpr bool OUT_BF16 = decltype(bf16_tag)::value;
+        constexpr int E = OUT_BF16 ? 8 : 4;        // elements of a 16-byte unit
+        const int units = n_valid * (S::C / E);
+#pragma unroll 4
+        for (int i = 0; i < S::C / E; ++i) {
+            const int u = i * 32 + lane;
+            if (u >= units) break;
+            uint32_t w;
+            if constexpr (OUT_BF16) w = *reinterpret_cast<const uint32_t*>(at(u * 4));
+            else w = *reinterpret_cast<const uint16_t*>(at(u * 2));
+            float q[8];
+            unpack_e2m1x8(w, q);
+            float xh[E];
+#pragma unroll
+            for (int e = 0; e < E; e += (B < E ? B : E)) {
+                const int blk = (u * E + e) / B;
+                float D;
+                if constexpr (BY_CODE) D = T.E[*dat(blk)].x;
+                else D = *reinterpret_cast<const float*>(dat(blk * 4));
+#pragma unroll
+                for (int j = 0; j < (B < E ? B : E); ++j) xh[e + j] = __fmul_rn(q[e + j], D);
+            }
+            const size_t e0 = wchunk * S::C + (size_t)u * E;
+            if constexpr (OUT_BF16) {
+                uint32_t h[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const __nv_bfloat162 b2 = __floats2bfloat162_rn(xh[2 * j], xh[2 * j + 1]);
+                    h[j] = *reinterpret_cast<const uint32_t*>(&b2);
+                }
+                store_bytes<16>(static_cast<__nv_bfloat16*>(p.xhat) + e0, h);
+            } else {
+                uint32_t o[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) o[j] = __float_as_uint(xh[j]);
+                store_bytes<16>(static_cast<float*>(p.xhat) + e0, o);
+            }
+        }
+    };
+    if (p.xhat_dtype == kBF16) store_units(std::integral_constant<bool, true>{});
+    else store_units(std::integral_constant<bool, false>{});
+}
+
 // LEAN == 2: the same loop under a tensor scale, see lean_scaled_allowed(): the block maximum is divided by g
 // first (corrected quotient), the residual is formed in binary32.
 // LEAN == 1 (launch-uniform; bf16 input, FP8 scale format, no tensor scale, every decode scale of the
@@ -508,7 +594,7 @@ __device__ __forceinline__ int target6_code(float u, int pow2_rule) {
 // (4 eps / 6 and 4 eps / 4 round to code 1; anything below rounds to 0 or 1, anything above to >= 1).
 template <int DT, int B, int FMT, bool DUAL, bool FAKE, int LEAN>
 __device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const QuantTables& T, const QuantConsts& k,
-                                               size_t chunk, const uint32_t* raw, double& sse_sum) {
+                                               size_t chunk, const uint32_t* raw, double& sse_sum, FakeChunk<DT, B>* fake) {
     static_assert(!LEAN || (DT == kBF16 && FMT != kUE8M0), "lean path: bf16 input, FP8 scale formats");
     using S = QuantShape<DT, B>;
     constexpr int NBG = S::NBG;
@@ -638,27 +724,9 @@ __device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const QuantTa
                 pk[0] = (pk4[0] & take) | (pk[0] & ~take);
             }
         }
-        if constexpr (FAKE) {   // fused fake-quantize: x_hat = fl32(grid(code) * D), optionally rounded to bf16
-            const size_t e0 = chunk * S::C + (size_t)gi * S::GE;
+        if constexpr (FAKE) {
 #pragma unroll
-            for (int w8 = 0; w8 < S::GE / 8; ++w8) {
-                float q[8];
-                unpack_e2m1x8(pk[w8], q);
-                uint32_t o[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(__fmul_rn(q[i], Dw[(w8 * 8 + i) / B]));
-                if (p.xhat_dtype == kF32) {
-                    store_bytes<32>(static_cast<float*>(p.xhat) + e0 + 8 * w8, o);
-                } else {
-                    uint32_t h[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(o[2 * i]), __uint_as_float(o[2 * i + 1]));
-                        h[i] = *reinterpret_cast<const uint32_t*>(&b2);
-                    }
-                    store_bytes<16>(static_cast<__nv_bfloat16*>(p.xhat) + e0 + 8 * w8, h);
-                }
-            }
+            for (int j = 0; j < NBG; ++j) fake->D[gi * NBG + j] = Dw[j];
         }
 #pragma unroll
         for (int i = 0; i < S::GE / 8; ++i) packed[gi * (S::GE / 8) + i] = pk[i];
@@ -670,7 +738,13 @@ __device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const QuantTa
             if constexpr (!FAKE) sse_sum = __dadd_rn(sse_sum, (double)sse[j]);
         }
     }
-    if constexpr (FAKE) return;
+    if constexpr (FAKE) {
+#pragma unroll
+        for (int i = 0; i < S::C / 8; ++i) fake->codes[i] = packed[i];
+#pragma unroll
+        for (int i = 0; i < (S::NBC + 3) / 4; ++i) fake->scales[i] = sc[i];
+        return;
+    }
     store_bytes<S::C / 2>(p.codes + chunk * (S::C / 2), packed);
     store_bytes<S::NBC>(p.scales + chunk * S::NBC, sc);
     if (p.block_sse) store_bytes<4 * S::NBC>(p.block_sse + chunk * S::NBC, sw);
@@ -698,7 +772,8 @@ __device__ __forceinline__ uint32_t absmax_bf16x2(uint32_t a, uint32_t b) {
 // Only one part is live in registers at a time, which keeps as many CTAs resident as for B = 16.
 template <int DT, int B, int FMT, bool DUAL, bool FAKE>
 __device__ __forceinline__ void quantize_long_block(const QuantArgs& p, const QuantTables& T, const QuantConsts& k,
-                                                    size_t chunk, const uint4* slot_warp, int lane, double& sse_sum) {
+                                                    size_t chunk, const uint4* slot_warp, int lane, double& sse_sum,
+                                                    FakeChunk<DT, B>* fake) {
     using S = QuantShape<DT, B>;
     static_assert(S::C == B && S::NBC == 1, "one block per chunk");
     constexpr int SG = 16;                        // elements per part
@@ -790,27 +865,11 @@ __device__ __forceinline__ void quantize_long_block(const QuantArgs& p, const Qu
 #pragma unroll
         for (int i = 0; i < B / 8; ++i) pk[i] = take ? pk4[i] : pk[i];
     }
-    if constexpr (FAKE) {   // fused fake-quantize: x_hat = fl32(grid(code) * D), optionally rounded to bf16
-        const size_t e0 = chunk * B;
+    if constexpr (FAKE) {
 #pragma unroll
-        for (int w8 = 0; w8 < B / 8; ++w8) {
-            float q[8];
-            unpack_e2m1x8(pk[w8], q);
-            uint32_t o[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(__fmul_rn(q[i], Dw));
-            if (p.xhat_dtype == kF32) {
-                store_bytes<32>(static_cast<float*>(p.xhat) + e0 + 8 * w8, o);
-            } else {
-                uint32_t h[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(o[2 * i]), __uint_as_float(o[2 * i + 1]));
-                    h[i] = *reinterpret_cast<const uint32_t*>(&b2);
-                }
-                store_bytes<16>(static_cast<__nv_bfloat16*>(p.xhat) + e0 + 8 * w8, h);
-            }
-        }
+        for (int i = 0; i < B / 8; ++i) fake->codes[i] = pk[i];
+        fake->scales[0] = (uint32_t)c6;
+        fake->D[0] = Dw;
         return;
     }
     store_bytes<B / 2>(p.codes + chunk * (B / 2), pk);
@@ -1055,7 +1114,7 @@ __device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, QuantTab
             const size_t chunk = (size_t)(row - cur_c.first) * 32 + lane;
             if (chunk >= cur_c.n_chunks) continue;      // a lane past the end of the tensor's last row
             if constexpr (long_block_path(B, DUAL)) {
-                quantize_long_block<DT, B, FMT, DUAL, false>(pl, T, k, chunk, slot_warp, lane, unused_sum);
+                quantize_long_block<DT, B, FMT, DUAL, false>(pl, T, k, chunk, slot_warp, lane, unused_sum, nullptr);
             } else {
                 uint32_t raw[S::PIECES * 4];
 #pragma unroll
@@ -1063,7 +1122,7 @@ __device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, QuantTab
                     const uint4 w = slot_warp[ring_index<S::COOP>(q, lane)];
                     raw[4 * q + 0] = w.x; raw[4 * q + 1] = w.y; raw[4 * q + 2] = w.z; raw[4 * q + 3] = w.w;
                 }
-                quantize_chunk<DT, B, FMT, DUAL, false, LEAN>(pl, T, k, chunk, raw, unused_sum);
+                quantize_chunk<DT, B, FMT, DUAL, false, LEAN>(pl, T, k, chunk, raw, unused_sum, nullptr);
             }
         }
     };
@@ -1173,7 +1232,8 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
     // Cooperative staging: the warp stays together, lanes past the end only take part in the copies.
     // (with fused MSE partial sums every thread stays for the CTA-wide sum at the end)
     double sse_sum = 0.0;   // binary64 sum of the SSEs of this thread's blocks, in the order it produced them
-    const bool has_work = (S::COOP ? wchunk0 : chunk) < p.n_items;
+    constexpr bool TOGETHER = S::COOP || FAKE;   // the warp stays together through the loop
+    const bool has_work = (TOGETHER ? wchunk0 : chunk) < p.n_items;
     if (!has_work && (FAKE || p.mse_partials == nullptr) && !TAIL) return;
     // The chunk loop, instantiated with and without the lean per-block path (see quantize_chunk);
     // which one runs is the same for every thread of the launch.
@@ -1182,13 +1242,13 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
         int slot = 0;                      // slot holding `chunk`
         int fill = DIST % S::SLOTS;        // slot that the next request goes to
         size_t ahead = (S::COOP ? wchunk0 : chunk) + (size_t)DIST * stride;
-        for (size_t lead = S::COOP ? wchunk0 : chunk; lead < p.n_items; lead += stride, chunk += stride) {
+        for (size_t lead = TOGETHER ? wchunk0 : chunk; lead < p.n_items; lead += stride, chunk += stride) {
             // all but the DIST - 1 most recent groups are complete: this thread's copies for `chunk` have landed
             asm volatile("cp.async.wait_group %0;" ::"n"(DIST - 1) : "memory");
             // cooperative staging: so have the other lanes' copies, and every lane is done reading the
-            // slot that the next request overwrites
-            if constexpr (S::COOP) __syncwarp();
-            const uint4* slot_warp = ring + (size_t)slot * (S::PIECES * kThreads) + (threadIdx.x - lane);
+            // slot that the next request overwrites (fake-quantize reads it across lanes too)
+            if constexpr (TOGETHER) __syncwarp();
+            uint4* const slot_warp = ring + (size_t)slot * (S::PIECES * kThreads) + (threadIdx.x - lane);
             // the slot read one trip ago is free again (its words were consumed by the arithmetic of
             // that trip): request the chunk DIST trips ahead into it.  The slot of the current chunk
             // is not requested into before the next trip, so it may be read throughout this one.
@@ -1197,19 +1257,26 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
             ahead += stride;
             slot = (slot + 1 == S::SLOTS) ? 0 : slot + 1;
             fill = (fill + 1 == S::SLOTS) ? 0 : fill + 1;
-            if (S::COOP && chunk >= p.n_items) continue;   // a lane past the end (the warp's last trip)
+            if (S::COOP && !FAKE && chunk >= p.n_items) continue;   // a lane past the end (the warp's last trip)
+            FakeChunk<DT, B> fake;
             // blocks longer than 16 elements go part by part, except 4-over-6 at B = 32, which measured
             // slightly faster with the whole block in registers
-            if constexpr (long_block_path(B, DUAL)) {
-                quantize_long_block<DT, B, FMT, DUAL, FAKE>(p, T, k, chunk, slot_warp, lane, sse_sum);
-            } else {
-                uint32_t raw[S::PIECES * 4];
+            if (!FAKE || chunk < p.n_items) {
+                if constexpr (long_block_path(B, DUAL)) {
+                    quantize_long_block<DT, B, FMT, DUAL, FAKE>(p, T, k, chunk, slot_warp, lane, sse_sum, &fake);
+                } else {
+                    uint32_t raw[S::PIECES * 4];
 #pragma unroll
-                for (int q = 0; q < S::PIECES; ++q) {
-                    const uint4 w = slot_warp[ring_index<S::COOP>(q, lane)];
-                    raw[4 * q + 0] = w.x; raw[4 * q + 1] = w.y; raw[4 * q + 2] = w.z; raw[4 * q + 3] = w.w;
+                    for (int q = 0; q < S::PIECES; ++q) {
+                        const uint4 w = slot_warp[ring_index<S::COOP>(q, lane)];
+                        raw[4 * q + 0] = w.x; raw[4 * q + 1] = w.y; raw[4 * q + 2] = w.z; raw[4 * q + 3] = w.w;
+                    }
+                    quantize_chunk<DT, B, FMT, DUAL, FAKE, LEAN>(p, T, k, chunk, raw, sse_sum, &fake);
                 }
-                quantize_chunk<DT, B, FMT, DUAL, FAKE, LEAN>(p, T, k, chunk, raw, sse_sum);
+            }
+            if constexpr (FAKE) {
+                const size_t left = p.n_items - lead;
+                store_fake_chunks<DT, B>(p, T, fake, lead, left < 32 ? (int)left : 32, slot_warp, lane);
             }
         }
     };
