@@ -58,17 +58,20 @@ __global__ void __launch_bounds__(kThreads) k_block_clip_sse(const void* x, size
     release_dependents();
     const float gs = d_g ? *d_g : g;
     const size_t stride = (size_t)gridDim.x * kThreads;
-    auto do_blocks = [&](auto count, size_t b) {   // blocks b, b + stride, ...: all loads first
+    // From the end of the tensor to its beginning: the pass that quantized it has left the end of it in L2 (scoring of 60.4 M fp32 elements,
+    // B = 8, quantization included: 129.2 -> 127.0 us).
+    const size_t last = n_blocks - 1;
+    auto do_blocks = [&](auto count, size_t b) {   // blocks last - b, last - b - stride, ...: all loads first
         constexpr int U = decltype(count)::value;
         float v[U][B];
         int c[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            load_elems<DT, B>(x, (b + u * stride) * B, v[u]);      // vector loads: a block is 4 .. 256 contiguous bytes
-            c[u] = scales[b + u * stride];
+            load_elems<DT, B>(x, (last - (b + u * stride)) * B, v[u]);      // vector loads: a block is 4 .. 256 contiguous bytes
+            c[u] = scales[last - (b + u * stride)];
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u) out[b + u * stride] = clip_sse<B>(v[u], c[u], fmt, gs);
+        for (int u = 0; u < U; ++u) out[last - (b + u * stride)] = clip_sse<B>(v[u], c[u], fmt, gs);
     };
     size_t b = (size_t)blockIdx.x * kThreads + threadIdx.x;
     if constexpr (B <= 16) {

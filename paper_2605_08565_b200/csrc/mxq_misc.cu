@@ -295,11 +295,6 @@ __global__ void __launch_bounds__(kThreads) k_dequantize(const uint8_t* codes, c
                                                          int log2B, int fmt, float g_host, const float* d_g, void* out) {
     wait_for_prior_grid();
     release_dependents();
-    const float g = d_g ? *d_g : g_host;   // device-resident tensor scale (written by an earlier kernel of the stream)
-    // decode scales of all 256 codes, one per thread: a table read replaces a dozen instructions per unit
-    __shared__ float Dtab[256];
-    Dtab[threadIdx.x] = decode_scale(fmt, (int)threadIdx.x, g);
-    __syncthreads();
     constexpr int E = (ODT == kF32) ? 4 : 8;      // elements per unit
     constexpr int LOG2E = (ODT == kF32) ? 2 : 3;
     constexpr int U = 4;
@@ -326,6 +321,11 @@ __global__ void __launch_bounds__(kThreads) k_dequantize(const uint8_t* codes, c
     size_t base = (size_t)blockIdx.x * (U * kThreads) + threadIdx.x;
     uint32_t w[U], sc[U];
     load_trip(base, w, sc);
+    // decode scales of all 256 codes, one per thread, while the first loads are on their way: a table read replaces a dozen instructions per unit
+    const float g = d_g ? *d_g : g_host;   // device-resident tensor scale (written by an earlier kernel of the stream)
+    __shared__ float Dtab[256];
+    Dtab[threadIdx.x] = decode_scale(fmt, (int)threadIdx.x, g);
+    __syncthreads();
     for (; base < n_units; base += stride * U) {
         uint32_t wn[U], scn[U];
         load_trip(base + stride * U, wn, scn);
