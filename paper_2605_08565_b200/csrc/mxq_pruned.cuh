@@ -20,8 +20,8 @@
 //
 // Measured against lists of the codes that bounds from the best of two probes left (9 to 17 a block), evaluated in the order of their
 // length after a sort in shared memory; 16.8 M elements, us before -> now:
-//   fp32 Laplace, tensor scale, UE4M3   B = 2 186 -> 76    4 124 -> 57   8 107 -> 50   16 109 -> 54   32 123 -> 55   64 145 -> 60
-//   bf16 Student-t, UE5M3               B = 2 205 -> 72    4 128 -> 49   8 99 -> 37    16 92 -> 35    32 92 -> 34    64 106 -> 38
+//   fp32 Laplace, tensor scale, UE4M3   B = 2 186 -> 62    4 124 -> 52   8 107 -> 48   16 109 -> 53   32 123 -> 54   64 145 -> 60
+//   bf16 Student-t, UE5M3               B = 2 205 -> 60    4 128 -> 43   8 99 -> 37    16 92 -> 36    32 92 -> 34    64 106 -> 38
 //   bf16 Student-t, UE4M3 (scale codes below 16)
 //                                       B = 2 217 -> 148   4 129 -> 98   8 91 -> 68    16 79 -> 52    32 80 -> 48    64 97 -> 51
 //   bf16 Student-t, UE8M0               B = 2 64 -> 36     4 51 -> 28    8 40 -> 21    16 31 -> 16    32 25 -> 15    64 27 -> 18
@@ -61,7 +61,8 @@ __device__ __forceinline__ float element(const float2 (&v)[pruned_values(B)], in
 // 2^60].  kModeHalf: -D is exact in f16 (and for bf16 input D has at most four significant bits, so that the quotient is one
 // multiply rounded toward zero).  kModeChecked (bf16): the one-multiply quotient with the reciprocal that
 // build_quant_tables() checked.
-enum { kModeExact = 0, kModeHalf = 1, kModeChecked = 2 };
+// kModeAny: a loop whose blocks choose.
+enum { kModeExact = 0, kModeHalf = 1, kModeChecked = 2, kModeAny = 3 };
 
 // The grid values that two quotients round to, widened by mixed-precision adds of -0 (exact).
 __device__ __forceinline__ float2 round_widen_pair(float2 t) {
@@ -81,9 +82,10 @@ __device__ __forceinline__ float2 round_widen_pair(float2 t) {
     return q;
 }
 
-// What an evaluation needs of two candidates (.x, .y).  The table holds for code c >= 1 what the pair c, c - 1 (code 1 twice) takes: -D of
+// What an evaluation needs of two candidates (.x, .y).  The table holds for code c what the pair c, c - 1 takes: -D of
 // the two, then their reciprocals (RN(1 / D), or the checked one of the launch), in the register pairs of the packed
-// instructions: one 128-bit read.
+// instructions: one 128-bit read.  Codes below 1 stand for code 1, down to the last that the eight codes from any first one on reach.
+constexpr int kLeadIn = 8;   // entries before that of code 0
 template <int DT, int MODE>
 struct Candidates {
     static constexpr bool ONE_MULTIPLY = (DT == kBF16) && MODE != kModeExact;
@@ -98,7 +100,7 @@ struct Candidates {
             nD16 = *reinterpret_cast<const uint32_t*>(&h);
         }
     }
-    __device__ __forceinline__ void read_down(const float4* tab, int c) {   // c, max(c - 1, 1)
+    __device__ __forceinline__ void read_down(const float4* tab, int c) {   // c, c - 1
         const float4 P = tab[c];
         set(P.x, P.y, P.z, P.w);
     }
@@ -258,7 +260,7 @@ __device__ __forceinline__ size_t pruned_first_unit() {
 struct PrunedConsts {
     float g, Rg;          // tensor scale and RN(1 / g)
     int first;            // smallest admissible code
-    bool g_ok;            // g within [2^-60, 2^60]
+    float a_lo, a_hi;     // largest magnitudes for which the shortcuts hold
 };
 
 // One block under the codes that the rules leave: the largest code with D <= 2 a / 7, `top` (0: none), and the seven below it, further down
@@ -285,12 +287,16 @@ __device__ __forceinline__ bool search_codes(const float4* tab, const float2 (&v
         int at = 0;   // the best code is `at` below top; in descending order an equal SSE replaces: the smallest code of a tie stays
 #pragma unroll (B <= 16 ? kMain : 1)
         for (int i = 0; i < kMain; ++i) {
-            c2.read_down(tab, max(top - 2 * i, 1));
+            c2.read_down(tab, top - 2 * i);
             const float2 s = sse_two_candidates<DT, B, MODE>(v, c2);
             keep_smaller_or_equal(best_bits, at, __float_as_uint(s.x), 2 * i);
             keep_smaller_or_equal(best_bits, at, __float_as_uint(s.y), 2 * i + 1);
         }
         best_code = max(top - at, 1);   // code 1 again and again at the end
+    }
+    {   // nearly every block ends here: no code below can be better, and there is none above
+        const float e = __fmaf_rn(6.0f, tab[top - 2 * kMain].x, a);
+        if (top >= 16 && e > 0.0f && __float_as_uint(__fmul_rn(e, e)) > best_bits) return true;
     }
     bool in_range = true, stopped = false;
 #pragma unroll 1
@@ -358,7 +364,8 @@ __global__ void __launch_bounds__(kThreads, pruned_min_ctas(B)) k_pruned(QuantAr
     constexpr int NC = num_codes(FMT);
     constexpr float kUp = 1.00000095367431640625f;   // 1 + 2^-20: above the rounding of a / g
     __shared__ QuantTables T;
-    __shared__ float4 tab[256];
+    __shared__ float4 pair_table[kLeadIn + 256];
+    const float4* const tab = pair_table + kLeadIn;
     __shared__ int short_end;   // f32: first code whose -D is not exact in f16
 
     wait_for_prior_grid();
@@ -369,54 +376,57 @@ __global__ void __launch_bounds__(kThreads, pruned_min_ctas(B)) k_pruned(QuantAr
     if (threadIdx.x == 0) short_end = NC;
     int first_bad;
     const bool checked = build_quant_tables<FMT, DT == kBF16>(T, k.g, first_bad);   // barriers inside
-    {
-        const int c = threadIdx.x;
-        const float4 E = T.E[c], F = T.E[max(c - 1, min(c, 1))];
-        tab[c] = make_float4(-E.x, -F.x, checked ? E.z : E.y, checked ? F.z : F.y);
-        if (DT == kF32 && c < NC && E.w < 2.0f) atomicMin(&short_end, c);
+    for (int c = (int)threadIdx.x - kLeadIn; c < 256; c += kThreads) {
+        const float4 E = T.E[max(c, 1)], F = T.E[max(c - 1, 1)];
+        pair_table[c + kLeadIn] = make_float4(-E.x, -F.x, checked ? E.z : E.y, checked ? F.z : F.y);
+        if (DT == kF32 && c >= 0 && c < NC && T.E[c].w < 2.0f) atomicMin(&short_end, c);
     }
     __syncthreads();
     const int fast_mode = checked ? kModeChecked : kModeHalf;
     const int fast_end = checked ? NC : (DT == kF32 ? short_end : first_bad);   // codes below it may be evaluated in fast_mode
-    k.g_ok = k.g >= kFastMin && k.g <= kFastMax;
-    k.Rg = k.g_ok ? __frcp_rn(k.g) : 1.0f;
+    const bool g_ok = k.g >= kFastMin && k.g <= kFastMax;
+    k.Rg = g_ok ? __frcp_rn(k.g) : 1.0f;
+    k.a_lo = g_ok ? 2.77555756156289135e-17f /* 2^-55 */ : 1.0f;
+    k.a_hi = g_ok ? 1.44115188075855872e17f /* 2^57 */ : 0.0f;   // no block at all
+    // the launch's mode; a block whose codes reach beyond its end is evaluated exactly
+    const int main_mode = fast_end >= 64 ? fast_mode : kModeExact;
+    const int top_end = main_mode == kModeExact ? NC : fast_end;
 
     const size_t n_units = (p.n_items + UB - 1) / UB;
     double sse_sum = 0.0;
-    for (size_t un = pruned_first_unit(); un < n_units; un += (size_t)gridDim.x * kThreads) {
-        const size_t blk = un * UB;
-        const bool whole = blk + UB <= p.n_items;   // else the tensor ends inside the unit (B = 2 and 4)
-        float v[UE];
-        if (whole) {
-            load_elems<DT, UE>(p.x, un * UE, v);
-        } else {
+    auto unit_loop = [&](auto mode_tag) {
+        constexpr int MODE = decltype(mode_tag)::value;
+        for (size_t un = pruned_first_unit(); un < n_units; un += (size_t)gridDim.x * kThreads) {
+            const size_t blk = un * UB;
+            const bool whole = blk + UB <= p.n_items;   // else the tensor ends inside the unit (B = 2 and 4)
+            float v[UE];
+            if (whole) {
+                load_elems<DT, UE>(p.x, un * UE, v);
+            } else {
 #pragma unroll
-            for (int i = 0; i < UE; ++i) v[i] = 0.0f;
+                for (int i = 0; i < UE; ++i) v[i] = 0.0f;
 #pragma unroll
-            for (int j = 0; j < UB; ++j) {
-                if (blk + j < p.n_items) {
-                    float w[B];
-                    load_elems<DT, B>(p.x, (blk + j) * B, w);
+                for (int j = 0; j < UB; ++j) {
+                    if (blk + j < p.n_items) {
+                        float w[B];
+                        load_elems<DT, B>(p.x, (blk + j) * B, w);
 #pragma unroll
-                    for (int i = 0; i < B; ++i) v[j * B + i] = w[i];
+                        for (int i = 0; i < B; ++i) v[j * B + i] = w[i];
+                    }
                 }
             }
-        }
-        uint32_t packed[UE / 8];
-        uint32_t sw[UB], sc = 0;
-        float t[UE];
+            uint32_t packed[UE / 8];
+            uint32_t sw[UB], sc = 0;
+            float t[UE];
 #pragma unroll
-        for (int j = 0; j < UB; ++j) {
-            float a = 0.0f;
+            for (int j = 0; j < UB; ++j) {
+                float a = 0.0f;
 #pragma unroll
-            for (int i = 0; i < B; ++i) a = fmaxf(a, fabsf(v[j * B + i]));
-            uint32_t bits = 0;
-            int code = k.first;   // a block of zeros: every code reproduces it
-            int mode = kModeExact;
-            bool divide = false;
-            if (a != 0.0f) {
-                divide = !(k.g_ok && a <= 1.44115188075855872e17f /* 2^57 */ && a >= 2.77555756156289135e-17f /* 2^-55 */);
-                if (!divide) {
+                for (int i = 0; i < B; ++i) a = fmaxf(a, fabsf(v[j * B + i]));
+                uint32_t bits = 0;
+                int code = k.first;   // a block of zeros: every code reproduces it
+                bool divide = false, one_multiply = false;
+                if (a >= k.a_lo && a <= k.a_hi) {
                     float2 vh[pruned_values(B)];
                     {
                         float2 w2[B / 2];
@@ -426,47 +436,60 @@ __global__ void __launch_bounds__(kThreads, pruned_min_ctas(B)) k_pruned(QuantAr
                     }
                     const float u = __fmul_rn(a, k.Rg);
                     const int top = floor_code<FMT>(__fmul_rn(u, 0.2857142857f * kUp));
-                    if (max(top, 15) < fast_end) mode = fast_mode;
-                    if (mode == kModeExact) divide = !search_codes<DT, B, FMT, kModeExact>(tab, vh, a, u, top, k, bits, code);
-                    else if (mode == kModeHalf) divide = !search_codes<DT, B, FMT, kModeHalf>(tab, vh, a, u, top, k, bits, code);
-                    else if constexpr (DT == kBF16) divide = !search_codes<DT, B, FMT, kModeChecked>(tab, vh, a, u, top, k, bits, code);
+                    auto search = [&](auto tag) {
+                        constexpr int M = decltype(tag)::value;
+                        divide = !search_codes<DT, B, FMT, M>(tab, vh, a, u, top, k, bits, code);
+                        one_multiply = DT == kBF16 && M != kModeExact;
+                    };
+                    const int mode = top < top_end ? (MODE == kModeAny ? main_mode : MODE) : kModeExact;
+                    if (mode == kModeExact) search(std::integral_constant<int, kModeExact>{});
+                    else if (MODE == kModeHalf || (MODE == kModeAny && mode == kModeHalf)) search(std::integral_constant<int, kModeHalf>{});
+                    else if constexpr (DT == kBF16 && (MODE == kModeChecked || MODE == kModeAny)) search(std::integral_constant<int, kModeChecked>{});
+                } else {
+                    divide = a != 0.0f;
                 }
                 if (divide) {
                     const unsigned long long key = search_block_by_division<DT, B, FMT>(p.x, blk + j, a, k.g, k.first);
                     bits = (uint32_t)(key >> 32);
                     code = (int)(key & 0xFFu);
                 }
+                sw[j] = bits;
+                sc |= (uint32_t)code << (8 * j);
+                // encode with the winner
+                const float4 E = T.E[code];
+                if (divide || E.y == 0.0f) {
+#pragma unroll
+                    for (int i = 0; i < B; ++i) t[j * B + i] = quotient_general(v[j * B + i], E.x);
+                } else if (one_multiply) {
+                    const float R = tab[code].z;
+#pragma unroll
+                    for (int i = 0; i < B; ++i) t[j * B + i] = __fmul_rz(v[j * B + i], R);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < B; ++i) t[j * B + i] = quotient_corrected(v[j * B + i], E.x, E.y);
+                }
             }
-            sw[j] = bits;
-            sc |= (uint32_t)code << (8 * j);
-            // encode with the winner
-            const float4 E = T.E[code];
-            if (divide || E.y == 0.0f) {
 #pragma unroll
-                for (int i = 0; i < B; ++i) t[j * B + i] = quotient_general(v[j * B + i], E.x);
-            } else if (DT == kBF16 && mode == fast_mode) {
-                const float R = tab[code].z;
-#pragma unroll
-                for (int i = 0; i < B; ++i) t[j * B + i] = __fmul_rz(v[j * B + i], R);
+            for (int w = 0; w < UE / 8; ++w)
+                packed[w] = pack_e2m1x8(t[8 * w], t[8 * w + 1], t[8 * w + 2], t[8 * w + 3], t[8 * w + 4], t[8 * w + 5], t[8 * w + 6], t[8 * w + 7]);
+            if (whole) {
+                store_bytes<UE / 2>(p.codes + un * (UE / 2), packed);
+                store_bytes<UB>(p.scales + blk, &sc);
+                if (p.block_sse) store_bytes<4 * UB>(p.block_sse + blk, sw);
             } else {
-#pragma unroll
-                for (int i = 0; i < B; ++i) t[j * B + i] = quotient_corrected(v[j * B + i], E.x, E.y);
+                store_whole_blocks<B>(p, blk, p.n_items - blk, packed[0], sc, sw);
             }
-        }
 #pragma unroll
-        for (int w = 0; w < UE / 8; ++w)
-            packed[w] = pack_e2m1x8(t[8 * w], t[8 * w + 1], t[8 * w + 2], t[8 * w + 3], t[8 * w + 4], t[8 * w + 5], t[8 * w + 6], t[8 * w + 7]);
-        if (whole) {
-            store_bytes<UE / 2>(p.codes + un * (UE / 2), packed);
-            store_bytes<UB>(p.scales + blk, &sc);
-            if (p.block_sse) store_bytes<4 * UB>(p.block_sse + blk, sw);
-        } else {
-            store_whole_blocks<B>(p, blk, p.n_items - blk, packed[0], sc, sw);
+            for (int j = 0; j < UB; ++j)
+                if (whole || blk + j < p.n_items) sse_sum = __dadd_rn(sse_sum, (double)__uint_as_float(sw[j]));
         }
-#pragma unroll
-        for (int j = 0; j < UB; ++j)
-            if (whole || blk + j < p.n_items) sse_sum = __dadd_rn(sse_sum, (double)__uint_as_float(sw[j]));
-    }
+    };
+    // a loop for the launch's mode pays for short blocks, whose tests and branches weigh (16.8 M elements, us: fp32, tensor scale, B = 2 76 -> 62, 4 57 ->
+    // 52, 8 50 -> 48; bf16, UE5M3, 72 -> 60, 49 -> 43, 38 -> 37); B = 32 lost 1 % on small tensors
+    if constexpr (B > 8) unit_loop(std::integral_constant<int, kModeAny>{});
+    else if (main_mode == kModeExact) unit_loop(std::integral_constant<int, kModeExact>{});
+    else if (main_mode == kModeHalf) unit_loop(std::integral_constant<int, kModeHalf>{});
+    else if constexpr (DT == kBF16) unit_loop(std::integral_constant<int, kModeChecked>{});
     if (p.mse_partials != nullptr) {   // launch-uniform: fused tensor-MSE partial sum of this CTA
         __syncthreads();               // the tables are no longer read: their memory serves as scratch
         const double total = cta_sum_fixed_order(sse_sum, reinterpret_cast<double*>(&T));
