@@ -61,7 +61,13 @@ namespace mxq {
 //      D = 0 counts as valid with R = 0: every quotient comes out as a zero with the sign of v.
 struct QuantTables {
     float4 E[256];
+    // What the lean loops read of an entry for blocks of 2 and 4, 64 bits (fill_lean_table()).  16-byte entries at per-lane codes cost four
+    // shared-memory wavefronts and as many conflicts for every block and candidate, which is what the kernels for small blocks waited for
+    // (16.8 M bf16 elements, 128- -> 64-bit reads, us: abs-max, UE4M3, B = 2 19.0 -> 18.3, 4 13.4 -> 13.2; 4-over-6, UE4M3, B = 2 22.1 -> 20.6, 4 16.1
+    // -> 15.2; UE5M3, B = 2 29.2 -> 24.7, 4 18.7 -> 17.6; longer blocks lose 1 to 3 %, and read E).
+    float2 L[256];
 };
+__host__ __device__ constexpr bool has_lean_table(int B) { return B <= 4; }
 
 // Does the FP4 code of RZ(v * R) equal the FP4 code of fl32(v / D) for EVERY bf16 value v?  (D a
 // normal binary32 number, R within a few units in the last place of 1 / D.)  Both codes are
@@ -458,6 +464,21 @@ __device__ __forceinline__ bool lean_scaled_allowed(const QuantConsts& k) {
     return k.onemul && k.g >= 9.094947017729282379e-13f /* 2^-40 */ && k.g <= 1048576.0f;
 }
 
+// LEAN 1: RN(1 / D) and f16(-D); LEAN 2: the checked reciprocal and D.  A barrier inside.
+template <int LEAN>
+__device__ __forceinline__ void fill_lean_table(QuantTables& T) {
+    const float4 E = T.E[threadIdx.x];
+    T.L[threadIdx.x] = LEAN == 1 ? make_float2(E.y, E.z) : make_float2(E.z, E.x);
+    __syncthreads();
+}
+// The fields of an entry that encode_group_fast() and its 4-over-6 form take in a lean loop.
+template <int B, int LEAN>
+__device__ __forceinline__ float4 lean_entry(const QuantTables& T, int c) {
+    if constexpr (!has_lean_table(B)) return T.E[c];
+    const float2 l = T.L[c];
+    return LEAN == 1 ? make_float4(0.0f, l.x, l.y, 0.0f) : make_float4(l.y, 0.0f, l.x, 0.0f);
+}
+
 // Both 4-over-6 scale codes of a block from one conversion (UE4M3): the code for w6 in bits 0..7,
 // the code for w4 in bits 8..15.
 __device__ __forceinline__ uint32_t round_scale_pair_ue4m3(float w4, float w6) {
@@ -635,8 +656,8 @@ __device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const QuantTa
                     c6[j] = round_scale<FMT>(w6);
                     if constexpr (DUAL) c4[j] = round_scale<FMT>(__fmul_rn(uf, 0.25f));
                 }
-                E6[j] = T.E[c6[j]];
-                if constexpr (DUAL) E4[j] = T.E[c4[j]];
+                E6[j] = lean_entry<B, LEAN>(T, c6[j]);
+                if constexpr (DUAL) E4[j] = lean_entry<B, LEAN>(T, c4[j]);
                 continue;
             }
             m[j] = a;
@@ -726,7 +747,7 @@ __device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const QuantTa
         }
         if constexpr (FAKE) {
 #pragma unroll
-            for (int j = 0; j < NBG; ++j) fake->D[gi * NBG + j] = Dw[j];
+            for (int j = 0; j < NBG; ++j) fake->D[gi * NBG + j] = LEAN == 1 && has_lean_table(B) ? T.E[c6[j]].x : Dw[j];   // not read so far
         }
 #pragma unroll
         for (int i = 0; i < S::GE / 8; ++i) packed[gi * (S::GE / 8) + i] = pk[i];
@@ -1041,6 +1062,11 @@ __device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, QuantTab
         k.m_lo = 0.0f;
     }
 
+    constexpr bool CAN_LEAN = (DT == kBF16) && (FMT != kUE8M0) && !(long_block_path(B, DUAL));
+    if constexpr (CAN_LEAN && has_lean_table(B)) {
+        if (lean_allowed<FMT>(first_bad, k.unit_g)) fill_lean_table<1>(T);
+        else if (lean_scaled_allowed(k)) fill_lean_table<2>(T);
+    }
     const uint32_t total_rows = row0[nt];
     const uint32_t row_stride = gridDim.x * (kThreads / 32);
     constexpr size_t kChunkBytes = (size_t)S::C * S::EB;
@@ -1126,7 +1152,6 @@ __device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, QuantTab
             }
         }
     };
-    constexpr bool CAN_LEAN = (DT == kBF16) && (FMT != kUE8M0) && !(long_block_path(B, DUAL));
     if constexpr (CAN_LEAN) {
         if (lean_allowed<FMT>(first_bad, k.unit_g)) row_loop(std::integral_constant<int, 1>{});
         else if (lean_scaled_allowed(k)) row_loop(std::integral_constant<int, 2>{});
@@ -1231,6 +1256,11 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
     // Thread-private staging: a thread leaves when its chunks are done (no barrier follows).
     // Cooperative staging: the warp stays together, lanes past the end only take part in the copies.
     // (with fused MSE partial sums every thread stays for the CTA-wide sum at the end)
+    constexpr bool CAN_LEAN = (DT == kBF16) && (FMT != kUE8M0) && !(long_block_path(B, DUAL));
+    if constexpr (CAN_LEAN && has_lean_table(B)) {
+        if (lean_allowed<FMT>(first_bad, k.unit_g)) fill_lean_table<1>(T);
+        else if (lean_scaled_allowed(k)) fill_lean_table<2>(T);
+    }
     double sse_sum = 0.0;   // binary64 sum of the SSEs of this thread's blocks, in the order it produced them
     constexpr bool TOGETHER = S::COOP || FAKE;   // the warp stays together through the loop
     const bool has_work = (TOGETHER ? wchunk0 : chunk) < p.n_items;
@@ -1280,7 +1310,6 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
             }
         }
     };
-    constexpr bool CAN_LEAN = (DT == kBF16) && (FMT != kUE8M0) && !(long_block_path(B, DUAL));
     if (has_work) {
         if constexpr (CAN_LEAN) {
             if (lean_allowed<FMT>(first_bad, k.unit_g)) chunk_loop(std::integral_constant<int, 1>{});
