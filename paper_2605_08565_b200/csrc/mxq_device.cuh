@@ -236,22 +236,28 @@ __device__ __forceinline__ void load_elems(const void* base, size_t first_elem, 
     }
 }
 
-// Write BYTES bytes held in 32-bit words (BYTES = 1, 2, 4, 8 or a multiple of 16).
-template <int BYTES>
+template <bool KEEP, typename V>
+__device__ __forceinline__ void store_word(V* dst, V v) {
+    if constexpr (KEEP) *dst = v;
+    else __stcs(dst, v);
+}
+
+// Write BYTES bytes held in 32-bit words (BYTES = 1, 2, 4, 8 or a multiple of 16).  KEEP: they are read next, else streaming.
+template <int BYTES, bool KEEP = false>
 __device__ __forceinline__ void store_bytes(void* dst, const uint32_t* w) {
     if constexpr (BYTES == 1) {
         *static_cast<uint8_t*>(dst) = (uint8_t)w[0];
     } else if constexpr (BYTES == 2) {
         *static_cast<uint16_t*>(dst) = (uint16_t)w[0];
     } else if constexpr (BYTES == 4) {
-        __stcs(static_cast<uint32_t*>(dst), w[0]);
+        store_word<KEEP>(static_cast<uint32_t*>(dst), w[0]);
     } else if constexpr (BYTES == 8) {
-        __stcs(static_cast<uint2*>(dst), make_uint2(w[0], w[1]));
+        store_word<KEEP>(static_cast<uint2*>(dst), make_uint2(w[0], w[1]));
     } else {
         static_assert(BYTES % 16 == 0, "unsupported store size");
 #pragma unroll
         for (int k = 0; k < BYTES / 16; ++k)
-            __stcs(static_cast<uint4*>(dst) + k, make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]));
+            store_word<KEEP>(static_cast<uint4*>(dst) + k, make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]));
     }
 }
 
