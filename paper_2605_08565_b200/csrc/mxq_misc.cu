@@ -244,9 +244,14 @@ __global__ void __launch_bounds__(kThreads) k_mse_partial(const float* sse, size
 // The second level of a tensor MSE: sum of n partials over a CTA of kThreads threads in a fixed order (thread t those at t, t + 256,
 // ..., then cta_sum_fixed_order()), valid in thread 0.  Read from L2: other CTAs have just written them.
 __device__ __forceinline__ double sum_partials(const double* partials, int n, double* scratch) {
-    double v = 0.0;
-    for (int i = threadIdx.x; i < n; i += kThreads) v = __dadd_rn(v, __ldcg(partials + i));
-    return cta_sum_fixed_order(v, scratch);
+    static_assert(kMsePartials == 4 * kThreads, "four partials per thread");
+    double w[4];   // all reads at once: one after the other they cost a large tensor 0.2 us
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = threadIdx.x + k * kThreads;
+        w[k] = i < n ? __ldcg(partials + i) : 0.0;
+    }
+    return cta_sum_fixed_order(__dadd_rn(__dadd_rn(__dadd_rn(w[0], w[1]), w[2]), w[3]), scratch);
 }
 
 __global__ void __launch_bounds__(kThreads) k_mse_final(const double* partials, int n_partials, double n, double* out) {
