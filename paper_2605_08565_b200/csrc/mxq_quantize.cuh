@@ -526,17 +526,21 @@ struct FakeChunk {
 // Fake-quantize: x_hat = fl32(grid(code) * D), optionally rounded to bf16, of the warp's n_valid chunks from chunk wchunk on.  A
 // thread's own x_hat is a run of 32 to 256 bytes; stored by the thread that made it, every 16-byte store of a warp would touch 16 or
 // 32 cache lines and write half sectors (33.5 M bf16 elements, B = 32, UE8M0, bf16 out: 26.7 us, here 22.2;
-// 16.8 M bf16 elements, B = 8, 4-over-6, fp32 out 33.4, here 17.7).  So the packed codes and the decode scales (for bf16 blocks of 2, where these
+// 16.8 M bf16 elements, B = 8, 4-over-6, fp32 out 33.4, here 17.7).  So the packed codes and the decode scales (for blocks of 2, where these
 // would not fit, the scale bytes) go through the ring slot that the chunk came from, and the warp forms and stores 512 contiguous bytes at a time.
+// Not for fp32 blocks of 2, whose chunks of 16 elements hold eight scales: there a thread's run is at least a sector, and staging the scales
+// costs more than it saves (16.8 M elements, bf16 out 19.5 us, staged 21 to 27).
 // Every lane of the warp calls it.
+__host__ __device__ constexpr bool fake_stores_together(int DT, int B) { return !(DT == kF32 && B == 2); }
 template <int DT, int B>
 __device__ __forceinline__ void store_fake_chunks(const QuantArgs& p, const QuantTables& T, const FakeChunk<DT, B>& f, size_t wchunk, int n_valid,
                                                   uint4* slot_warp, int lane) {
     using S = QuantShape<DT, B>;
     constexpr int ROW = 512, ROW_STRIDE = kThreads * 16;   // a row of the slot: 16 bytes per lane of the warp
     constexpr int CODE_ROWS = (32 * S::C / 2 + ROW - 1) / ROW;
-    constexpr bool BY_CODE = (B == 2 && DT == kBF16);
+    constexpr bool BY_CODE = (B == 2);
     constexpr int D_BYTES = BY_CODE ? S::NBC : 4 * S::NBC;   // per lane
+    constexpr int V = S::NBC >= 4 ? 4 : S::NBC;
     static_assert(CODE_ROWS + (32 * D_BYTES + ROW - 1) / ROW <= S::PIECES, "fits the slot");
     unsigned char* const base = reinterpret_cast<unsigned char*>(slot_warp);
     auto at = [&](int o) { return base + o / ROW * ROW_STRIDE + o % ROW; };
@@ -553,7 +557,11 @@ __device__ __forceinline__ void store_fake_chunks(const QuantArgs& p, const Quan
         for (int i = 0; i < S::NBC / 4; ++i) *reinterpret_cast<uint32_t*>(dat(lane * D_BYTES + 4 * i)) = f.scales[i];
     } else {
 #pragma unroll
-        for (int i = 0; i < S::NBC; ++i) *reinterpret_cast<float*>(dat(lane * D_BYTES + 4 * i)) = f.D[i];
+        for (int i = 0; i < S::NBC; i += V) {   // as wide as they come: 4-byte stores 32 bytes apart meet eight to a bank
+            if constexpr (V == 4) *reinterpret_cast<float4*>(dat(lane * D_BYTES + 4 * i)) = make_float4(f.D[i], f.D[i + 1], f.D[i + 2], f.D[i + 3]);
+            else if constexpr (V == 2) *reinterpret_cast<float2*>(dat(lane * D_BYTES + 4 * i)) = make_float2(f.D[i], f.D[i + 1]);
+            else *reinterpret_cast<float*>(dat(lane * D_BYTES + 4 * i)) = f.D[i];
+        }
     }
     __syncwarp();
     auto store_units = [&](auto bf16_tag) {
@@ -598,6 +606,32 @@ __device__ __forceinline__ void store_fake_chunks(const QuantArgs& p, const Quan
     };
     if (p.xhat_dtype == kBF16) store_units(std::integral_constant<bool, true>{});
     else store_units(std::integral_constant<bool, false>{});
+}
+
+// The same by the thread itself.
+template <int DT, int B>
+__device__ __forceinline__ void store_fake_chunk(const QuantArgs& p, const FakeChunk<DT, B>& f, size_t chunk) {
+    using S = QuantShape<DT, B>;
+#pragma unroll
+    for (int w8 = 0; w8 < S::C / 8; ++w8) {
+        float q[8];
+        unpack_e2m1x8(f.codes[w8], q);
+        uint32_t o[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(__fmul_rn(q[i], f.D[(8 * w8 + i) / B]));
+        const size_t e0 = chunk * S::C + 8 * w8;
+        if (p.xhat_dtype == kF32) {
+            store_bytes<32>(static_cast<float*>(p.xhat) + e0, o);
+        } else {
+            uint32_t h[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(o[2 * i]), __uint_as_float(o[2 * i + 1]));
+                h[i] = *reinterpret_cast<const uint32_t*>(&b2);
+            }
+            store_bytes<16>(static_cast<__nv_bfloat16*>(p.xhat) + e0, h);
+        }
+    }
 }
 
 // LEAN == 2: the same loop under a tensor scale, see lean_scaled_allowed(): the block maximum is divided by g
@@ -1316,9 +1350,11 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
                     quantize_chunk<DT, B, FMT, DUAL, FAKE, LEAN>(p, T, k, chunk, raw, sse_sum, &fake);
                 }
             }
-            if constexpr (FAKE) {
+            if constexpr (FAKE && fake_stores_together(DT, B)) {
                 const size_t left = p.n_items - lead;
                 store_fake_chunks<DT, B>(p, T, fake, lead, left < 32 ? (int)left : 32, slot_warp, lane);
+            } else if constexpr (FAKE) {
+                if (chunk < p.n_items) store_fake_chunk<DT, B>(p, fake, chunk);
             }
         }
     };
