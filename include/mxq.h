@@ -21,7 +21,9 @@
  *     mxq_last_cuda_error() is per thread.  Two things are process-wide and therefore shared by all
  *     threads: the options of mxq_set_option() (a call reads the option once, when it is made; changing
  *     it while another thread is inside mxq_quantize_ex affects only calls made afterwards), and the
- *     scratch array of mxq_tensor_mse_static() (see there).  As with any CUDA library, the device that
+ *     scratch array of mxq_tensor_mse_static() (see there).  mxq_tensor_amax() beyond 256 KB takes a slot of
+ *     a ring of 2^18 that the library keeps on each device (2 MB, handed out in turn, zero between
+ *     launches); under stream capture it takes none.  As with any CUDA library, the device that
  *     owns the pointers must be the calling thread's current device.
  *
  * Data layout
