@@ -545,6 +545,10 @@ __device__ __forceinline__ unsigned long long pow2_search(const float2 (&v2)[B /
     // 2^c0 <= a / 6g < 2^(c0 + 1), to within the rounding: code c0 + 2 and all above it are beyond 2 a / 7
     try_two(0);
     const uint32_t ubits = (uint32_t)(best >> 32);
+    if (ubits > 0x7F800000u) {   // a NaN element: so is every SSE, no rule ends the search, and the codes it would end at are out of the shortcuts' range
+        fast = false;
+        return sse_key(__uint_as_float(ubits), 0);
+    }
     for (int k = -1; c0 + k >= 0; --k) {
         const float nD = shifted(nD0, k), R = shifted(R0, -k);
         const float e = __fmaf_rn(6.0f, nD, a);

@@ -586,6 +586,29 @@ def test_non_finite_elements_stay_inside_their_own_blocks(dtype, B, sweep_mode):
     check_parity(clean, B, mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6_PZ, 1.0)
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B", BLOCKS)
+def test_both_searches_agree_on_blocks_with_a_nan(dtype, B):
+    """Every code of such a block has a NaN for its SSE, so both searches fall to the smallest code and encode under it; with the
+    power-of-two format its scale lies far below the range in which the pruned search forms scales from exponents."""
+    nb = 300
+    x = inputs.normal(nb * B, 77 + B, 1.0, torch.float32).view(nb, B)
+    x[0::3, 0] = float("nan")
+    x[1::3, B - 1] = float("nan")
+    x = x.reshape(-1).to(dtype)
+    for fmt in FMTS:
+        for recipe, g in ((mxq.MXQ_BRUTE, 1.0), (mxq.MXQ_BRUTE_PZ, 0.0131), (mxq.MXQ_BRUTE, 2.0 ** -43), (mxq.MXQ_BRUTE_PZ, 2.0 ** 45)):
+            out = []
+            for prune in (0, 1):
+                mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, prune)
+                try:
+                    out.append(gpu_quantize(x, B, fmt, recipe, g))
+                finally:
+                    mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 0)
+            for full, pruned in zip(out[0][:3], out[1][:3]):
+                assert np.array_equal(full.view(np.uint8), pruned.view(np.uint8)), (fmt, recipe, g)
+
+
 def test_device_resident_global_scale_matches_host_scale():
     x = _mixed(8192, 5, torch.bfloat16)
     for recipe in (mxq.MXQ_ABSMAX, mxq.MXQ_4O6, mxq.MXQ_BRUTE):
