@@ -1,6 +1,5 @@
 // Small kernels around the quantization pass: per-tensor abs-max (first stage of hierarchical
-// scaling), deterministic tensor MSE, de-quantization, and a scalar kernel for the few blocks
-// that do not fill a whole per-thread chunk.
+// scaling), deterministic tensor MSE and de-quantization.
 #include <cuda_bf16.h>
 
 #include <atomic>
@@ -22,23 +21,14 @@ struct DoneSlot {
 constexpr unsigned kDoneSlots = 1u << 18;
 static __device__ DoneSlot g_done_slots[kDoneSlots];
 
-// A slot for one launch on the current device, or NULL while the stream is being captured (a graph replays with the same slot at any
-// later time, beside launches that were given it meanwhile): the launch then takes the route with the initialising kernel.
-static DoneSlot* done_slot(cudaStream_t s) {
-    static std::atomic<DoneSlot*> ring_of_device[kMaxDevices];   // first-use cache; racing threads store the same value
+// The number of a slot for one launch (a number and not an address: the kernel finds the array of the context that it runs in, whichever
+// device that is and however often its context was made anew), or -1 while the stream is being captured (a graph replays with the
+// same slot at any later time, beside launches that were given it meanwhile): the launch then takes the route with the initialising kernel.
+static int done_slot(cudaStream_t s) {
     static std::atomic<unsigned> next{0};
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
-    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return nullptr;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-    DoneSlot* ring = ring_of_device[dev].load(std::memory_order_relaxed);
-    if (ring == nullptr) {
-        void* p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_done_slots) != cudaSuccess) return nullptr;
-        ring = static_cast<DoneSlot*>(p);
-        ring_of_device[dev].store(ring, std::memory_order_relaxed);
-    }
-    return ring + next.fetch_add(1, std::memory_order_relaxed) % kDoneSlots;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return -1;
+    return (int)(next.fetch_add(1, std::memory_order_relaxed) % kDoneSlots);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -70,7 +60,7 @@ __device__ __forceinline__ float scale_of_amax(float a) { return (a > 0.0f && a 
 // the tensor in L2, was measured on 33 to 117 MB tensors and gains nothing (that pass is not DRAM-bound
 // enough at those sizes), while it slows this kernel by 5 %.
 template <int DT>
-__global__ void __launch_bounds__(kThreads) k_tensor_amax(const void* x, size_t n, uint32_t* out_bits, uint32_t* g_word, DoneSlot* done) {
+__global__ void __launch_bounds__(kThreads) k_tensor_amax(const void* x, size_t n, uint32_t* out_bits, uint32_t* g_word, int slot) {
     constexpr int VEC = 16 / elem_bytes(DT);
     constexpr int U = 4;
     const size_t n_vec = n / VEC;
@@ -119,6 +109,7 @@ __global__ void __launch_bounds__(kThreads) k_tensor_amax(const void* x, size_t 
         m = threadIdx.x < kThreads / 32 ? warp_m[threadIdx.x] : 0.0f;
         m = warp_max(m);
         if (threadIdx.x == 0) {
+            DoneSlot* const done = slot >= 0 ? &g_done_slots[slot] : nullptr;
             unsigned* const run = done ? &done->max_bits : out_bits;
             unsigned* const count = done ? &done->arrived : g_word;
             atomicMax(run, __float_as_uint(m));
@@ -202,9 +193,9 @@ cudaError_t launch_tensor_amax(const void* x, int dtype, size_t n, float* d_amax
     }
     uint32_t* amax_bits = reinterpret_cast<uint32_t*>(d_amax);
     uint32_t* g_word = reinterpret_cast<uint32_t*>(d_g);
-    DoneSlot* const done = done_slot(s);
+    const int slot = done_slot(s);
     cudaError_t err = cudaSuccess;
-    if (!done) {
+    if (slot < 0) {
         err = launch_pdl(k_amax_init, 1u, 1u, 0, s, amax_bits, g_word);
         count_launch();
         if (err != cudaSuccess) return err;
@@ -217,8 +208,8 @@ cudaError_t launch_tensor_amax(const void* x, int dtype, size_t n, float* d_amax
     if (want == 0) want = 1;
     const size_t cap = (size_t)sm_count(dev) * 8;
     const unsigned grid = (unsigned)(want < cap ? want : cap);
-    if (dtype == kF32) err = launch_pdl(k_tensor_amax<kF32>, grid, (unsigned)kThreads, 0, s, x, n, amax_bits, g_word, done);
-    else err = launch_pdl(k_tensor_amax<kBF16>, grid, (unsigned)kThreads, 0, s, x, n, amax_bits, g_word, done);
+    if (dtype == kF32) err = launch_pdl(k_tensor_amax<kF32>, grid, (unsigned)kThreads, 0, s, x, n, amax_bits, g_word, slot);
+    else err = launch_pdl(k_tensor_amax<kBF16>, grid, (unsigned)kThreads, 0, s, x, n, amax_bits, g_word, slot);
     count_launch();
     return err;
 }

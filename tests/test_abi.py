@@ -112,3 +112,13 @@ def test_native_calls_hand_on_what_they_do_not_know(lib):
     with pytest.raises(binding.MxqError, match="status 2"):
         binding.mxq_set_option(7, 1)
     assert binding.mxq_get_option(binding.MXQ_OPT_BRUTE_PRUNE) == 0
+
+
+def test_only_the_static_mse_keeps_a_device_address(lib):
+    """A device address kept on the host outlives the context that it belongs to.  The library keeps one per device, that of the scratch
+    array of mxq_tensor_mse_static(); the slots of the tensor abs-max are handed to their kernel by number."""
+    import subprocess
+    from paper_2605_08565_b200 import binding
+    names = subprocess.run(["nm", "-C", binding.LIB_PATH], capture_output=True, text=True, check=True).stdout.splitlines()
+    kept = [n for n in names if n.endswith("of_device")]
+    assert len(kept) == 1 and "launch_tensor_mse_static" in kept[0], kept
