@@ -1,7 +1,8 @@
 """Thin binding of libmxq (argument marshalling only; every step runs in the CUDA kernels).
 
 The calls of an inner loop go through the extension module ``_native`` (csrc/mxq_python.cpp), which unpacks the usual
-arguments in C++; everything else, and whatever ``_native`` does not take, goes through ctypes.
+arguments in C++; everything else, and whatever ``_native`` does not take, goes through ctypes (all of it where ``_native``
+has not been built).
 
 The functions carry the names of the C-ABI declared in ``include/mxq.h`` and take torch CUDA
 tensors (torch supplies device memory and streams, nothing else).  There is no CPU fallback: if
@@ -11,6 +12,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 
 import torch
 
@@ -39,6 +41,13 @@ class TensorDesc(ctypes.Structure):
     """mxq_tensor_desc of include/mxq.h (one tensor of a multi-tensor launch)."""
     _fields_ = [("x", ctypes.c_void_p), ("out_codes", ctypes.c_void_p), ("out_scales", ctypes.c_void_p),
                 ("out_block_sse", ctypes.c_void_p), ("n", ctypes.c_size_t)]
+
+
+class _CtypesOnly:
+    """In the place of the extension module where it is missing: knows no arguments."""
+
+    def __getattr__(self, name):
+        return lambda *args: -1
 
 
 _lib = None
@@ -102,9 +111,11 @@ def load_library() -> ctypes.CDLL:
     L.mxq_version.argtypes = []
     try:
         from . import _native as native
+        native.bind({name: c.cast(getattr(L, name), vp).value for name in EXPORTS})
     except ImportError as e:
-        raise MxqError(f"extension module _native not found ({e}): build it with `python -m paper_2605_08565_b200.build`") from e
-    native.bind({name: c.cast(getattr(L, name), vp).value for name in EXPORTS})
+        warnings.warn(f"extension module _native not usable ({e}): every call goes through ctypes, 2 to 3 us slower; build it with "
+                      "`python -m paper_2605_08565_b200.build`", RuntimeWarning, stacklevel=2)
+        native = _CtypesOnly()
     _native = native
     _lib = L
     return L
@@ -319,7 +330,12 @@ def mxq_mask_interval(x, n, lo, hi, d_out, stream=None) -> None:
 
 
 def mxq_set_option(option: int, value: int) -> None:
-    _check((_native or _load_native()).set_option(int(option), int(value)))
+    st = (_native or _load_native()).set_option(int(option), int(value))
+    if st == 0:
+        return
+    if st > 0:
+        _check(st)
+    _check(load_library().mxq_set_option(int(option), int(value)))
 
 
 def mxq_get_option(option: int) -> int:

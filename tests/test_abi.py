@@ -122,3 +122,50 @@ def test_only_the_static_mse_keeps_a_device_address(lib):
     names = subprocess.run(["nm", "-C", binding.LIB_PATH], capture_output=True, text=True, check=True).stdout.splitlines()
     kept = [n for n in names if n.endswith("of_device")]
     assert len(kept) == 1 and "launch_tensor_mse_static" in kept[0], kept
+
+
+def test_the_binding_works_without_the_extension_module(lib, tmp_path, monkeypatch):
+    """The extension only unpacks arguments: a package without it loads, warns once and answers through ctypes; a build in which it
+    fails still delivers the library."""
+    import shutil
+    import subprocess
+    import sys
+    from paper_2605_08565_b200 import binding, build
+    copy = tmp_path / "paper_2605_08565_b200"
+    copy.mkdir()
+    for f in os.listdir(os.path.dirname(binding.__file__)):
+        if f.endswith(".py"):
+            shutil.copy(os.path.join(os.path.dirname(binding.__file__), f), copy)
+    code = """
+import warnings
+import torch
+from paper_2605_08565_b200 import binding
+with warnings.catch_warnings(record=True) as w:
+    warnings.simplefilter("always")
+    binding.load_library()
+    binding.load_library()
+assert len(w) == 1 and "_native" in str(w[0].message), [str(x.message) for x in w]
+def refused(f, text):
+    try:
+        f()
+    except binding.MxqError as e:
+        assert text in str(e), e
+    else:
+        raise AssertionError(text)
+class Stream:
+    cuda_stream = 0
+x = torch.zeros(64)
+refused(lambda: binding.mxq_quantize_ex(x, 64, 16, 1, 0, 1.0, None, x, x, None), "CUDA tensors only")
+refused(lambda: binding.mxq_segment_mse(None, 1, 1, 1, None, stream=Stream()), "status 1")
+refused(lambda: binding.mxq_set_option(7, 1), "status 2")
+binding.mxq_set_option(binding.MXQ_OPT_BRUTE_PRUNE, 1)
+assert binding.mxq_get_option(binding.MXQ_OPT_BRUTE_PRUNE) == 1
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=tmp_path, env=dict(os.environ, MXQ_LIB=binding.LIB_PATH), capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+
+    def fails(*args):
+        raise RuntimeError("no compiler")
+    monkeypatch.setattr(build, "build_native", fails)
+    with pytest.warns(RuntimeWarning, match="no compiler"):
+        assert build.build() == build.LIB
