@@ -11,10 +11,13 @@ tensors (torch supplies device memory and streams, nothing else).  There is no C
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 import warnings
 
 import torch
+
+from .build import native_path
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # MXQ_LIB: path of another build of the library; the default is the in-tree build
@@ -48,6 +51,16 @@ class _CtypesOnly:
 
     def __getattr__(self, name):
         return lambda *args: -1
+
+
+def _import_native():
+    path = native_path()
+    spec = importlib.util.spec_from_file_location(__package__ + "._native", path)
+    if not os.path.exists(path):
+        raise ImportError(f"no {os.path.basename(path)}")
+    native = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(native)
+    return native
 
 
 _lib = None
@@ -110,7 +123,7 @@ def load_library() -> ctypes.CDLL:
     L.mxq_version.restype = i32
     L.mxq_version.argtypes = []
     try:
-        from . import _native as native
+        native = _import_native()
         native.bind({name: c.cast(getattr(L, name), vp).value for name in EXPORTS})
     except ImportError as e:
         warnings.warn(f"extension module _native not usable ({e}): every call goes through ctypes, 2 to 3 us slower; build it with "

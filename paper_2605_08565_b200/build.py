@@ -5,7 +5,7 @@
 Every ``csrc/*.cu`` is compiled to an object file in ``_build/`` (in parallel) and linked into
 ``paper_2605_08565_b200/libmxq.so``.  No fast-math, no flush-to-zero, no FMA contraction: the
 kernels must reproduce IEEE binary32 results bit for bit.  ``csrc/mxq_python.cpp``, which unpacks the arguments of the
-binding's inner-loop calls, is compiled against the installed torch to ``paper_2605_08565_b200/_native.so``; where that fails (no g++, no
+binding's inner-loop calls, is compiled against the installed torch to ``paper_2605_08565_b200/_native.<versions>.so``; where that fails (no g++, no
 headers of Python or torch) the library is complete without it and the binding uses ctypes.
 """
 from __future__ import annotations
@@ -16,13 +16,13 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 import warnings
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmxq.so")
-NATIVE = os.path.join(HERE, "_native.so")
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -44,18 +44,24 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def native_path() -> str:
+    """The extension module's file.  It holds the layouts of torch's tensors and of Python's objects, so its name carries both versions:
+    another torch or Python finds no module, not this one."""
+    import torch
+    return os.path.join(HERE, f"_native.torch{torch.__version__}{sysconfig.get_config_var('EXT_SUFFIX')}")
+
+
 def build_native(force: bool = False, verbose: bool = False) -> str:
     src = os.path.join(CSRC, "mxq_python.cpp")
-    if not force and not _stale(NATIVE, [src, os.path.join(os.path.dirname(HERE), "include", "mxq.h"), os.path.abspath(__file__)]):
-        return NATIVE
-    import sysconfig
-
+    target = native_path()
+    if not force and not _stale(target, [src, os.path.join(os.path.dirname(HERE), "include", "mxq.h"), os.path.abspath(__file__)]):
+        return target
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
     include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
                os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
-    tmp = NATIVE + f".{os.getpid()}.tmp"
+    tmp = target + f".{os.getpid()}.tmp"
     cmd = [shutil.which("g++") or "g++", "-O2", "-std=c++17", "-fPIC", "-shared",
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(f"-I{d}" for d in include), src, "-o", tmp,
            "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
@@ -64,8 +70,8 @@ def build_native(force: bool = False, verbose: bool = False) -> str:
         sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
     if r.returncode != 0:
         raise RuntimeError("build of the extension module _native failed")
-    os.replace(tmp, NATIVE)
-    return NATIVE
+    os.replace(tmp, target)
+    return target
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

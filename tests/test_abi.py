@@ -169,3 +169,18 @@ assert binding.mxq_get_option(binding.MXQ_OPT_BRUTE_PRUNE) == 1
     monkeypatch.setattr(build, "build_native", fails)
     with pytest.warns(RuntimeWarning, match="no compiler"):
         assert build.build() == build.LIB
+
+
+def test_the_extension_module_is_of_this_torch_and_python(lib, monkeypatch):
+    """The module was compiled against the layout of torch's tensors: its file name carries both versions, and under another torch the
+    one that is there is neither loaded nor taken for built."""
+    import sysconfig
+    import torch
+    from paper_2605_08565_b200 import binding, build
+    here = build.native_path()
+    assert os.path.exists(here) and torch.__version__ in here and here.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    assert binding._native.__file__ == here
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert build.native_path() != here and not os.path.exists(build.native_path())
+    with pytest.raises(ImportError):
+        binding._import_native()
