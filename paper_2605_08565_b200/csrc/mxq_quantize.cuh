@@ -635,10 +635,12 @@ __device__ __forceinline__ void store_fake_chunk(const QuantArgs& p, const FakeC
 }
 
 // LEAN == 2: the same loop under a tensor scale, see lean_scaled_allowed(): the block maximum is divided by g
-// first (corrected quotient), the residual is formed in binary32.  This is the pass over activations between their abs-max and their
-// de-quantization: the elements are read for the last time and marked evict-first in L2, the codes and scales are read next and stored
-// without that mark (8192 x 4096 bf16, the three calls: 52.1 -> 49.3 us; without a tensor scale, where nothing of the kind follows, the
-// same policy costs a weight matrix 3 % and the study's scoring pass 4 %).
+// first (corrected quotient), the residual is formed in binary32, and the codes and scales are stored with L2's default policy instead of
+// evict-first: activations are de-quantized next (8192 x 4096 bf16, 4-over-6, inputs in rotation, us: abs-max, quantize,
+// de-quantize 51.3 -> 51.1, the last two 35.2 -> 34.8; a second quantization or a clipping pass behind it as before).  The elements are
+// not marked evict-first beside that: the three calls would take 49.9, but whoever reads the elements again pays for it (clipping pass
+// behind it 32.6 -> 34.4, 117 MB 52.9 -> 56.8; copy, abs-max and quantization of 117 MB 87.6 -> 91.8; two recipes on 235 MB, B = 8, UE5M3, 135 -> 142),
+// and the call cannot tell.  Without a tensor scale the default policy costs a weight matrix 3 %.
 // LEAN == 1 (launch-uniform; bf16 input, FP8 scale format, no tensor scale, every decode scale of the
 // table of class 3 -- for UE5M3 all but its last few codes, whose scales from 2^16 on are not f16
 // values: a group whose code lands there is redone on the general path): nothing of a block can leave
@@ -963,23 +965,14 @@ __device__ __forceinline__ void stage_warp_chunks(uint32_t slot_warp_addr, const
 // of a ring slot (piece k of thread t at ((slot * PIECES + k) * 256 + t) * 16), as one commit
 // group.  An empty group is committed when there is no chunk left, so that the group count per
 // loop trip stays fixed.
-// LAST_USE: the elements need not stay in L2 (see quantize_chunk(), LEAN == 2).
-template <int PIECES, bool LAST_USE = false>
+template <int PIECES>
 __device__ __forceinline__ void stage_chunk(uint32_t slot_addr, const void* src, bool valid) {
     if (valid) {
         const char* g = static_cast<const char*>(src);
-        [[maybe_unused]] unsigned long long evict_first;
-        if constexpr (LAST_USE) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(evict_first));
 #pragma unroll
-        for (int k = 0; k < PIECES; ++k) {
-            if constexpr (LAST_USE)
-                asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(slot_addr + k * (kThreads * 16)), "l"(g + 16 * k),
-                             "l"(evict_first)
-                             : "memory");
-            else
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(slot_addr + k * (kThreads * 16)), "l"(g + 16 * k)
-                             : "memory");
-        }
+        for (int k = 0; k < PIECES; ++k)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(slot_addr + k * (kThreads * 16)), "l"(g + 16 * k)
+                         : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
@@ -1329,7 +1322,7 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
             // that trip): request the chunk DIST trips ahead into it.  The slot of the current chunk
             // is not requested into before the next trip, so it may be read throughout this one.
             if constexpr (S::COOP) stage_warp_chunks<S::PIECES>(ring_warp + fill * kSlotBytes, x, kChunkBytes, ahead, p.n_items, lane);
-            else stage_chunk<S::PIECES, LEAN == 2>(ring_base + fill * kSlotBytes, x + ahead * kChunkBytes, ahead < p.n_items);
+            else stage_chunk<S::PIECES>(ring_base + fill * kSlotBytes, x + ahead * kChunkBytes, ahead < p.n_items);
             ahead += stride;
             slot = (slot + 1 == S::SLOTS) ? 0 : slot + 1;
             fill = (fill + 1 == S::SLOTS) ? 0 : fill + 1;
