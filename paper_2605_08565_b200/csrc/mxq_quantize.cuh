@@ -61,13 +61,24 @@ namespace mxq {
 //      D = 0 counts as valid with R = 0: every quotient comes out as a zero with the sign of v.
 struct QuantTables {
     float4 E[256];
-    // What the lean loops read of an entry for blocks of 2 and 4, 64 bits (fill_lean_table()).  16-byte entries at per-lane codes cost four
-    // shared-memory wavefronts and as many conflicts for every block and candidate, which is what the kernels for small blocks waited for
-    // (16.8 M bf16 elements, 128- -> 64-bit reads, us: abs-max, UE4M3, B = 2 19.0 -> 18.3, 4 13.4 -> 13.2; 4-over-6, UE4M3, B = 2 22.1 -> 20.6, 4 16.1
-    // -> 15.2; UE5M3, B = 2 29.2 -> 24.7, 4 18.7 -> 17.6; longer blocks lose 1 to 3 %, and read E).
+};
+// What the lean loops read of an entry for blocks of 2 and 4, 64 bits (fill_lean_table()).  16-byte entries at per-lane codes cost four
+// shared-memory wavefronts and as many conflicts for every block and candidate, which is what the kernels for small blocks waited for
+// (16.8 M bf16 elements, 128- -> 64-bit reads, us: abs-max, UE4M3, B = 2 19.0 -> 18.3, 4 13.4 -> 13.2; 4-over-6, UE4M3, B = 2 22.1 -> 20.6, 4 16.1
+// -> 15.2; UE5M3, B = 2 29.2 -> 24.7, 4 18.7 -> 17.6; longer blocks lose 1 to 3 %, and read E).
+struct QuantLeanTables : QuantTables {
     float2 L[256];
 };
-__host__ __device__ constexpr bool has_lean_table(int B) { return B <= 4; }
+
+// Blocks longer than 16 elements go part by part (quantize_long_block()), except 4-over-6 at B = 32, which
+// is faster with the whole block in registers (33.5 M bf16 elements: 0.775 against 0.711 of the copy bandwidth).
+__host__ __device__ constexpr bool long_block_path(int B, bool dual) { return B > 16 && !(dual && B == 32); }
+
+// Kernels with lean loops (see quantize_chunk()), and those of them whose lean loops read the short entries.
+__host__ __device__ constexpr bool can_lean(int DT, int B, int FMT, bool dual) { return DT == kBF16 && FMT != kUE8M0 && !long_block_path(B, dual); }
+__host__ __device__ constexpr bool has_lean_table(int DT, int B, int FMT) { return can_lean(DT, B, FMT, false) && B <= 4; }
+template <int DT, int B, int FMT>
+using TablesOf = std::conditional_t<has_lean_table(DT, B, FMT), QuantLeanTables, QuantTables>;
 
 // Does the FP4 code of RZ(v * R) equal the FP4 code of fl32(v / D) for EVERY bf16 value v?  (D a
 // normal binary32 number, R within a few units in the last place of 1 / D.)  Both codes are
@@ -466,15 +477,16 @@ __device__ __forceinline__ bool lean_scaled_allowed(const QuantConsts& k) {
 
 // LEAN 1: RN(1 / D) and f16(-D); LEAN 2: the checked reciprocal and D.  A barrier inside.
 template <int LEAN>
-__device__ __forceinline__ void fill_lean_table(QuantTables& T) {
+__device__ __forceinline__ void fill_lean_table(QuantLeanTables& T) {
     const float4 E = T.E[threadIdx.x];
     T.L[threadIdx.x] = LEAN == 1 ? make_float2(E.y, E.z) : make_float2(E.z, E.x);
     __syncthreads();
 }
 // The fields of an entry that encode_group_fast() and its 4-over-6 form take in a lean loop.
-template <int B, int LEAN>
-__device__ __forceinline__ float4 lean_entry(const QuantTables& T, int c) {
-    if constexpr (!has_lean_table(B)) return T.E[c];
+template <int LEAN>
+__device__ __forceinline__ float4 lean_entry(const QuantTables& T, int c) { return T.E[c]; }
+template <int LEAN>
+__device__ __forceinline__ float4 lean_entry(const QuantLeanTables& T, int c) {
     const float2 l = T.L[c];
     return LEAN == 1 ? make_float4(0.0f, l.x, l.y, 0.0f) : make_float4(l.y, 0.0f, l.x, 0.0f);
 }
@@ -653,7 +665,7 @@ __device__ __forceinline__ void store_fake_chunk(const QuantArgs& p, const FakeC
 // formats max(code_M(u), 1) = code_M(max(u, 4 eps)) for M = 6 and M = 4, eps = value(code 1)
 // (4 eps / 6 and 4 eps / 4 round to code 1; anything below rounds to 0 or 1, anything above to >= 1).
 template <int DT, int B, int FMT, bool DUAL, bool FAKE, int LEAN>
-__device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const QuantTables& T, const QuantConsts& k,
+__device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const TablesOf<DT, B, FMT>& T, const QuantConsts& k,
                                                size_t chunk, const uint32_t* raw, double& sse_sum, FakeChunk<DT, B>* fake) {
     static_assert(!LEAN || (DT == kBF16 && FMT != kUE8M0), "lean path: bf16 input, FP8 scale formats");
     using S = QuantShape<DT, B>;
@@ -695,8 +707,8 @@ __device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const QuantTa
                     c6[j] = round_scale<FMT>(w6);
                     if constexpr (DUAL) c4[j] = round_scale<FMT>(__fmul_rn(uf, 0.25f));
                 }
-                E6[j] = lean_entry<B, LEAN>(T, c6[j]);
-                if constexpr (DUAL) E4[j] = lean_entry<B, LEAN>(T, c4[j]);
+                E6[j] = lean_entry<LEAN>(T, c6[j]);
+                if constexpr (DUAL) E4[j] = lean_entry<LEAN>(T, c4[j]);
                 continue;
             }
             m[j] = a;
@@ -786,7 +798,7 @@ __device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const QuantTa
         }
         if constexpr (FAKE) {
 #pragma unroll
-            for (int j = 0; j < NBG; ++j) fake->D[gi * NBG + j] = LEAN == 1 && has_lean_table(B) ? T.E[c6[j]].x : Dw[j];   // not read so far
+            for (int j = 0; j < NBG; ++j) fake->D[gi * NBG + j] = LEAN == 1 && has_lean_table(DT, B, FMT) ? T.E[c6[j]].x : Dw[j];   // not read so far
         }
 #pragma unroll
         for (int i = 0; i < S::GE / 8; ++i) packed[gi * (S::GE / 8) + i] = pk[i];
@@ -977,10 +989,6 @@ __device__ __forceinline__ void stage_chunk(uint32_t slot_addr, const void* src,
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// Blocks longer than 16 elements go part by part (quantize_long_block()), except 4-over-6 at B = 32, which
-// is faster with the whole block in registers (33.5 M bf16 elements: 0.775 against 0.711 of the copy bandwidth).
-__host__ __device__ constexpr bool long_block_path(int B, bool dual) { return B > 16 && !(dual && B == 32); }
-
 // One block past the last whole chunk (a chunk of several blocks, B <= 16; fewer blocks than a chunk holds), by the general quotient; the
 // elements are read again for each candidate.  Out of line, to leave the registers of the kernel alone.  Returns its SSE.
 template <int DT, int B, int FMT, bool DUAL, bool FAKE>
@@ -1043,7 +1051,7 @@ __device__ __noinline__ float quantize_tail_block(const QuantArgs& p, size_t blk
 
 // Body of the multi-tensor kernel (k_quantize_batch).
 template <int DT, int B, int FMT, bool DUAL>
-__device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, QuantTables& T, uint4* ring) {
+__device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, TablesOf<DT, B, FMT>& T, uint4* ring) {
     using S = QuantShape<DT, B>;
     __shared__ uint32_t row0[kMaxBatch + 1];   // row0[t] = first row of tensor t; row0[n_tensors] = all rows
     __shared__ uint32_t warp_rows[kThreads / 32];
@@ -1101,8 +1109,8 @@ __device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, QuantTab
         k.m_lo = 0.0f;
     }
 
-    constexpr bool CAN_LEAN = (DT == kBF16) && (FMT != kUE8M0) && !(long_block_path(B, DUAL));
-    if constexpr (CAN_LEAN && has_lean_table(B)) {
+    constexpr bool CAN_LEAN = can_lean(DT, B, FMT, DUAL);
+    if constexpr (has_lean_table(DT, B, FMT)) {
         if (lean_allowed<FMT>(first_bad, k.unit_g)) fill_lean_table<1>(T);
         else if (lean_scaled_allowed(k)) fill_lean_table<2>(T);
     }
@@ -1219,7 +1227,7 @@ __global__ void __launch_bounds__(kThreads, quantize_batch_min_ctas(B)) k_quanti
     using S = QuantShape<DT, B>;
     static_assert(S::C == quantize_chunk_elems(DT, B), "host and kernel agree on the chunk size");
     extern __shared__ uint4 ring[];
-    __shared__ QuantTables T;
+    __shared__ TablesOf<DT, B, FMT> T;
     wait_for_prior_grid();
     release_dependents();
     quantize_batch_body<DT, B, FMT, DUAL>(p, T, ring);
@@ -1232,7 +1240,7 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
     using S = QuantShape<DT, B>;
     static_assert(S::C == quantize_chunk_elems(DT, B), "host and kernel agree on the chunk size");
     extern __shared__ uint4 ring[];
-    __shared__ QuantTables T;
+    __shared__ TablesOf<DT, B, FMT> T;
     {
         // While the kernel before this one in the stream drains: ask L2 for this thread's first chunk.
         // A prefetch changes no architectural state and L2 is the point of coherence, so this is safe
@@ -1295,8 +1303,8 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
     // Thread-private staging: a thread leaves when its chunks are done (no barrier follows).
     // Cooperative staging: the warp stays together, lanes past the end only take part in the copies.
     // (with fused MSE partial sums every thread stays for the CTA-wide sum at the end)
-    constexpr bool CAN_LEAN = (DT == kBF16) && (FMT != kUE8M0) && !(long_block_path(B, DUAL));
-    if constexpr (CAN_LEAN && has_lean_table(B)) {
+    constexpr bool CAN_LEAN = can_lean(DT, B, FMT, DUAL);
+    if constexpr (has_lean_table(DT, B, FMT)) {
         if (lean_allowed<FMT>(first_bad, k.unit_g)) fill_lean_table<1>(T);
         else if (lean_scaled_allowed(k)) fill_lean_table<2>(T);
     }
