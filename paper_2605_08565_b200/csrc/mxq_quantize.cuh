@@ -62,7 +62,8 @@ namespace mxq {
 struct QuantTables {
     float4 E[256];
 };
-// What the lean loops read of an entry for blocks of 2 and 4, 64 bits (fill_lean_table()).  16-byte entries at per-lane codes cost four
+// What the lean loops read of an entry for blocks of 2 and 4, 64 bits: LEAN 1 RN(1 / D) and f16(-D), LEAN 2 the checked
+// reciprocal and D.  16-byte entries at per-lane codes cost four
 // shared-memory wavefronts and as many conflicts for every block and candidate, which is what the kernels for small blocks waited for
 // (16.8 M bf16 elements, 128- -> 64-bit reads, us: abs-max, UE4M3, B = 2 19.0 -> 18.3, 4 13.4 -> 13.2; 4-over-6, UE4M3, B = 2 22.1 -> 20.6, 4 16.1
 // -> 15.2; UE5M3, B = 2 29.2 -> 24.7, 4 18.7 -> 17.6; longer blocks lose 1 to 3 %, and read E).
@@ -122,8 +123,8 @@ __device__ __forceinline__ bool one_multiply_codes_agree_at(float D, float R, fl
 // pass in every class); an entry records it only if its own significand bits are those of its class
 // (always, unless g is denormal).  If some class has no passing candidate the launch keeps the
 // corrected quotient throughout.
-template <int FMT, bool BF16_IN>
-__device__ __forceinline__ bool build_quant_tables(QuantTables& T, float g, int& first_bad) {
+template <int FMT, bool BF16_IN, typename TABLES>
+__device__ __forceinline__ bool build_quant_tables(TABLES& T, float g, int& first_bad) {
     static_assert(kThreads == 256, "one thread per table entry");
     __shared__ int leading_good[kThreads / 32];   // per warp: how many of its 32 codes, from the first on, have class 3
     __shared__ uint32_t class_sig[8];             // significand bits of fl((1 + m / 8) * g)
@@ -171,6 +172,8 @@ __device__ __forceinline__ bool build_quant_tables(QuantTables& T, float g, int&
         }
     }
     T.E[c] = make_float4(D, R, __uint_as_float(z), w);
+    if constexpr (std::is_same_v<TABLES, QuantLeanTables>)   // LEAN 2 has the check behind it, LEAN 1 has g = 1
+        T.L[c] = check ? make_float2(__uint_as_float(z), D) : make_float2(R, __uint_as_float(z));
     const uint32_t good = __ballot_sync(0xFFFFFFFFu, w == 3.0f);
     if ((c & 31) == 0) leading_good[c >> 5] = (good == 0xFFFFFFFFu) ? 32 : (__ffs(~good) - 1);
     const bool all_voted = __syncthreads_and(vote) != 0;
@@ -475,13 +478,6 @@ __device__ __forceinline__ bool lean_scaled_allowed(const QuantConsts& k) {
     return k.onemul && k.g >= 9.094947017729282379e-13f /* 2^-40 */ && k.g <= 1048576.0f;
 }
 
-// LEAN 1: RN(1 / D) and f16(-D); LEAN 2: the checked reciprocal and D.  A barrier inside.
-template <int LEAN>
-__device__ __forceinline__ void fill_lean_table(QuantLeanTables& T) {
-    const float4 E = T.E[threadIdx.x];
-    T.L[threadIdx.x] = LEAN == 1 ? make_float2(E.y, E.z) : make_float2(E.z, E.x);
-    __syncthreads();
-}
 // The fields of an entry that encode_group_fast() and its 4-over-6 form take in a lean loop.
 template <int LEAN>
 __device__ __forceinline__ float4 lean_entry(const QuantTables& T, int c) { return T.E[c]; }
@@ -1110,10 +1106,6 @@ __device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, TablesOf
     }
 
     constexpr bool CAN_LEAN = can_lean(DT, B, FMT, DUAL);
-    if constexpr (has_lean_table(DT, B, FMT)) {
-        if (lean_allowed<FMT>(first_bad, k.unit_g)) fill_lean_table<1>(T);
-        else if (lean_scaled_allowed(k)) fill_lean_table<2>(T);
-    }
     const uint32_t total_rows = row0[nt];
     const uint32_t row_stride = gridDim.x * (kThreads / 32);
     constexpr size_t kChunkBytes = (size_t)S::C * S::EB;
@@ -1304,10 +1296,6 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
     // Cooperative staging: the warp stays together, lanes past the end only take part in the copies.
     // (with fused MSE partial sums every thread stays for the CTA-wide sum at the end)
     constexpr bool CAN_LEAN = can_lean(DT, B, FMT, DUAL);
-    if constexpr (has_lean_table(DT, B, FMT)) {
-        if (lean_allowed<FMT>(first_bad, k.unit_g)) fill_lean_table<1>(T);
-        else if (lean_scaled_allowed(k)) fill_lean_table<2>(T);
-    }
     double sse_sum = 0.0;   // binary64 sum of the SSEs of this thread's blocks, in the order it produced them
     constexpr bool TOGETHER = S::COOP || FAKE;   // the warp stays together through the loop
     const bool has_work = (TOGETHER ? wchunk0 : chunk) < p.n_items;
