@@ -536,10 +536,19 @@ struct FakeChunk {
 // 32 cache lines and write half sectors (33.5 M bf16 elements, B = 32, UE8M0, bf16 out: 26.7 us, here 22.2;
 // 16.8 M bf16 elements, B = 8, 4-over-6, fp32 out 33.4, here 17.7).  So the packed codes and the decode scales (for blocks of 2, where these
 // would not fit, the scale bytes) go through the ring slot that the chunk came from, and the warp forms and stores 512 contiguous bytes at a time.
-// Not for fp32 blocks of 2, whose chunks of 16 elements hold eight scales: there a thread's run is at least a sector, and staging the scales
-// costs more than it saves (16.8 M elements, bf16 out 19.5 us, staged 21 to 27).
 // Every lane of the warp calls it.
-__host__ __device__ constexpr bool fake_stores_together(int DT, int B) { return !(DT == kF32 && B == 2); }
+// Who stores x_hat: nobody (codes, scales and SSE are stored instead), the warp together, or each thread its own.
+enum { kNoFake = 0, kFakeTogether = 1, kFakeDirect = 2 };
+// Each thread its own where its run is a sector or more and holding a chunk's scales back costs more than it saves:
+//   fp32 input (chunks of 16 elements), blocks of 2: eight scales a chunk (16.8 M elements, bf16 out 19.5 us, together 21 to 27);
+//   fp32 input, 4-over-6, bf16 output, B <= 16: together costs a resident CTA (16.8 M elements, us, together -> own: B = 4 25.9 -> 24.5,
+//   8 21.8 -> 20.9, 16 20.6 -> 19.1; with fp32 output or one candidate together is faster by 5 to 25 %);
+//   bf16 input, 4-over-6, UE8M0, bf16 output, the general loops of blocks of 2 (67 M elements 91.6 -> 86.0) and, under a tensor scale, of 16
+//   (4 M elements 7.1 -> 6.1, 67 M 60.4 -> 57.4; without one 54.3 -> 55.3).
+__host__ __device__ constexpr bool fake_direct_always(int DT, int B) { return DT == kF32 && B == 2; }
+__host__ __device__ constexpr bool fake_direct_for_bf16_out(int DT, int B, int FMT, bool dual) {
+    return dual && (DT == kF32 ? B <= 16 : FMT == kUE8M0 && (B == 2 || B == 16));
+}
 template <int DT, int B>
 __device__ __forceinline__ void store_fake_chunks(const QuantArgs& p, const QuantTables& T, const FakeChunk<DT, B>& f, size_t wchunk, int n_valid,
                                                   uint4* slot_warp, int lane) {
@@ -616,29 +625,24 @@ __device__ __forceinline__ void store_fake_chunks(const QuantArgs& p, const Quan
     else store_units(std::integral_constant<bool, false>{});
 }
 
-// The same by the thread itself.
-template <int DT, int B>
-__device__ __forceinline__ void store_fake_chunk(const QuantArgs& p, const FakeChunk<DT, B>& f, size_t chunk) {
-    using S = QuantShape<DT, B>;
+// The same by the thread itself, group by group (kFakeDirect): eight elements and the decode scales of their blocks.
+template <int B>
+__device__ __forceinline__ void store_fake_direct(const QuantArgs& p, size_t e0, uint32_t codes, const float* D) {
+    float q[8];
+    unpack_e2m1x8(codes, q);
+    uint32_t o[8];
 #pragma unroll
-    for (int w8 = 0; w8 < S::C / 8; ++w8) {
-        float q[8];
-        unpack_e2m1x8(f.codes[w8], q);
-        uint32_t o[8];
+    for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(__fmul_rn(q[i], D[i / B]));
+    if (p.xhat_dtype == kF32) {
+        store_bytes<32>(static_cast<float*>(p.xhat) + e0, o);
+    } else {
+        uint32_t h[4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(__fmul_rn(q[i], f.D[(8 * w8 + i) / B]));
-        const size_t e0 = chunk * S::C + 8 * w8;
-        if (p.xhat_dtype == kF32) {
-            store_bytes<32>(static_cast<float*>(p.xhat) + e0, o);
-        } else {
-            uint32_t h[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(o[2 * i]), __uint_as_float(o[2 * i + 1]));
-                h[i] = *reinterpret_cast<const uint32_t*>(&b2);
-            }
-            store_bytes<16>(static_cast<__nv_bfloat16*>(p.xhat) + e0, h);
+        for (int i = 0; i < 4; ++i) {
+            const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(o[2 * i]), __uint_as_float(o[2 * i + 1]));
+            h[i] = *reinterpret_cast<const uint32_t*>(&b2);
         }
+        store_bytes<16>(static_cast<__nv_bfloat16*>(p.xhat) + e0, h);
     }
 }
 
@@ -660,7 +664,7 @@ __device__ __forceinline__ void store_fake_chunk(const QuantArgs& p, const FakeC
 // above it both formats saturate.  Prevent-zero is a floor on the block maximum: for both
 // formats max(code_M(u), 1) = code_M(max(u, 4 eps)) for M = 6 and M = 4, eps = value(code 1)
 // (4 eps / 6 and 4 eps / 4 round to code 1; anything below rounds to 0 or 1, anything above to >= 1).
-template <int DT, int B, int FMT, bool DUAL, bool FAKE, int LEAN>
+template <int DT, int B, int FMT, bool DUAL, int FAKE, int LEAN>
 __device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const TablesOf<DT, B, FMT>& T, const QuantConsts& k,
                                                size_t chunk, const uint32_t* raw, double& sse_sum, FakeChunk<DT, B>* fake) {
     static_assert(!LEAN || (DT == kBF16 && FMT != kUE8M0), "lean path: bf16 input, FP8 scale formats");
@@ -792,7 +796,12 @@ __device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const TablesO
                 pk[0] = (pk4[0] & take) | (pk[0] & ~take);
             }
         }
-        if constexpr (FAKE) {
+        if constexpr (FAKE == kFakeDirect) {
+            static_assert(!LEAN, "the lean loops do not read D");
+#pragma unroll
+            for (int i = 0; i < S::GE / 8; ++i)
+                store_fake_direct<B>(p, chunk * S::C + (size_t)gi * S::GE + 8 * i, pk[i], Dw + (B < 8 ? 0 : 8 * i / B));
+        } else if constexpr (FAKE) {
 #pragma unroll
             for (int j = 0; j < NBG; ++j) fake->D[gi * NBG + j] = LEAN == 1 && has_lean_table(DT, B, FMT) ? T.E[c6[j]].x : Dw[j];   // not read so far
         }
@@ -806,6 +815,7 @@ __device__ __forceinline__ void quantize_chunk(const QuantArgs& p, const TablesO
             if constexpr (!FAKE) sse_sum = __dadd_rn(sse_sum, (double)sse[j]);
         }
     }
+    if constexpr (FAKE == kFakeDirect) return;
     if constexpr (FAKE) {
 #pragma unroll
         for (int i = 0; i < S::C / 8; ++i) fake->codes[i] = packed[i];
@@ -838,12 +848,12 @@ __device__ __forceinline__ uint32_t absmax_bf16x2(uint32_t a, uint32_t b) {
 // elements read from the thread's ring slot, which stays valid until the next trip's request:
 // once for the block maximum, once for the encode with the SSE chains carried from part to part.
 // Only one part is live in registers at a time, which keeps as many CTAs resident as for B = 16.
-template <int DT, int B, int FMT, bool DUAL, bool FAKE>
+template <int DT, int B, int FMT, bool DUAL, int FAKE>
 __device__ __forceinline__ void quantize_long_block(const QuantArgs& p, const QuantTables& T, const QuantConsts& k,
                                                     size_t chunk, const uint4* slot_warp, int lane, double& sse_sum,
                                                     FakeChunk<DT, B>* fake) {
     using S = QuantShape<DT, B>;
-    static_assert(S::C == B && S::NBC == 1, "one block per chunk");
+    static_assert(S::C == B && S::NBC == 1 && FAKE != kFakeDirect, "one block per chunk");
     constexpr int SG = 16;                        // elements per part
     constexpr int NSG = B / SG;
     constexpr int PPS = SG * S::EB / 16;          // 16-byte pieces per part
@@ -987,7 +997,7 @@ __device__ __forceinline__ void stage_chunk(uint32_t slot_addr, const void* src,
 
 // One block past the last whole chunk (a chunk of several blocks, B <= 16; fewer blocks than a chunk holds), by the general quotient; the
 // elements are read again for each candidate.  Out of line, to leave the registers of the kernel alone.  Returns its SSE.
-template <int DT, int B, int FMT, bool DUAL, bool FAKE>
+template <int DT, int B, int FMT, bool DUAL, int FAKE>
 __device__ __noinline__ float quantize_tail_block(const QuantArgs& p, size_t blk, float g, int c_min, int pow2_rule) {
     auto pair = [&](int i) {
         float v[2];
@@ -1179,7 +1189,7 @@ __device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, TablesOf
             const size_t chunk = (size_t)(row - cur_c.first) * 32 + lane;
             if (chunk >= cur_c.n_chunks) continue;      // a lane past the end of the tensor's last row
             if constexpr (long_block_path(B, DUAL)) {
-                quantize_long_block<DT, B, FMT, DUAL, false>(pl, T, k, chunk, slot_warp, lane, unused_sum, nullptr);
+                quantize_long_block<DT, B, FMT, DUAL, kNoFake>(pl, T, k, chunk, slot_warp, lane, unused_sum, nullptr);
             } else {
                 uint32_t raw[S::PIECES * 4];
 #pragma unroll
@@ -1187,7 +1197,7 @@ __device__ __forceinline__ void quantize_batch_body(const QuantArgs& p, TablesOf
                     const uint4 w = slot_warp[ring_index<S::COOP>(q, lane)];
                     raw[4 * q + 0] = w.x; raw[4 * q + 1] = w.y; raw[4 * q + 2] = w.z; raw[4 * q + 3] = w.w;
                 }
-                quantize_chunk<DT, B, FMT, DUAL, false, LEAN>(pl, T, k, chunk, raw, unused_sum, nullptr);
+                quantize_chunk<DT, B, FMT, DUAL, kNoFake, LEAN>(pl, T, k, chunk, raw, unused_sum, nullptr);
             }
         }
     };
@@ -1227,7 +1237,7 @@ __global__ void __launch_bounds__(kThreads, quantize_batch_min_ctas(B)) k_quanti
 
 // TAIL: with blocks past the last whole chunk.  An instantiation of its own: the call that takes care of them costs the chunk loop of some
 // others registers (fp32, B = 16, abs-max, 16.8 M elements 15.7 -> 16.0 us without a single such block).
-template <int DT, int B, int FMT, bool DUAL, bool FAKE, bool TAIL>
+template <int DT, int B, int FMT, bool DUAL, int FAKE, bool TAIL>
 __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ QuantArgs p) {
     using S = QuantShape<DT, B>;
     static_assert(S::C == quantize_chunk_elems(DT, B), "host and kernel agree on the chunk size");
@@ -1297,7 +1307,7 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
     // (with fused MSE partial sums every thread stays for the CTA-wide sum at the end)
     constexpr bool CAN_LEAN = can_lean(DT, B, FMT, DUAL);
     double sse_sum = 0.0;   // binary64 sum of the SSEs of this thread's blocks, in the order it produced them
-    constexpr bool TOGETHER = S::COOP || FAKE;   // the warp stays together through the loop
+    constexpr bool TOGETHER = S::COOP || FAKE == kFakeTogether;   // the warp stays together through the loop
     const bool has_work = (TOGETHER ? wchunk0 : chunk) < p.n_items;
     if (!has_work && (FAKE || p.mse_partials == nullptr) && !TAIL) return;
     // The chunk loop, instantiated with and without the lean per-block path (see quantize_chunk);
@@ -1322,11 +1332,11 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
             ahead += stride;
             slot = (slot + 1 == S::SLOTS) ? 0 : slot + 1;
             fill = (fill + 1 == S::SLOTS) ? 0 : fill + 1;
-            if (S::COOP && !FAKE && chunk >= p.n_items) continue;   // a lane past the end (the warp's last trip)
+            if (S::COOP && FAKE != kFakeTogether && chunk >= p.n_items) continue;   // a lane past the end (the warp's last trip)
             FakeChunk<DT, B> fake;
             // blocks longer than 16 elements go part by part, except 4-over-6 at B = 32, which measured
             // slightly faster with the whole block in registers
-            if (!FAKE || chunk < p.n_items) {
+            if (FAKE != kFakeTogether || chunk < p.n_items) {
                 if constexpr (long_block_path(B, DUAL)) {
                     quantize_long_block<DT, B, FMT, DUAL, FAKE>(p, T, k, chunk, slot_warp, lane, sse_sum, &fake);
                 } else {
@@ -1339,11 +1349,9 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
                     quantize_chunk<DT, B, FMT, DUAL, FAKE, LEAN>(p, T, k, chunk, raw, sse_sum, &fake);
                 }
             }
-            if constexpr (FAKE && fake_stores_together(DT, B)) {
+            if constexpr (FAKE == kFakeTogether) {
                 const size_t left = p.n_items - lead;
                 store_fake_chunks<DT, B>(p, T, fake, lead, left < 32 ? (int)left : 32, slot_warp, lane);
-            } else if constexpr (FAKE) {
-                if (chunk < p.n_items) store_fake_chunk<DT, B>(p, fake, chunk);
             }
         }
     };
@@ -1375,7 +1383,7 @@ __global__ void __launch_bounds__(kThreads) k_quantize(const __grid_constant__ Q
 }
 
 // Host side: pick the instantiation and launch a persistent grid over the whole chunks and the blocks behind them.
-template <int DT, int B, int FMT, bool DUAL, bool FAKE, bool TAIL>
+template <int DT, int B, int FMT, bool DUAL, int FAKE, bool TAIL>
 static cudaError_t launch_quantize_inst(const QuantArgs& a, cudaStream_t stream) {
     using S = QuantShape<DT, B>;
     static std::atomic<int> ctas_per_sm[kMaxDevices];   // first-use cache; racing threads store the same value
@@ -1408,13 +1416,33 @@ static cudaError_t launch_quantize_inst(const QuantArgs& a, cudaStream_t stream)
     return err;
 }
 
-template <int DT, int B, int FMT, bool FAKE>
-static cudaError_t launch_quantize_kind(const QuantArgs& a, bool dual, cudaStream_t s) {
+template <int DT, int B, int FMT, bool DUAL, int FAKE>
+static cudaError_t launch_quantize_tail(const QuantArgs& a, cudaStream_t s) {
     using S = QuantShape<DT, B>;
     if constexpr (S::NBC > 1) {
-        if (a.n_items % S::NBC != 0) return dual ? launch_quantize_inst<DT, B, FMT, true, FAKE, true>(a, s) : launch_quantize_inst<DT, B, FMT, false, FAKE, true>(a, s);
+        if (a.n_items % S::NBC != 0) return launch_quantize_inst<DT, B, FMT, DUAL, FAKE, true>(a, s);
     }
-    return dual ? launch_quantize_inst<DT, B, FMT, true, FAKE, false>(a, s) : launch_quantize_inst<DT, B, FMT, false, FAKE, false>(a, s);
+    return launch_quantize_inst<DT, B, FMT, DUAL, FAKE, false>(a, s);
+}
+
+template <int DT, int B, int FMT, bool DUAL, bool FAKE>
+static cudaError_t launch_quantize_store(const QuantArgs& a, cudaStream_t s) {
+    if constexpr (!FAKE) {
+        return launch_quantize_tail<DT, B, FMT, DUAL, kNoFake>(a, s);
+    } else if constexpr (fake_direct_always(DT, B)) {
+        return launch_quantize_tail<DT, B, FMT, DUAL, kFakeDirect>(a, s);
+    } else {
+        if constexpr (fake_direct_for_bf16_out(DT, B, FMT, DUAL)) {
+            const bool scaled = a.d_global_scale != nullptr || a.global_scale != 1.0f;
+            if (a.xhat_dtype == kBF16 && (DT == kF32 || B == 2 || scaled)) return launch_quantize_tail<DT, B, FMT, DUAL, kFakeDirect>(a, s);
+        }
+        return launch_quantize_tail<DT, B, FMT, DUAL, kFakeTogether>(a, s);
+    }
+}
+
+template <int DT, int B, int FMT, bool FAKE>
+static cudaError_t launch_quantize_kind(const QuantArgs& a, bool dual, cudaStream_t s) {
+    return dual ? launch_quantize_store<DT, B, FMT, true, FAKE>(a, s) : launch_quantize_store<DT, B, FMT, false, FAKE>(a, s);
 }
 
 template <int DT, int B, bool FAKE>

@@ -211,6 +211,28 @@ def test_fake_quantize_equals_quantize_then_dequantize(dtype, B):
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B", [2, 4, 8, 16, 32, 64])
+def test_fake_quantize_of_several_trips(dtype, B):
+    """Several chunks for every warp, the last warp partial and blocks past the last whole chunk: the copies of a later trip go to
+    the memory that the lanes of an earlier one stored their codes and scales in.  Both stores (each thread its own, the warp together),
+    both outputs, and in place."""
+    chunk = max(B, 16 if dtype == torch.float32 else 32)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = chunk * (3 * 4 * sms * 256 + 5 * 256 + 77) + (chunk // B - 1) * B      # three trips of four resident CTAs per SM
+    x = inputs.student_t(n, 4, 0.05, 51 + B, dtype, "cuda")
+    for fmt, recipe, g in ((mxq.MXQ_SF_UE4M3, mxq.MXQ_ABSMAX, 1.0), (mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6_PZ, 0.0131),
+                           (mxq.MXQ_SF_UE5M3, mxq.MXQ_4O6, 1.0), (mxq.MXQ_SF_UE8M0, mxq.MXQ_4O6, 0.0131), (mxq.MXQ_SF_UE8M0, mxq.MXQ_4O6, 1.0)):
+        codes, scales, _ = mxq.quantize(x, B, fmt, recipe, g)
+        for odt, bits in ((torch.float32, torch.int32), (torch.bfloat16, torch.int16)):
+            want = torch.empty(n, dtype=odt, device="cuda")
+            mxq.mxq_dequantize(codes, scales, n, B, fmt, g, want)
+            out = x.clone() if odt == dtype else torch.full((n,), float("nan"), dtype=odt, device="cuda")
+            mxq.mxq_fake_quantize(out if odt == dtype else x, n, B, fmt, recipe, g, None, out)
+            torch.cuda.synchronize()
+            assert torch.equal(out.view(bits), want.view(bits)), (fmt, recipe, g, odt)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_mask_interval_matches_definition(dtype):
     for n in (1, 7, 8, 4096 + 5):
         x = (inputs.normal(max(n, 8), 4 + n, 0.02, torch.float32)[:n]).to(dtype).contiguous()
