@@ -286,11 +286,21 @@ __device__ __forceinline__ float decode_scale(int fmt, int c, float g) {
 // codes + scales + output; a plain fill of the same output alone takes 82 us) whatever was tried -- plain
 // instead of streaming stores, 4, 8 or 16 resident CTAs per SM, grid-stride or CTA-contiguous tiles, with
 // or without the table and the early loads; those two shorten B = 2 by about 5 % and were kept.
-template <int ODT>
+// EARLY: the first loads are issued before the table is built, else between the table and its barrier.  Early is right from the third trip of a
+// CTA on, behind it up to the second (launch_dequantize() counts them; B = 16, us, early / behind: bf16 out 2.1 M elements 2.65 / 2.39, 8.4 M
+// 5.6 / 5.0, 67 M 32.7 / 33.8 or more; fp32 out 4.2 M 5.0 / 4.4, 67 M 56.3 / 57.4).
+template <int ODT, bool EARLY>
 __global__ void __launch_bounds__(kThreads) k_dequantize(const uint8_t* codes, const uint8_t* scales, size_t n,
                                                          int log2B, int fmt, float g_host, const float* d_g, void* out) {
     wait_for_prior_grid();
     release_dependents();
+    // decode scales of all 256 codes, one per thread: a table read replaces a dozen instructions per unit
+    __shared__ float Dtab[256];
+    auto build_table = [&] {
+        const float g = d_g ? *d_g : g_host;   // device-resident tensor scale (written by an earlier kernel of the stream)
+        Dtab[threadIdx.x] = decode_scale(fmt, (int)threadIdx.x, g);
+    };
+    if constexpr (!EARLY) build_table();
     constexpr int E = (ODT == kF32) ? 4 : 8;      // elements per unit
     constexpr int LOG2E = (ODT == kF32) ? 2 : 3;
     constexpr int U = 4;
@@ -317,10 +327,7 @@ __global__ void __launch_bounds__(kThreads) k_dequantize(const uint8_t* codes, c
     size_t base = (size_t)blockIdx.x * (U * kThreads) + threadIdx.x;
     uint32_t w[U], sc[U];
     load_trip(base, w, sc);
-    // decode scales of all 256 codes, one per thread, while the first loads are on their way: a table read replaces a dozen instructions per unit
-    const float g = d_g ? *d_g : g_host;   // device-resident tensor scale (written by an earlier kernel of the stream)
-    __shared__ float Dtab[256];
-    Dtab[threadIdx.x] = decode_scale(fmt, (int)threadIdx.x, g);
+    if constexpr (EARLY) build_table();
     __syncthreads();
     for (; base < n_units; base += stride * U) {
         uint32_t wn[U], scn[U];
@@ -382,8 +389,10 @@ cudaError_t launch_dequantize(const uint8_t* codes, const uint8_t* scales, size_
     if (want == 0) want = 1;
     const size_t cap = (size_t)sm_count(dev) * 8;
     const unsigned grid = (unsigned)(want < cap ? want : cap);
-    if (out_dtype == kF32) err = launch_pdl(k_dequantize<kF32>, grid, kThreads, 0, s, codes, scales, n, log2B, fmt, g, d_g, out);
-    else err = launch_pdl(k_dequantize<kBF16>, grid, kThreads, 0, s, codes, scales, n, log2B, fmt, g, d_g, out);
+    const bool early = want > 2 * cap;
+    auto* const kernel = out_dtype == kF32 ? (early ? k_dequantize<kF32, true> : k_dequantize<kF32, false>)
+                                           : (early ? k_dequantize<kBF16, true> : k_dequantize<kBF16, false>);
+    err = launch_pdl(kernel, grid, (unsigned)kThreads, 0, s, codes, scales, n, log2B, fmt, g, d_g, out);
     count_launch();
     return err;
 }

@@ -609,6 +609,29 @@ def test_both_searches_agree_on_blocks_with_a_nan(dtype, B):
                 assert np.array_equal(full.view(np.uint8), pruned.view(np.uint8)), (fmt, recipe, g)
 
 
+@pytest.mark.parametrize("odt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B", [2, 16])
+def test_dequantize_where_its_loads_move(odt, B):
+    """Two trips of every CTA and the first block of a third, where the first loads go before the table of decode scales: against the
+    products formed by torch, in binary32 like the kernel's."""
+    per_cta = 1024 * (4 if odt == torch.float32 else 8)
+    limit = 2 * 8 * torch.cuda.get_device_properties(0).multi_processor_count * per_cta
+    gen = torch.Generator(device="cuda").manual_seed(B)
+    grid = torch.tensor([0.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, 6.0], device="cuda")
+    grid = torch.cat([grid, -grid])
+    value = torch.tensor([orc.scale_value(mxq.MXQ_SF_UE4M3, c) for c in range(127)], dtype=torch.float32, device="cuda")
+    g = torch.tensor([0.0131], device="cuda")
+    for n in (limit - B, limit, limit + B, limit + 2 * per_cta + B):
+        codes = torch.randint(0, 256, (n // 2,), dtype=torch.uint8, device="cuda", generator=gen)
+        scales = torch.randint(0, 127, (n // B,), dtype=torch.uint8, device="cuda", generator=gen)
+        out = torch.empty(n, dtype=odt, device="cuda")
+        mxq.mxq_dequantize_ex(codes, scales, n, B, mxq.MXQ_SF_UE4M3, 1.0, g, out)
+        q = grid[torch.stack([codes & 15, codes >> 4], 1).reshape(-1).long()].view(-1, B)
+        want = (q * (value * g)[scales.long()].view(-1, 1)).reshape(-1).to(odt)
+        bits = torch.int32 if odt == torch.float32 else torch.int16
+        assert torch.equal(out.view(bits), want.view(bits)), n
+
+
 def test_device_resident_global_scale_matches_host_scale():
     x = _mixed(8192, 5, torch.bfloat16)
     for recipe in (mxq.MXQ_ABSMAX, mxq.MXQ_4O6, mxq.MXQ_BRUTE):
