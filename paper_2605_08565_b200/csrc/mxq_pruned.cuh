@@ -23,7 +23,7 @@
 //   fp32 Laplace, tensor scale, UE4M3   B = 2 186 -> 62    4 124 -> 52   8 107 -> 48   16 109 -> 53   32 123 -> 54   64 145 -> 60
 //   bf16 Student-t, UE5M3               B = 2 205 -> 60    4 128 -> 43   8 99 -> 37    16 92 -> 36    32 92 -> 34    64 106 -> 38
 //   bf16 Student-t, UE4M3 (scale codes below 16)
-//                                       B = 2 217 -> 148   4 129 -> 98   8 91 -> 68    16 79 -> 52    32 80 -> 48    64 97 -> 51
+//                                       B = 2 217 -> 124   4 129 -> 85   8 91 -> 68    16 79 -> 52    32 80 -> 48    64 97 -> 51
 //   bf16 Student-t, UE8M0               B = 2 64 -> 36     4 51 -> 28    8 40 -> 21    16 31 -> 16    32 25 -> 15    64 27 -> 18
 // 65 K elements, B = 16, 8.0 -> 4.8.
 #pragma once
@@ -331,11 +331,16 @@ __device__ __forceinline__ bool search_codes(const float4* tab, const float2 (&v
         const int end = min(15, floor_code<FMT>(__fmul_rn(u, limit)) + (limit > 2.0f ? 1 : 0));
         in_range &= tab[1].z != 0.0f;
         uint32_t left = 0;
+        const int begin = (max(top, 1) + 1) | 1;
+        if constexpr (B <= 4) {   // so few elements are evaluated in less than the largest takes to be looked at
+            left = (0xAAAAu >> begin << begin) & ((2u << max(end, 0)) - 1u);
+        } else {
 #pragma unroll 1
-        for (int c = (max(top, 1) + 1) | 1; c <= end; c += 2) {
-            const float nD = tab[c].x;   // a rounded product: next to a midpoint of the grid the error of either side is the same to 2^-16
-            const float e = __fmaf_rn(round_widen_pair(make_float2(__fmul_rn(a, tab[c].z), 0.0f)).x, nD, a);
-            if (!(__float_as_uint(__fmul_rn(__fmul_rn(e, 0.999f), e)) > best_bits)) left |= 1u << c;
+            for (int c = begin; c <= end; c += 2) {
+                const float nD = tab[c].x;   // a rounded product: next to a midpoint of the grid the error of either side is the same to 2^-16
+                const float e = __fmaf_rn(round_widen_pair(make_float2(__fmul_rn(a, tab[c].z), 0.0f)).x, nD, a);
+                if (!(__float_as_uint(__fmul_rn(__fmul_rn(e, 0.999f), e)) > best_bits)) left |= 1u << c;
+            }
         }
 #pragma unroll 1
         while (left != 0) {
