@@ -23,7 +23,7 @@
 //   fp32 Laplace, tensor scale, UE4M3   B = 2 186 -> 62    4 124 -> 52   8 107 -> 48   16 109 -> 53   32 123 -> 54   64 145 -> 60
 //   bf16 Student-t, UE5M3               B = 2 205 -> 60    4 128 -> 43   8 99 -> 37    16 92 -> 36    32 92 -> 34    64 106 -> 38
 //   bf16 Student-t, UE4M3 (scale codes below 16)
-//                                       B = 2 217 -> 124   4 129 -> 85   8 91 -> 68    16 79 -> 52    32 80 -> 48    64 97 -> 51
+//                                       B = 2 218 -> 118   4 127 -> 84   8 91 -> 68    16 79 -> 52    32 80 -> 48    64 97 -> 51
 //   bf16 Student-t, UE8M0               B = 2 64 -> 36     4 51 -> 28    8 40 -> 21    16 31 -> 16    32 25 -> 15    64 27 -> 18
 // 65 K elements, B = 16, 8.0 -> 4.8.
 #pragma once
@@ -550,10 +550,6 @@ __device__ __forceinline__ unsigned long long pow2_search(const float2 (&v2)[B /
     // 2^c0 <= a / 6g < 2^(c0 + 1), to within the rounding: code c0 + 2 and all above it are beyond 2 a / 7
     try_two(0);
     const uint32_t ubits = (uint32_t)(best >> 32);
-    if (ubits > 0x7F800000u) {   // a NaN element: so is every SSE, no rule ends the search, and the codes it would end at are out of the shortcuts' range
-        fast = false;
-        return sse_key(__uint_as_float(ubits), 0);
-    }
     for (int k = -1; c0 + k >= 0; --k) {
         const float nD = shifted(nD0, k), R = shifted(R0, -k);
         const float e = __fmaf_rn(6.0f, nD, a);
@@ -565,6 +561,10 @@ __device__ __forceinline__ unsigned long long pow2_search(const float2 (&v2)[B /
             z = __fmaf_rn(x, x, z);
         }
         if (__float_as_uint(z) > ubits) break;
+        if (ubits > 0x7F800000u) {   // a NaN element: so is every SSE, no rule ends the search, and the codes it would end at are out of the shortcuts' range
+            fast = false;
+            return sse_key(__uint_as_float(ubits), 0);
+        }
         best = min(best, sse_key(pow2_sse_two<B, POW2>(v2, nD, R, nD, R).x, c0 + k));
     }
     return best;
