@@ -128,15 +128,15 @@ def test_brute_force_on_warps_of_unlike_blocks(B, fmt, sweep_mode):
 @pytest.mark.parametrize("B", BLOCKS)
 @pytest.mark.parametrize("fmt", FMTS)
 def test_pruned_sweep_at_the_edges_of_its_bounds(dtype, B, fmt):
-    """Tensors of one block, of part of a store unit and of a few thousand blocks (in tiles of 32 to 64, which is what tensors of
-    this size are cut into); blocks whose bounds leave nearly every code (several elements far above the largest decode
+    """Tensors of one block, of part of a unit (eight elements, or a block), of parts of a warp's 32 units and of more units than the
+    threads of one CTA; blocks whose bounds leave nearly every code (several elements far above the largest decode
     scale), whose codes are subnormal, whose elements are exact grid multiples of a scale (the bounds are met with equality),
     and blocks and tensor scales outside the shortcuts' ranges."""
-    tile = 512 if B == 16 else max(256, 4096 // B)     # blocks of a full tile
+    many = 512 if B == 16 else max(256, 4096 // B)
     gen = torch.Generator().manual_seed(77 + B + fmt)
     mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 1)
     try:
-        for nb in (1, 2, 3, 31, tile + 1, 3 * tile + 5):
+        for nb in (1, 2, 3, 31, many + 1, 3 * many + 5):
             x = inputs.student_t(nb * B, 4, 0.05, 31 + nb, torch.float32).view(nb, B)
             x[1::9] *= 2.0 ** 26                       # above 6 times the top scale
             x[2::9] = x[2::9].sign() * 2.0 ** 24       # all elements equal and above it
@@ -187,8 +187,8 @@ def test_pruned_search_around_its_first_and_last_code(dtype, B, fmt):
 @pytest.mark.parametrize("B", BLOCKS)
 @pytest.mark.parametrize("fmt", FMTS)
 def test_both_searches_on_tensors_that_fill_the_chip(dtype, B, fmt):
-    """5.2 million elements on 148 SMs: the full sweep's kernels without a split, their last group partial, and more full tiles of
-    the pruned search than CTAs, the last one partial.  Hard blocks dense at the start, in the middle and at the end and
+    """5.2 million elements on 148 SMs: the full sweep's kernels without a split, their last group partial, and more units
+    of the pruned search than threads on the chip, the last one partial.  Hard blocks dense at the start, in the middle and at the end and
     sprinkled over the rest.  The two searches give the same bytes everywhere (but for blocks with a NaN or an infinity);
     the hard blocks and the end agree with the oracle, and the fused MSE with the block SSEs."""
     nb = torch.cuda.get_device_properties(0).multi_processor_count * 35200 // B + 13
@@ -288,7 +288,7 @@ def test_full_sweep_around_the_limits_of_its_split(B, fmt, g):
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_tensor_amax_around_the_limit_of_one_cta(dtype):
-    """One launch of one CTA up to 256 KB, two kernels beyond: the largest magnitude at the first, the last and a middle
+    """One launch of one CTA up to 256 KB, one of many beyond, two under capture: the largest magnitude at the first, the last and a middle
     element, ragged ends, and a tensor of zeros (tensor scale 1)."""
     limit = 256 * 1024 // (4 if dtype == torch.float32 else 2)
     for n in (1, 7, 8, 4097, 16385, limit - 1, limit, limit + 1):
@@ -300,6 +300,14 @@ def test_tensor_amax_around_the_limit_of_one_cta(dtype):
             assert float(amax.cpu()) == 7.25 and float(g.cpu()) == np.float32(7.25) / np.float32(2688.0)
     mxq.mxq_tensor_amax(torch.zeros(100, dtype=dtype, device="cuda"), 100, amax, g)
     assert float(amax.cpu()) == 0.0 and float(g.cpu()) == 1.0
+    x = torch.zeros(limit + 1, dtype=dtype, device="cuda")
+    before = mxq.mxq_launch_count()
+    mxq.mxq_tensor_amax(x, limit + 1, amax, g)
+    assert mxq.mxq_launch_count() == before + 1
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        mxq.mxq_tensor_amax(x, limit + 1, amax, g)
+    assert mxq.mxq_launch_count() == before + 3
 
 
 def test_option_calls_reject_bad_arguments():
@@ -607,6 +615,57 @@ def test_both_searches_agree_on_blocks_with_a_nan(dtype, B):
                     mxq.mxq_set_option(mxq.MXQ_OPT_BRUTE_PRUNE, 0)
             for full, pruned in zip(out[0][:3], out[1][:3]):
                 assert np.array_equal(full.view(np.uint8), pruned.view(np.uint8)), (fmt, recipe, g)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B", [2, 4, 8, 16])
+def test_blocks_past_the_last_whole_chunk(dtype, B):
+    """Every number of such blocks behind no chunk at all, behind 255 (the first of them on the CTA's last thread) and behind one chunk less
+    than fills a persistent grid of up to six CTAs per SM a whole number of times (they go round from the grid's last thread to
+    its first).  The end of the tensor against the oracle, the chunks against a call without the rest, nothing written behind the
+    outputs, the fused MSE against the block SSEs, both fake-quantize outputs against the de-quantization."""
+    chunk = 16 if dtype == torch.float32 else 32
+    many = 60 * torch.cuda.get_device_properties(0).multi_processor_count * 256 - 1
+    nbc = chunk // B
+    if nbc == 1:
+        return                               # a chunk is a block
+    x_all = inputs.student_t((many + 1) * chunk, 4, 0.05, 61 + B, dtype, "cuda")
+    mse = torch.empty(1, dtype=torch.float64, device="cuda")
+    ws = torch.empty(mxq.mxq_tensor_mse_workspace_bytes(1) // 8, dtype=torch.float64, device="cuda")
+    guard = 64
+
+    def call(x, n, fmt, recipe, g):
+        out = [torch.full((n // 2 + guard,), 0xA5, dtype=torch.uint8, device="cuda"),
+               torch.full((n // B + guard,), 0xA5, dtype=torch.uint8, device="cuda"),
+               torch.full((n // B + guard,), float("nan"), dtype=torch.float32, device="cuda")]
+        mxq.mxq_quantize_mse(x, n, B, fmt, recipe, g, None, *out, mse, ws)
+        assert (out[0][n // 2:] == 0xA5).all() and (out[1][n // B:] == 0xA5).all() and out[2][n // B:].isnan().all()
+        return out[0][:n // 2], out[1][:n // B], out[2][:n // B]
+
+    for chunks in (0, 255, many):
+        for tail in ((1, nbc - 1) if chunks == many else range(1, nbc)):
+            n = chunks * chunk + tail * B
+            x = x_all[:n]
+            end = min(n, 256 * chunk + tail * B)             # elements compared with the oracle
+            for fmt, recipe, g in ((mxq.MXQ_SF_UE4M3, mxq.MXQ_4O6_PZ, 1.0), (mxq.MXQ_SF_UE5M3, mxq.MXQ_4O6, 0.0131),
+                                   (mxq.MXQ_SF_UE4M3, mxq.MXQ_ABSMAX, 0.0131), (mxq.MXQ_SF_UE8M0, mxq.MXQ_ABSMAX_OCP, 1.0)):
+                codes, scales, sse = call(x, n, fmt, recipe, g)
+                total = float(sse.double().sum() / n)
+                assert abs(float(mse) - total) <= 1e-12 * total, (chunks, tail, fmt, recipe)
+                oc, os_, oe = orc.quantize(inputs.to_numpy_bits(x[n - end:].clone()), B, fmt, recipe, g, threads=8)
+                assert np.array_equal(scales[(n - end) // B:].cpu().numpy(), os_), (chunks, tail, fmt, recipe)
+                assert np.array_equal(codes[(n - end) // 2:].cpu().numpy(), oc), (chunks, tail, fmt, recipe)
+                assert np.array_equal(sse[(n - end) // B:].cpu().numpy().view(np.uint32), oe.view(np.uint32)), (chunks, tail, fmt, recipe)
+                if chunks:
+                    m = chunks * chunk
+                    c2, s2, e2 = call(x[:m], m, fmt, recipe, g)
+                    assert torch.equal(codes[:m // 2], c2) and torch.equal(scales[:m // B], s2) and torch.equal(sse[:m // B], e2)
+                for odt, bits in ((torch.float32, torch.int32), (torch.bfloat16, torch.int16)):
+                    want = torch.empty(n, dtype=odt, device="cuda")
+                    mxq.mxq_dequantize(codes, scales, n, B, fmt, g, want)
+                    out = torch.full((n + guard,), float("nan"), dtype=odt, device="cuda")
+                    mxq.mxq_fake_quantize(x, n, B, fmt, recipe, g, None, out)
+                    assert torch.equal(out[:n].view(bits), want.view(bits)) and out[n:].isnan().all(), (chunks, tail, fmt, recipe, odt)
 
 
 @pytest.mark.parametrize("odt", [torch.float32, torch.bfloat16])
