@@ -284,7 +284,8 @@ __device__ __forceinline__ float decode_scale(int fmt, int c, float g) {
 // units per thread and trip, and the loads of the next trip issued before this trip's stores, keep
 // eight independent loads in flight.  Measured on 134 M elements: 110 to 115 us for fp32 output (5.4 TB/s of
 // codes + scales + output; a plain fill of the same output alone takes 82 us) whatever was tried -- plain
-// instead of streaming stores, 4, 8 or 16 resident CTAs per SM, grid-stride or CTA-contiguous tiles, with
+// instead of streaming stores, grids of 4, 8 or 16 CTAs per SM (five are resident with fp32 output, four with bf16), grid-stride or
+// CTA-contiguous tiles, with
 // or without the table and the early loads; those two shorten B = 2 by about 5 % and were kept.
 // EARLY: the first loads are issued before the table is built, else between the table and its barrier.  Early is right from the third trip of a
 // CTA on, behind it up to the second (launch_dequantize() counts them; B = 16, us, early / behind: bf16 out 2.1 M elements 2.65 / 2.39, 8.4 M

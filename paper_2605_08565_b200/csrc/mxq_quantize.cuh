@@ -63,8 +63,7 @@ struct QuantTables {
     float4 E[256];
 };
 // What the lean loops read of an entry for blocks of 2 and 4, 64 bits: LEAN 1 RN(1 / D) and f16(-D), LEAN 2 the checked
-// reciprocal and D.  16-byte entries at per-lane codes cost four
-// shared-memory wavefronts and as many conflicts for every block and candidate, which is what the kernels for small blocks waited for
+// reciprocal and D.  16-byte entries at per-lane codes cost four shared-memory wavefronts and as many conflicts for every block and candidate, which is what the kernels for small blocks waited for
 // (16.8 M bf16 elements, 128- -> 64-bit reads, us: abs-max, UE4M3, B = 2 19.0 -> 18.3, 4 13.4 -> 13.2; 4-over-6, UE4M3, B = 2 22.1 -> 20.6, 4 16.1
 // -> 15.2; UE5M3, B = 2 29.2 -> 24.7, 4 18.7 -> 17.6; longer blocks lose 1 to 3 %, and read E).
 struct QuantLeanTables : QuantTables {
@@ -1416,6 +1415,7 @@ static cudaError_t launch_quantize_inst(const QuantArgs& a, cudaStream_t stream)
     return err;
 }
 
+// With or without blocks past the last whole chunk; then who stores x_hat.
 template <int DT, int B, int FMT, bool DUAL, int FAKE>
 static cudaError_t launch_quantize_tail(const QuantArgs& a, cudaStream_t s) {
     using S = QuantShape<DT, B>;
